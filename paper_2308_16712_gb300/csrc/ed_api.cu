@@ -236,6 +236,88 @@ bool factorize(int n, int ne, const int32_t *perms, Factorization &F)
     return nc * L == ne;
 }
 
+// Shift a when p rotates every block of d sites by a (site d q + r -> d q + (r +
+// a) mod d), else -1.
+int block_shift(int n, int d, const int32_t *p)
+{
+    const int a = ((p[0] % d) + d) % d;
+    for (int i = 0; i < n; ++i)
+        if (p[i] != i / d * d + (i % d + a) % d)
+            return -1;
+    return a;
+}
+
+// Rewrites the cosets that rotate within blocks of d = F.d sites (translations
+// along the rows of a torus) as such: representative the pure block rotation,
+// kind 3, shift[c] = a; if they are all d of them, coset c is the shift c and
+// the result is true (rep_search_blocks applies).
+bool block_cosets(int n, int ne, const int32_t *perms, Factorization &F, std::vector<int> &shift)
+{
+    const int nc = (int)F.rep.size(), L = F.L, d = F.d;
+    shift.assign(nc, -1);
+    if (d < 2)
+        return false;
+    int n_block = 0;
+    for (int c = 0; c < nc; ++c) {
+        for (int b0 = 0; b0 < L; ++b0) {
+            const int m = F.elem[(size_t)c * L + b0];
+            const int a = block_shift(n, d, perms + (size_t)m * n);
+            if (a < 0)
+                continue;
+            // rho^b m for b = 0 .. L-1 is the coset's list started at b0
+            std::rotate(F.elem.begin() + (size_t)c * L, F.elem.begin() + (size_t)c * L + b0,
+                        F.elem.begin() + (size_t)(c + 1) * L);
+            F.rep[c] = m;
+            F.kind[c] = a ? 3 : 0;
+            shift[c] = a;
+            ++n_block;
+            break;
+        }
+    }
+    if (nc != d || n_block != d)
+        return false;
+    Factorization S = F;
+    for (int c = 0; c < d; ++c) {
+        S.rep[shift[c]] = F.rep[c];
+        S.kind[shift[c]] = F.kind[c];
+        std::copy(F.elem.begin() + (size_t)c * L, F.elem.begin() + (size_t)(c + 1) * L,
+                  S.elem.begin() + (size_t)shift[c] * L);
+    }
+    F = S;
+    for (int c = 0; c < d; ++c)
+        shift[c] = c;
+    return true;
+}
+
+// Key table of rep_search_blocks for blocks of d bits, keys of `rows` of them.
+std::vector<uint32_t> block_table(int d, int rows, bool flip)
+{
+    const int kb = d * rows;
+    const uint32_t full = (1u << kb) - 1u;
+    uint32_t unit = 0;  // bit 0 of every block
+    for (int r = 0; r < rows; ++r)
+        unit |= 1u << (r * d);
+    std::vector<uint32_t> tab(1u << kb);
+    for (uint32_t v = 0; v <= full; ++v) {
+        uint32_t low = full, who = 0;
+        for (int t = 0; t < (flip ? 2 * d : d); ++t) {
+            const int a = t % d;
+            const uint32_t up = full & ~(unit * ((1u << a) - 1u));  // positions >= a of every block
+            uint32_t w = ((v << a) & up) | ((v >> (d - a)) & (full & ~up));
+            if (t >= d)
+                w ^= full;
+            if (w < low) {
+                low = w;
+                who = 0;
+            }
+            if (w == low)
+                who |= 1u << t;
+        }
+        tab[v] = low | (who << 16);
+    }
+    return tab;
+}
+
 bool g_force_generic = false;
 bool g_force_prefix = false;
 bool g_force_all_rotations = false;  // test hook: factored search over every rotation
@@ -326,6 +408,7 @@ void free_basis(ed_basis *b)
     cudaFree(b->d_fchi);
     cudaFree(b->d_fchif);
     cudaFree(b->d_fchi_one);
+    cudaFree(b->d_blk_tab);
     edk::ws_free(b->d_states, 0);
     edk::ws_free(b->d_norms, 0);
     edk::ws_free(b->d_keys, 0);
@@ -609,7 +692,12 @@ edk::GroupView ed_basis::group_view() const
     g.rot_L = rot_L;
     g.rot_d = rot_d;
     g.n_cos = n_cos;
-    g.prune = g.fact && rot_d == 1 && !g_force_all_rotations;
+    g.prune = !g.fact || g_force_all_rotations ? 0 : rot_d == 1 ? 1 : d_blk_tab ? 2 : 0;
+    g.cos_id = cos_id;
+    g.cos_rev = cos_rev;
+    g.blk_tab = d_blk_tab;
+    g.blk_rows = blk_rows;
+    g.blk_bits = blk_bits;
     g.cos_kind = d_cos_kind;
     g.cos_masks32 = d_cos_masks32;
     g.cos_masks64 = d_cos_masks64;
@@ -750,9 +838,43 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         Factorization F;
         if (factorize(n_sites, n_elems, perms, F)) {
             const int nc = (int)F.rep.size();
+            std::vector<int> shift;
+            const bool torus = block_cosets(n_sites, n_elems, perms, F, shift);
+            if (torus && 2 * F.d <= 16) {
+                // keys of as many whole rows as fit in 12 bits and in the
+                // doubled 64-bit word the rows are read from
+                int rows = std::max(1, std::min(12 / F.d, F.L));
+                while (rows > 1 && n_sites + (rows - 1) * F.d > 64)
+                    --rows;
+                std::vector<uint32_t> tab = block_table(F.d, rows, false);
+                const std::vector<uint32_t> inv = block_table(F.d, rows, true);
+                tab.insert(tab.end(), inv.begin(), inv.end());
+                ED_B_TRY(upload(&b->d_blk_tab, tab.data(), tab.size()));
+                b->blk_rows = rows;
+                b->blk_bits = rows * F.d;
+            }
+            b->cos_id = b->cos_rev = -1;
+            for (int c = 0; c < nc; ++c) {
+                if (F.kind[c] == 0)
+                    b->cos_id = c;
+                if (F.kind[c] == 1)
+                    b->cos_rev = c;
+            }
             std::vector<uint32_t> cm32((size_t)nc * edk::kMaskStride, 0);
             std::vector<uint64_t> cm64((size_t)nc * edk::kMaskStride, 0);
             for (int c = 0; c < nc; ++c) {
+                if (shift[c] >= 0) {  // rotation within blocks: see rotate_blocks
+                    uint64_t up = 0, all = n_sites >= 64 ? ~0ULL : (1ULL << n_sites) - 1;
+                    for (int i = 0; i < n_sites; ++i)
+                        if (i % F.d >= shift[c])
+                            up |= 1ULL << i;
+                    const uint64_t m[4] = {up, (uint64_t)shift[c], (uint64_t)(F.d - shift[c]), all & ~up};
+                    for (int k = 0; k < 4; ++k) {
+                        cm64[(size_t)c * edk::kMaskStride + k] = m[k];
+                        cm32[(size_t)c * edk::kMaskStride + k] = (uint32_t)m[k];
+                    }
+                    continue;
+                }
                 const int32_t *pm = perms + (size_t)F.rep[c] * n_sites;
                 if (n_sites <= 32) {
                     auto m = benes_masks(5, n_sites, pm);

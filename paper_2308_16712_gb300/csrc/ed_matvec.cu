@@ -72,7 +72,7 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
                             void *y, int nvec, ed_dtype dtype, MatvecVariant v, cudaStream_t stream)
 {
     if (v.prune >= 0 && g.fact && g.rot_d == 1)
-        g.prune = v.prune;
+        g.prune = v.prune;  // ring translations: pruned or exhaustive (autotuner)
     // the term-parallel kernel: one vector (use_term_parallel), or a real
     // block of 8 vectors: by default in fp32 (ring N=32 / 36 / 40: 1.69 /
     // 43.6 / 724 ms against 2.04 / 48.4 / 788 ms row-per-lane), in fp64 when
@@ -165,9 +165,10 @@ __global__ void __launch_bounds__(256) k_count_nnz(const OpView op, const GroupV
                         const W s = r ^ (W((fl >> 1) & 1) << i) ^ (W(fl & 1) << j);
                         W best;
                         int gb;
-                        if (kFact && g.prune && sizeof(W) == 8)
-                            rep_search_rot1<W, false>(s, sm_kind, sm_masks, g.n_cos, n, g.n_perm, g.flip, full,
-                                                      best, gb);
+                        if (kFact && g.prune == 1)
+                            rep_search_rot1<W, false>(s, sm_kind, sm_masks, g, g.flip, full, best, gb);
+                        else if (kFact && g.prune == 2)
+                            rep_search_blocks<W, false>(s, sm_masks, g, g.flip, full, best, gb);
                         else if (kFact)
                             rep_search_fact<W, false>(s, sm_kind, sm_masks, g.n_cos, g.rot_L, g.rot_d, n, g.n_perm,
                                                       g.flip, full, best, gb);

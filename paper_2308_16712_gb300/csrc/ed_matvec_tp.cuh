@@ -458,9 +458,10 @@ __global__ void __launch_bounds__(kTpThreads, kTpMinBlocks<W, kIdx, NV>)
             // representative search (every lane; idle lanes search s = 0)
             W best;
             int gbest = 0;
-            if (kFact && a.g.prune && (sizeof(W) == 8 || kTrack)) {
-                rep_search_rot1<W, kTrack>(s, sm_kind, sm_masks, a.g.n_cos, n, a.g.n_perm, flip, full, best,
-                                           gbest);
+            if (kFact && a.g.prune == 1) {
+                rep_search_rot1<W, kTrack>(s, sm_kind, sm_masks, a.g, flip, full, best, gbest);
+            } else if (kFact && a.g.prune == 2) {
+                rep_search_blocks<W, kTrack>(s, sm_masks, a.g, flip, full, best, gbest);
             } else if (kFact) {
                 if (kTrack)
                     rep_search_fact<W, true>(s, sm_kind, sm_masks, a.g.n_cos, a.g.rot_L, a.g.rot_d, n,
