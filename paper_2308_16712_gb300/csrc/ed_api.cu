@@ -326,6 +326,8 @@ bool g_force_all_rotations = false;  // test hook: factored search over every ro
 // every lookup is DRAM traffic), else the hash index; 1 = always the hash
 // index; 2 = the bucketed index wherever its entry fits in 64 bits.
 int g_index_policy = 0;
+// Sectors of at least this many states get a slot index.
+uint64_t g_slot_min_dim = 32768;
 constexpr uint64_t kBucketAutoDim = 1ULL << 23;
 
 // Bucketed index over the basis (see find_bucketed): 2^bbits >= dim / 1.8
@@ -416,6 +418,7 @@ void free_basis(ed_basis *b)
     edk::ws_free(b->d_hent, 0);
     edk::ws_free(b->d_bkt, 0);
     edk::ws_free(b->d_stash, 0);
+    edk::free_slot_index(b);
     edk::ws_free(b->d_tab, 0);
     cudaFree(b->d_masks32);
     cudaFree(b->d_masks64);
@@ -547,6 +550,18 @@ ed_operator *build_operator_host(int n_sites, int n_terms, const double *coeff,
                 offmask[(size_t)k * 4 + c] |= (uint8_t)(1u << r);
         }
     }
+    op->uniform = op->real;
+    bool first = true;
+    for (int k = 0; k < op->n_mats && op->uniform; ++k)
+        for (int e = 0; e < 16; ++e) {
+            const double re = op->mats[(size_t)k * 32 + 2 * e];
+            if (e / 4 == e % 4 || re == 0.0)
+                continue;
+            if (first)
+                op->scale = re;
+            op->uniform = op->uniform && re == op->scale;
+            first = false;
+        }
     // the most off-diagonal elements one row can produce
     int worst = 0;
     for (int t = 0; t < n_terms; ++t) {
@@ -593,7 +608,7 @@ edk::OpView op_view(const ed_operator *op)
             exch = 0;
     }
     return edk::OpView{(int)op->h_fams.size(), op->n_mats, op->max_offdiag, op->d_fams, op->d_mats,
-                       op->d_matsf, op->d_offmask, exch};
+                       op->d_matsf, op->d_offmask, exch, op->real ? 1 : 0, op->uniform ? 1 : 0, op->scale};
 }
 
 }  // namespace
@@ -601,6 +616,8 @@ edk::OpView op_view(const ed_operator *op)
 namespace edk {
 
 OpView make_op_view(const ed_operator *op) { return op_view(op); }
+
+uint64_t slot_min_dim() { return g_slot_min_dim; }
 
 int index_policy_get() { return g_index_policy; }
 void index_policy_set(int policy) { g_index_policy = policy; }
@@ -721,6 +738,7 @@ edk::IndexView ed_basis::index_view() const
     v.n_stash = n_stash;
     v.bbits = bbits;
     v.brem = brem;
+    v.slots = g_force_prefix ? edk::SlotView{} : slots;
     return v;
 }
 
@@ -819,6 +837,8 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
             free_basis(b);                       \
             edk::ws_free(d_counts, stream);      \
             edk::ws_free(d_flags, stream);       \
+            edk::ws_free(d_ghosts, stream);      \
+            edk::ws_free(d_ghost_n, stream);     \
             edk::ws_free(d_offsets, stream);     \
             edk::ws_free(d_tmp, stream);         \
             cudaFree(d_binom);                   \
@@ -826,7 +846,8 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
             return _e == cudaErrorMemoryAllocation ? ED_ERR_OOM : ED_ERR_CUDA; \
         }                                        \
     } while (0)
-    uint32_t *d_counts = nullptr, *d_flags = nullptr;
+    uint32_t *d_counts = nullptr, *d_flags = nullptr, *d_ghost_n = nullptr;
+    uint64_t *d_ghosts = nullptr;
     uint64_t *d_offsets = nullptr, *d_tmp = nullptr, *d_binom = nullptr;
     int *d_flag = nullptr;
     ED_B_TRY(upload(&b->d_masks32, m32.data(), m32.size()));
@@ -941,11 +962,27 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         }
         (void)cudaGetLastError();
     }
+    if (!count_only && plan.total / b->order >= edk::slot_min_dim() / 2) {
+        // the weightless representatives, for the slot index: they are fixed by
+        // some element, a vanishing share of all at the sizes where it is built
+        const uint64_t cap = std::min<uint64_t>(1ULL << 24, plan.total / b->order / 8 + 65536);
+        if (edk::ws_alloc((void **)&d_ghosts, cap * sizeof(uint64_t), stream) == cudaSuccess &&
+            edk::ws_alloc((void **)&d_ghost_n, sizeof(uint32_t), stream) == cudaSuccess) {
+            plan.ghosts = d_ghosts;
+            plan.ghost_count = d_ghost_n;
+            plan.ghost_cap = (uint32_t)cap;
+            ED_B_TRY(cudaMemsetAsync(d_ghost_n, 0, sizeof(uint32_t), stream));
+        }
+        (void)cudaGetLastError();
+    }
     ED_B_TRY(edk::launch_enum_count(plan, gv, d_counts, stream));
     ED_B_TRY(edk::launch_scan(d_counts, plan.n_chunks, d_offsets, d_tmp, stream));
     uint64_t dim = 0;
+    uint32_t n_ghost = 0;
     ED_B_TRY(cudaMemcpyAsync(&dim, d_offsets + plan.n_chunks, sizeof(uint64_t),
                              cudaMemcpyDeviceToHost, stream));
+    if (plan.ghosts)
+        ED_B_TRY(cudaMemcpyAsync(&n_ghost, d_ghost_n, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
     ED_B_TRY(cudaStreamSynchronize(stream));
     if (count_only) {
         *count_only = dim;
@@ -957,6 +994,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     if (dim >= (1ULL << 32)) {
         free_basis(b);
         edk::ws_free(d_counts, stream); edk::ws_free(d_flags, stream); edk::ws_free(d_offsets, stream);
+        edk::ws_free(d_ghosts, stream); edk::ws_free(d_ghost_n, stream);
         edk::ws_free(d_tmp, stream); cudaFree(d_binom);
         return ED_ERR_UNSUPPORTED;
     }
@@ -964,6 +1002,24 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     ED_B_TRY(edk::ws_alloc((void **)&b->d_states, std::max<uint64_t>(dim, 1) * sizeof(uint64_t), stream));
     ED_B_TRY(edk::ws_alloc((void **)&b->d_norms, std::max<uint64_t>(dim, 1) * sizeof(uint16_t), stream));
     ED_B_TRY(edk::launch_enum_write(plan, gv, d_offsets, b->d_states, b->d_norms, stream));
+
+    if (plan.ghosts && dim >= edk::slot_min_dim() && n_ghost <= plan.ghost_cap) {
+        // the list shrunk to its length, owned by the index
+        uint64_t *list = nullptr;
+        bool ok = !n_ghost || edk::ws_alloc((void **)&list, n_ghost * sizeof(uint64_t), stream) == cudaSuccess;
+        if (ok && n_ghost)
+            ok = cudaMemcpyAsync(list, d_ghosts, n_ghost * sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream) ==
+                 cudaSuccess;
+        ok = ok && edk::build_slot_index(b, list, n_ghost, stream);
+        if (!ok) {
+            (void)cudaGetLastError();
+            edk::ws_free(list, stream);
+        }
+    }
+    edk::ws_free(d_ghosts, stream);
+    edk::ws_free(d_ghost_n, stream);
+    d_ghosts = nullptr;
+    d_ghost_n = nullptr;
 
     // prefix table over the bit-length range of the basis
     uint64_t ends[2] = {0, 0};
@@ -1306,6 +1362,21 @@ void edx_force_prefix_search(int on) { g_force_prefix = on != 0; }
 // Test hook: the index later basis builds make (0 automatic, 1 hash index,
 // 2 bucketed index wherever its entry fits).
 void edx_index_policy(int policy) { g_index_policy = policy; }
+
+// Test hook: later basis builds make a slot index for sectors of at least this
+// many states (0: the library's own threshold).
+void edx_slot_min_dim(uint64_t dim) { g_slot_min_dim = dim ? dim : 32768; }
+
+// Diagnostics hook: whether a basis has a slot index, its slots and the
+// weightless representatives among its keys.
+int edx_basis_slots(const ed_basis *b, uint64_t *n_slots, uint32_t *n_ghost)
+{
+    if (!b)
+        return -1;
+    if (n_slots) *n_slots = b->slots.n_slots;
+    if (n_ghost) *n_ghost = b->slots.n_ghost;
+    return b->slots.pilots ? 1 : 0;
+}
 
 // Diagnostics hook: whether a basis has the bucketed index, its log2 bucket
 // count and the number of stashed keys.

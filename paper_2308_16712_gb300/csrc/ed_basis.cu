@@ -46,7 +46,8 @@ __device__ __forceinline__ uint64_t next_combination(uint64_t s)
 }
 
 // Orbit norm of s if s is the minimum of its orbit, else 0.  Norm = number of
-// group elements fixing s, or 0 when a fixing element has chi != 1.
+// group elements fixing s; -1 for a minimum without weight (a fixing element has
+// chi != 1: norm 0, not in the basis).
 template <typename W>
 __device__ __forceinline__ int rep_norm(W s, const W *sm_masks, const uint32_t *sm_one, int n_perm,
                                         int flip, W full)
@@ -71,7 +72,7 @@ __device__ __forceinline__ int rep_norm(W s, const W *sm_masks, const uint32_t *
             }
         }
     }
-    return ok ? stab : 0;
+    return ok ? stab : -1;
 }
 
 // Same test over the factored group (rotation subgroup x coset representatives).
@@ -93,7 +94,7 @@ __device__ __forceinline__ int rep_norm_fact(W s, const uint8_t *kinds, const W 
                           }
                           return false;
                       });
-    return (rep && ok) ? stab : 0;
+    return rep ? (ok ? stab : -1) : 0;
 }
 
 __host__ __device__ inline size_t enum_smem_bytes(const GroupView &g, size_t wbytes, bool fact)
@@ -151,7 +152,12 @@ __global__ void __launch_bounds__(kEnumThreads) k_enumerate(EnumPlan plan, Group
                 nrm = kFact ? rep_norm_fact<W>((W)s, sm_kind, sm_masks, sm_one, g, full)
                             : rep_norm<W>((W)s, sm_masks, sm_one, g.n_perm, g.flip, full);
             }
-            if (nrm) {
+            if (!kWrite && nrm < 0 && plan.ghosts) {
+                const uint32_t at = atomicAdd(plan.ghost_count, 1u);
+                if (at < plan.ghost_cap)
+                    plan.ghosts[at] = s;
+            }
+            if (nrm > 0) {
                 if (kWrite) {
                     states[out] = s;
                     norms[out] = (uint16_t)nrm;
@@ -160,7 +166,7 @@ __global__ void __launch_bounds__(kEnumThreads) k_enumerate(EnumPlan plan, Group
                 ++kept;
             }
             if (!kWrite && cflags) {
-                word |= (nrm ? 1u : 0u) << (q & 31);
+                word |= (nrm > 0 ? 1u : 0u) << (q & 31);
                 if ((q & 31) == 31 || q + 1 == cnt) {
                     cflags[q >> 5] = word;
                     word = 0;
@@ -183,13 +189,8 @@ cudaError_t enum_launch(const EnumPlan &plan, const GroupView &g, uint32_t *coun
 {
     auto kern = k_enumerate<W, kU1, kWrite, kFact>;
     const size_t smem = enum_smem_bytes(g, sizeof(W), kFact);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kEnumThreads, smem);
+    int sms = 0, per_sm = 0;
+    const cudaError_t e = kernel_occupancy((const void *)kern, kEnumThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
         return e;
     const uint64_t want = (plan.n_chunks + kEnumThreads - 1) / kEnumThreads;

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/ed.h"
+#include "ed_slots.cuh"
 
 namespace edk {
 
@@ -138,6 +139,7 @@ struct IndexView {
     uint32_t n_stash;
     int bbits;               // log2 of the bucket count
     int brem;                // remainder bits kept per entry: n_sites - bbits
+    SlotView slots;          // slot index (ed_slots.cuh), if the basis has one
 };
 
 // ---------------------------------------------------------------------------
@@ -532,6 +534,7 @@ struct ed_basis {
     ulonglong2 *d_stash = nullptr;
     uint32_t n_stash = 0;
     int bbits = 0, brem = 0;
+    edk::SlotView slots{};  // slot index, sectors of at least slot_min_dim() states
 
     edk::GroupView group_view() const;
     edk::IndexView index_view() const;
@@ -544,6 +547,8 @@ struct ed_operator {
     std::vector<double> mats;         // n_mats x 16 x 2: coeff * h, deduplicated
     int max_offdiag = 0;              // max off-diagonal entries one row can produce
     bool real = true;                 // every matrix entry real
+    bool uniform = false;             // every off-diagonal entry is the real number `scale`
+    double scale = 1.0;
     // host copies of the device tables
     std::vector<edk::OpFamily> h_fams;
     std::vector<double2> h_mats;

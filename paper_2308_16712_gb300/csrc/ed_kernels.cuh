@@ -35,6 +35,11 @@ struct EnumPlan {
     // tests only those states again (for their norms) instead of all of them.
     uint32_t *flags = nullptr;
     uint32_t flag_words = 0;
+    // Optional: the count pass lists the representatives of norm 0 here (at
+    // most ghost_cap of them; *ghost_count counts all)
+    uint64_t *ghosts = nullptr;
+    uint32_t *ghost_count = nullptr;
+    uint32_t ghost_cap = 0;
 };
 
 // Reads and clears the basis kernels' device status word (synchronous).
@@ -94,6 +99,9 @@ struct OpView {
     const float2 *matsf;
     const uint8_t *offmask;  // n_mats x 4: bit c' set if h[c'][c] != 0, c' != c
     int exchange_only;       // every off-diagonal entry couples |01> and |10>
+    int real;                // every entry is real
+    int uniform;             // every nonzero off-diagonal entry is the real number `scale`
+    double scale;
 };
 
 // Host tables (generic group search) for counting a sector; validates the group.
@@ -126,9 +134,38 @@ cudaError_t launch_matvec(const OpView &op, const GroupView &g, const IndexView 
 struct MatvecVariant {
     int kernel = 0;
     int prune = -1;
+    void *scratch = nullptr;   // the caller's memory for the slotted copy of x, if any
+    size_t scratch_bytes = 0;
 };
 cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, bool track, const void *x,
                             void *y, int nvec, ed_dtype dtype, MatvecVariant v, cudaStream_t stream);
+// ---- slot index (ed_slots.cu) and the product over it (ed_matvec_slot.cuh) --------
+// Sectors of at least this many states get a slot index (test hook: any size).
+uint64_t slot_min_dim();
+bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, cudaStream_t stream);
+void free_slot_index(ed_basis *b);
+// Layout of a row of the slotted copy: scalars of a row, scalars per access, row stride.
+struct SlotRow {
+    int scalars, el, stride;
+};
+SlotRow slot_row(int nvec, ed_dtype dtype);
+size_t slot_copy_bytes(const SlotView &v, int nvec, ed_dtype dtype);
+// scratch of one product: the copy and, behind it, the tile queue
+constexpr size_t kSlotQueueBytes = 256;
+inline size_t slot_scratch_bytes(const SlotView &v, int nvec, ed_dtype dtype)
+{
+    return slot_copy_bytes(v, nvec, dtype) + kSlotQueueBytes;
+}
+cudaError_t launch_slot_fill(const IndexView &ix, const void *x, void *xs, int nvec, ed_dtype dtype,
+                             unsigned long long *queue, cudaStream_t s);
+// Whether the slot kernel serves products of this operator over this basis.
+bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, ed_dtype dtype);
+
+// Multiprocessors of the current device and resident blocks of a kernel on one
+// of them at this block size and dynamic shared memory (set as its limit);
+// asked of the driver once per device, kernel and size.
+cudaError_t kernel_occupancy(const void *kern, int threads, size_t smem, int *sms, int *per_sm);
+
 // The variant ed_autotune found fastest for this basis, nvec and dtype on the
 // current GPU (the default variant when none was tuned).
 MatvecVariant tuned_variant(const ed_basis *b, int nvec, ed_dtype dtype);

@@ -807,6 +807,26 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
         ED_L_TRY(S.get(&d_eigs, n_eig));
     ED_L_TRY(cudaMemsetAsync(beta, 0, (mmax + 2) * sizeof(double), st));
 
+    // scratch of the slot kernel for the main run's products, kept for the whole
+    // call where half of what is left has room (allocated per product otherwise)
+    void *slot_ws = nullptr;
+    size_t slot_bytes = 0;
+    if (iv.slots.pilots) {
+        const size_t want = slot_scratch_bytes(iv.slots, 1, f32 && n > kGraphMaxDim ? dt32 : dt64);
+        cudaMemGetInfo(&free_b, &total_b);
+        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc(&slot_ws, want, st) == cudaSuccess) {
+            S.ptrs.push_back(slot_ws);
+            slot_bytes = want;
+        }
+        (void)cudaGetLastError();
+    }
+    auto variant = [&](ed_dtype dt) {
+        MatvecVariant v = tuned_variant(b, 1, dt);
+        v.scratch = slot_ws;
+        v.scratch_bytes = slot_bytes;
+        return v;
+    };
+
     int matvecs = 0;
     MatvecTimer timer;
     auto timed_matvec = [&](const void *in, void *out, ed_dtype dt) -> cudaError_t {
@@ -814,7 +834,7 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
         cudaError_t e = timer.mark(st);
         if (e == cudaSuccess)
             e = push ? launch_matvec_push(ov, gv, iv, track, in, out, dt, st)
-                     : launch_matvec_v(ov, gv, iv, track, in, out, 1, dt, tuned_variant(b, 1, dt), st);
+                     : launch_matvec_v(ov, gv, iv, track, in, out, 1, dt, variant(dt), st);
         if (e == cudaSuccess)
             e = timer.mark(st);
         return e;
@@ -883,14 +903,14 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
             }
             cudaError_t e2;
             if (use_f32) {
-                if ((e2 = launch_matvec_v(ov, gv, iv, track, x32, w32, 1, dt32, tuned_variant(b, 1, dt32), s)) !=
+                if ((e2 = launch_matvec_v(ov, gv, iv, track, x32, w32, 1, dt32, variant(dt32), s)) !=
                     cudaSuccess)
                     return e2;
                 k_dot_part<kC, true><<<nparts, kRedThreads, 0, s>>>(v, w32, n, part_a, tickets, alpha, jdev); count_launch();
                 k_update<kC, true><<<nparts, kRedThreads, 0, s>>>(w32, w, v, vp, n, alpha, beta, part_b,
                                                                    tickets + 1, beta + 1, jdev); count_launch();
             } else {
-                if ((e2 = launch_matvec_v(ov, gv, iv, track, v, w, 1, dt64, tuned_variant(b, 1, dt64), s)) !=
+                if ((e2 = launch_matvec_v(ov, gv, iv, track, v, w, 1, dt64, variant(dt64), s)) !=
                     cudaSuccess)
                     return e2;
                 k_dot_part<kC, false><<<nparts, kRedThreads, 0, s>>>(v, w, n, part_a, tickets, alpha, jdev); count_launch();

@@ -1010,7 +1010,19 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     double *C = sm, *G = sm + 2 * P * P, *R1i = sm + 4 * P * P, *G2 = sm + 5 * P * P, *R2i = sm + 7 * P * P;
     int *stop = flags;
     const int yk = f32 ? 0 : 1;
-    const MatvecVariant tuned = tuned_variant(b, P, f32 ? ED_F32 : ED_F64);
+    MatvecVariant tuned = tuned_variant(b, P, f32 ? ED_F32 : ED_F64);
+    if (iv.slots.pilots) {  // scratch of the slot kernel, kept for the whole call where half of what is left has room
+        const size_t want = slot_scratch_bytes(iv.slots, P, f32 ? ED_F32 : ED_F64);
+        size_t free_b = 0, total_b = 0;
+        cudaMemGetInfo(&free_b, &total_b);
+        void *ws = nullptr;
+        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc(&ws, want, st) == cudaSuccess) {
+            S.ptrs.push_back(ws);
+            tuned.scratch = ws;
+            tuned.scratch_bytes = want;
+        }
+        (void)cudaGetLastError();
+    }
     const void *Yh = f32 ? (const void *)W32 : (const void *)W64;
     auto bh = [&](int k) { return Vh + (size_t)(reorth ? k : (k & 1)) * blk; };
     auto bl = [&](int k) { return Vl + (size_t)(reorth ? k : (k & 1)) * blk; };

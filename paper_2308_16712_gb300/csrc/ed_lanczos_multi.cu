@@ -522,12 +522,36 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         track = track || !sectors[k].basis->trivial_chars;
         max_order = std::max(max_order, sectors[k].basis->order);
     }
+    // scratch of the slot kernel (allocated here: products are captured); without
+    // it the other kernels serve every sector
+    void *scratch = nullptr;
+    size_t scratch_bytes = slot_batch_bytes(sectors, ns, 1, C ? ED_C128 : ED_F64);
+    if (scratch_bytes && ws_alloc(&scratch, scratch_bytes, st) == cudaSuccess) {
+        O.ptrs.push_back(scratch);
+    } else {
+        (void)cudaGetLastError();
+        scratch_bytes = 0;
+    }
     auto matvec = [&](const void *xin, void *yout, bool single, cudaStream_t s) -> cudaError_t {
         const size_t esize = single ? sizeof(F) : sizeof(D);
+        std::vector<char> taken(ns, 0);
+        if (scratch_bytes) {
+            std::vector<ed_sector> prod(sectors, sectors + ns);
+            for (int k = 0; k < ns; ++k) {
+                prod[k].d_x = (const char *)xin + off[k] * esize;
+                prod[k].d_y = (char *)yout + off[k] * esize;
+            }
+            LM_CHK(launch_slot_batch(ov, prod.data(), ns, 1, single ? (C ? ED_C64 : ED_F32) : (C ? ED_C128 : ED_F64),
+                                     scratch, scratch_bytes, taken, s));
+        }
+        if (std::find(taken.begin(), taken.end(), 0) == taken.end())
+            return cudaSuccess;
         if (per_sector) {
             const ed_dtype dt = single ? (C ? ED_C64 : ED_F32) : (C ? ED_C128 : ED_F64);
             for (int k = 0; k < ns; ++k) {
                 const ed_basis *b = sectors[k].basis;
+                if (taken[k])
+                    continue;
                 LM_CHK(launch_matvec(ov, b->group_view(), b->index_view(), !b->trivial_chars,
                                      (const char *)xin + off[k] * esize, (char *)yout + off[k] * esize, 1,
                                      dt, s));
@@ -540,13 +564,15 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         a.g.flip = 0;  // spin inversion is per sector
         a.nvec = 1;
         a.max_order = max_order;
-        a.n_sectors = ns;
         uint64_t tiles = 0;
+        int m = 0;
         for (int k = 0; k < ns; ++k) {
+            if (taken[k])
+                continue;
             const ed_basis *b = sectors[k].basis;
             const GroupView gv = b->group_view();
             const IndexView iv = b->index_view();
-            SectorDesc &d = a.sec[k];
+            SectorDesc &d = a.sec[m++];
             d.keys = iv.keys;
             d.states = iv.states;
             d.norms = iv.norms;
@@ -560,6 +586,7 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
             d.flip = b->spin_inversion != 0;
             tiles += (b->dim + 31) / 32;
         }
+        a.n_sectors = m;
         a.total_tiles = tiles;
         const cudaError_t ce = batch_ctl(s, &a.ctl);  // first used in the eager step 0, before any capture
         if (ce != cudaSuccess)

@@ -1,5 +1,5 @@
 // ed_matvec.cu -- kernel choice and dtype dispatch of the matvec.
-#include "ed_matvec_tp.cuh"
+#include "ed_matvec_slot.cuh"
 
 namespace edk {
 
@@ -68,11 +68,119 @@ cudaError_t launch_matvec(const OpView &op, const GroupView &g, const IndexView 
     return launch_matvec_v(op, g, ix, track, x, y, nvec, dtype, MatvecVariant{}, stream);
 }
 
+// ---- the slot kernel -----------------------------------------------------------
+namespace {
+
+// log2 of the rows of a tile: as many as keep a tile's terms within the list,
+// and fewer where the sector would not give every resident warp a tile
+// (152 x 32 warps).  A function of the sector and the operator only: it fixes
+// the order of the sums.
+int slot_log_rows(const OpView &op, uint64_t dim)
+{
+    int lg = 4;
+    while (lg > 0 && (op.max_terms << lg) > kSlTerms)
+        --lg;
+    while (lg > 0 && (dim >> lg) < 152 * 32)
+        --lg;
+    return lg;
+}
+
+int slot_search(const GroupView &g) { return g.fact ? g.prune : 0; }
+
+}  // namespace
+
+bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, ed_dtype dtype)
+{
+    if (!ix.slots.pilots || !op.exchange_only || op.max_terms > kSlTerms)
+        return false;
+    if (g_kernel_policy != 0 && g_kernel_policy != 3)
+        return false;
+    // the coefficient table: in shared memory, its entries counted in 16 bits
+    const int order = track ? g.order : 1;
+    const size_t bytes = dtype == ED_F64 || dtype == ED_C128 ? slot_table_bytes<double>(op, order, false)
+                                                             : slot_table_bytes<float>(op, order, false);
+    return bytes <= (size_t)kSlMaxTable && (size_t)op.n_mats * 2 * g.order < 65536 &&
+           (size_t)op.n_fam * sizeof(OpFamily) <= 16384;
+}
+
+SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix, const void *x, const void *xs,
+                       void *y)
+{
+    SlotSector d;
+    d.v = ix.slots;
+    d.states = ix.states;
+    d.norms = ix.norms;
+    d.chi = g.fact ? g.fchi : g.chi;
+    d.chif = g.fact ? g.fchif : g.chif;
+    d.x = x;
+    d.xs = xs;
+    d.y = y;
+    d.dim = ix.dim;
+    d.tile_begin = 0;
+    d.log_rows = slot_log_rows(op, ix.dim);
+    d.flip = g.flip;
+    return d;
+}
+
+uint64_t slot_tiles(const SlotSector &d) { return (d.dim + (1ull << d.log_rows) - 1) >> d.log_rows; }
+
+static cudaError_t launch_slot(const OpView &op, const GroupView &g, const IndexView &ix, bool track, const void *x,
+                               void *y, void *xs, int nvec, ed_dtype dtype, cudaStream_t stream)
+{
+    unsigned long long *queue = (unsigned long long *)((char *)xs + slot_copy_bytes(ix.slots, nvec, dtype));
+    cudaError_t e = launch_slot_fill(ix, x, xs, nvec, dtype, queue, stream);
+    if (e != cudaSuccess)
+        return e;
+    const SlotRow row = slot_row(nvec, dtype);
+    SlotArgs<1> a;
+    a.op = op;
+    a.g = g;
+    a.n_sectors = 1;
+    a.max_order = g.order;
+    a.order = track ? g.order : 1;
+    a.scalars = row.scalars;
+    a.stride = row.stride;
+    a.log_parts = 0;
+    while ((row.el << a.log_parts) < row.scalars)
+        ++a.log_parts;
+    a.beyond_l2 = slot_copy_bytes(ix.slots, nvec, dtype) > kSlotL2Bytes;
+    a.ctl = BatchCtl{queue, nullptr, nullptr};
+    a.sec[0] = slot_sector(op, g, ix, x, xs, y);
+    a.total_tiles = slot_tiles(a.sec[0]);
+    const int search = slot_search(g);
+    switch (dtype) {
+    case ED_F64: return slot1_f64(a, search, track, row.el, stream);
+    case ED_F32: return slot1_f32(a, search, track, row.el, stream);
+    case ED_C128: return slot1_c128(a, search, track, row.el, stream);
+    case ED_C64: return slot1_c64(a, search, track, row.el, stream);
+    }
+    return cudaErrorInvalidValue;
+}
+
 cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, bool track, const void *x,
                             void *y, int nvec, ed_dtype dtype, MatvecVariant v, cudaStream_t stream)
 {
     if (v.prune >= 0 && g.fact && g.rot_d == 1)
         g.prune = v.prune;  // ring translations: pruned or exhaustive (autotuner)
+    // the slot kernel wherever the sector has a slot index and memory for the
+    // slotted copy can be had (ring N=32 fp32 / N=36 fp64 / 6x6 torus
+    // complex128: see ed_matvec_slot.cuh); else the kernels below
+    if (v.kernel == 0 && slot_applies(op, g, ix, track, dtype)) {
+        const size_t bytes = slot_scratch_bytes(ix.slots, nvec, dtype);
+        void *xs = v.scratch_bytes >= bytes ? v.scratch : nullptr;
+        void *own = nullptr;
+        if (!xs) {
+            if (ws_alloc(&own, bytes, stream) == cudaSuccess)
+                xs = own;
+            else
+                (void)cudaGetLastError();
+        }
+        if (xs) {
+            const cudaError_t e = launch_slot(op, g, ix, track, x, y, xs, nvec, dtype, stream);
+            const cudaError_t e2 = ws_free(own, stream);
+            return e != cudaSuccess ? e : e2;
+        }
+    }
     // the term-parallel kernel: one vector (use_term_parallel), or a real
     // block of 8 vectors: by default in fp32 (ring N=32 / 36 / 40: 1.69 /
     // 43.6 / 724 ms against 2.04 / 48.4 / 788 ms row-per-lane), in fp64 when

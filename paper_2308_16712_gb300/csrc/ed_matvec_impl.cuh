@@ -506,13 +506,8 @@ cudaError_t matvec_launch(const MatvecArgs &a, cudaStream_t stream)
 {
     auto kern = k_matvec<W, T, kC, kTrack, kFact, NV>;
     const size_t smem = matvec_smem_bytes<W, T, kTrack, kFact>(a.g, a.op);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMvThreads, smem);
+    int sms = 0, per_sm = 0;
+    const cudaError_t e = kernel_occupancy((const void *)kern, kMvThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
         return e;
     const uint64_t warps_needed = (a.ix.dim + 31) / 32;

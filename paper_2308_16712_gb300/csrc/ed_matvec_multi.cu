@@ -4,7 +4,7 @@
 #include <mutex>
 #include <vector>
 
-#include "ed_matvec_tp.cuh"
+#include "ed_matvec_slot.cuh"
 
 namespace edk {
 
@@ -24,6 +24,8 @@ struct CtlWords {
 std::mutex g_ctl_mutex;
 CtlWords g_ctl[kCtlDevices];
 bool g_inject_stall = false;
+// One batch's slotted copies: what stays in L2 between the fill and the product.
+constexpr size_t kSlotBatchBytes = 96ull << 20;
 // 0 and 1: one batched launch (measured faster than per-sector launches on
 // all 140 XXZ N=28 sectors, also for single vectors in single precision:
 // 51.7 against 54.4 ms); 2: one launch per sector where the term-parallel
@@ -31,7 +33,7 @@ bool g_inject_stall = false;
 int g_multi_policy = 0;
 }  // namespace
 
-cudaError_t batch_ctl(cudaStream_t s, BatchCtl *out)
+static cudaError_t batch_words(CtlWords **out)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -39,7 +41,6 @@ cudaError_t batch_ctl(cudaStream_t s, BatchCtl *out)
         return e;
     if (dev < 0 || dev >= kCtlDevices)
         return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(g_ctl_mutex);
     CtlWords &c = g_ctl[dev];
     if (!c.queues) {
         void *p = nullptr;
@@ -52,6 +53,29 @@ cudaError_t batch_ctl(cudaStream_t s, BatchCtl *out)
         c.status = reinterpret_cast<unsigned int *>(c.queues + kQueueRing);
         c.gate = reinterpret_cast<int *>(c.status + 1);
     }
+    *out = &c;
+    return cudaSuccess;
+}
+
+// status word and gate of a launch that brings its own tile queue
+cudaError_t batch_gate(BatchCtl *out)
+{
+    std::lock_guard<std::mutex> lock(g_ctl_mutex);
+    CtlWords *c = nullptr;
+    const cudaError_t e = batch_words(&c);
+    if (e == cudaSuccess)
+        *out = BatchCtl{nullptr, c->status, g_inject_stall ? c->gate : nullptr};
+    return e;
+}
+
+cudaError_t batch_ctl(cudaStream_t s, BatchCtl *out)
+{
+    std::lock_guard<std::mutex> lock(g_ctl_mutex);
+    CtlWords *w = nullptr;
+    cudaError_t e = batch_words(&w);
+    if (e != cudaSuccess)
+        return e;
+    CtlWords &c = *w;
     unsigned long long *q = c.queues + (c.next++ % kQueueRing);
     if ((e = cudaMemsetAsync(q, 0, sizeof(*q), s)) != cudaSuccess)
         return e;
@@ -81,6 +105,106 @@ cudaError_t multi_f64(const MultiArgs &a, bool track, cudaStream_t s) { return m
 cudaError_t multi_f32(const MultiArgs &a, bool track, cudaStream_t s) { return multi_dispatch_prec<float, false>(a, track, s); }
 cudaError_t multi_c128(const MultiArgs &a, bool track, cudaStream_t s) { return multi_dispatch_prec<double, true>(a, track, s); }
 cudaError_t multi_c64(const MultiArgs &a, bool track, cudaStream_t s) { return multi_dispatch_prec<float, true>(a, track, s); }
+
+// The sectors of a batch that have a slot index, by the slot kernel: sectors
+// with characters all 1 and the others in separate launches (their kernels
+// differ, and a sector's result must not depend on its company).  The slotted
+// copies of a launch share one scratch area of at most kSlotBatchBytes (more
+// only for a single sector that needs it): filled right before they are read,
+// they are still in L2 where they fit.  `taken` marks the sectors done here;
+// the rest, also when no scratch memory can be had, are left to the caller.
+size_t slot_batch_bytes(const ed_sector *sectors, int n, int nvec, ed_dtype dtype)
+{
+    size_t largest = 0, total = 0;
+    for (int k = 0; k < n; ++k) {
+        const size_t b = slot_copy_bytes(sectors[k].basis->slots, nvec, dtype);
+        largest = std::max(largest, b);
+        total += b;
+    }
+    return total ? std::max(largest, std::min(total, kSlotBatchBytes)) + kSlotQueueBytes : 0;
+}
+
+cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n, int nvec, ed_dtype dtype,
+                              void *scratch, size_t scratch_bytes, std::vector<char> &taken, cudaStream_t s)
+{
+    const SlotRow row = slot_row(nvec, dtype);
+    static thread_local SlotArgs<kMaxSectors> a;  // host staging (22 KB); copied at launch
+    for (int track = 0; track < 2; ++track) {
+        std::vector<int> todo;
+        for (int k = 0; k < n; ++k) {
+            const ed_basis *b = sectors[k].basis;
+            if (b->dim && !taken[k] && (track != 0) == !b->trivial_chars &&
+                slot_applies(op, b->group_view(), b->index_view(), track != 0, dtype))
+                todo.push_back(k);
+        }
+        std::stable_sort(todo.begin(), todo.end(),
+                         [&](int u, int v) { return sectors[u].basis->dim > sectors[v].basis->dim; });
+        for (size_t i = 0; i < todo.size();) {
+            size_t j = i, bytes = 0;
+            for (; j < todo.size(); ++j) {
+                const size_t more = slot_copy_bytes(sectors[todo[j]].basis->slots, nvec, dtype);
+                if (j > i && bytes + more > kSlotBatchBytes)
+                    break;
+                bytes += more;
+            }
+            char *xs = scratch_bytes >= bytes + kSlotQueueBytes ? (char *)scratch : nullptr;
+            void *own = nullptr;
+            if (!xs) {
+                if (ws_alloc(&own, bytes + kSlotQueueBytes, s) != cudaSuccess) {
+                    (void)cudaGetLastError();
+                    return cudaSuccess;  // the remaining sectors take the other kernels
+                }
+                xs = (char *)own;
+            }
+            unsigned long long *queue = (unsigned long long *)(xs + bytes);
+            const ed_basis *b0 = sectors[todo[i]].basis;
+            a.op = op;
+            a.g = b0->group_view();
+            const int search = a.g.fact ? a.g.prune : 0;
+            a.g.flip = 0;  // spin inversion is per sector
+            a.n_sectors = (int)(j - i);
+            a.max_order = 0;
+            a.scalars = row.scalars;
+            a.stride = row.stride;
+            a.log_parts = 0;
+            while ((row.el << a.log_parts) < row.scalars)
+                ++a.log_parts;
+            uint64_t tiles = 0;
+            size_t at = 0;
+            cudaError_t e = cudaSuccess;
+            for (size_t q = i; q < j && e == cudaSuccess; ++q) {
+                const ed_sector &sec = sectors[todo[q]];
+                const IndexView iv = sec.basis->index_view();
+                e = launch_slot_fill(iv, sec.d_x, xs + at, nvec, dtype, q == i ? queue : nullptr, s);
+                SlotSector &d = a.sec[q - i];
+                d = slot_sector(op, sec.basis->group_view(), iv, sec.d_x, xs + at, sec.d_y);
+                d.tile_begin = tiles;
+                tiles += slot_tiles(d);
+                at += slot_copy_bytes(iv.slots, nvec, dtype);
+                a.max_order = std::max(a.max_order, sec.basis->order);
+                taken[todo[q]] = 1;
+            }
+            a.order = track ? a.max_order : 1;
+            a.beyond_l2 = bytes > kSlotL2Bytes;
+            a.total_tiles = tiles;
+            if (e == cudaSuccess)
+                e = batch_gate(&a.ctl);
+            a.ctl.queue = queue;
+            if (e == cudaSuccess)
+                switch (dtype) {
+                case ED_F64: e = slotn_f64(a, search, track != 0, row.el, s); break;
+                case ED_F32: e = slotn_f32(a, search, track != 0, row.el, s); break;
+                case ED_C128: e = slotn_c128(a, search, track != 0, row.el, s); break;
+                case ED_C64: e = slotn_c64(a, search, track != 0, row.el, s); break;
+                }
+            const cudaError_t e2 = ws_free(own, s);
+            if (e != cudaSuccess || e2 != cudaSuccess)
+                return e != cudaSuccess ? e : e2;
+            i = j;
+        }
+    }
+    return cudaSuccess;
+}
 
 // The batched product: the term-parallel kernel where use_term_parallel
 // chooses it (its warps take tiles of one sector each), else the row-per-lane
@@ -146,27 +270,8 @@ extern "C" ed_status ed_matvec_multi(const ed_operator *op, const ed_sector *sec
     const ed_basis *b0 = sectors[0].basis;
     if (!b0)
         return ED_ERR_INVALID_ARG;
-    static MultiArgs args;  // 17 KB: built on the host, passed by value to the kernel
-    static std::mutex args_mutex;
-    std::lock_guard<std::mutex> lock(args_mutex);
-    args.op = make_op_view(op);
-    args.g = b0->group_view();
-    args.nvec = nvec;
-    args.max_order = 0;
-    bool track = false;
-    int m = 0;
-    uint64_t tiles = 0;
-    // the tile list (and the work queue) runs through the sectors largest first
-    std::vector<int> order(n_sectors);
-    for (int s = 0; s < n_sectors; ++s)
-        order[s] = s;
-    std::stable_sort(order.begin(), order.end(), [&](int u, int v) {
-        const uint64_t du = sectors[u].basis ? sectors[u].basis->dim : 0;
-        const uint64_t dv = sectors[v].basis ? sectors[v].basis->dim : 0;
-        return du > dv;
-    });
-    for (int oi = 0; oi < n_sectors; ++oi) {
-        const int s = order[oi];
+    const OpView ov = make_op_view(op);
+    for (int s = 0; s < n_sectors; ++s) {
         const ed_basis *b = sectors[s].basis;
         if (!b || b->n_sites != b0->n_sites || b->n_perm != b0->n_perm || b->perms != b0->perms)
             return ED_ERR_INVALID_ARG;  // every sector must use the same lattice permutations
@@ -178,11 +283,37 @@ extern "C" ed_status ed_matvec_multi(const ed_operator *op, const ed_sector *sec
         if (!b->dim)
             continue;
         const void *x = sectors[s].d_x;
-        void *y = sectors[s].d_y;
+        const void *y = sectors[s].d_y;
         if (!x || !y || x == y || (((uintptr_t)x | (uintptr_t)y) & 15))
             return ED_ERR_INVALID_ARG;
         if (!b->d_htab && !b->d_bkt)
             return ED_ERR_UNSUPPORTED;
+    }
+    std::vector<char> taken(n_sectors, 0);
+    if (g_multi_policy != 2 &&
+        launch_slot_batch(ov, sectors, n_sectors, nvec, dtype, nullptr, 0, taken, (cudaStream_t)stream) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return ED_ERR_CUDA;
+    }
+    static MultiArgs args;  // 17 KB: built on the host, passed by value to the kernel
+    static std::mutex args_mutex;
+    std::lock_guard<std::mutex> lock(args_mutex);
+    args.op = ov;
+    args.g = b0->group_view();
+    args.nvec = nvec;
+    args.max_order = 0;
+    bool track = false;
+    int m = 0;
+    uint64_t tiles = 0;
+    // the tile list (and the work queue) runs through the sectors largest first
+    std::vector<int> order;
+    for (int s = 0; s < n_sectors; ++s)
+        if (!taken[s] && sectors[s].basis->dim)
+            order.push_back(s);
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int u, int v) { return sectors[u].basis->dim > sectors[v].basis->dim; });
+    for (int s : order) {
+        const ed_basis *b = sectors[s].basis;
         const GroupView gv = b->group_view();
         const IndexView iv = b->index_view();
         SectorDesc &d = args.sec[m++];
@@ -192,8 +323,8 @@ extern "C" ed_status ed_matvec_multi(const ed_operator *op, const ed_sector *sec
         sector_index_from(d, b);
         d.chi = gv.fact ? gv.fchi : gv.chi;
         d.chif = gv.fact ? gv.fchif : gv.chif;
-        d.x = x;
-        d.y = y;
+        d.x = sectors[s].d_x;
+        d.y = sectors[s].d_y;
         d.dim = b->dim;
         d.tile_begin = tiles;
         d.flip = b->spin_inversion != 0;

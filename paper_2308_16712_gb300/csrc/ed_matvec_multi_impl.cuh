@@ -492,13 +492,8 @@ cudaError_t multi_launch(const MultiArgs &a, cudaStream_t stream)
 {
     auto kern = k_matvec_multi<W, T, kC, kTrack, kFact, NV>;
     const size_t smem = multi_smem_bytes<W, T, kTrack, kFact>(a.g, a.op, a.n_sectors, a.max_order);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMvThreads, smem);
+    int sms = 0, per_sm = 0;
+    const cudaError_t e = kernel_occupancy((const void *)kern, kMvThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
         return e;
     const uint64_t blocks_needed = (a.total_tiles * 32 + kMvThreads - 1) / kMvThreads;
@@ -537,6 +532,12 @@ cudaError_t multi_dispatch_prec(const MultiArgs &a, bool track, cudaStream_t str
 // control words of a batched launch on stream s (a fresh work-queue counter,
 // zeroed on s; the status word; the gate when a stall is injected)
 cudaError_t batch_ctl(cudaStream_t s, BatchCtl *out);
+cudaError_t batch_gate(BatchCtl *out);
+// the sectors of a batch that the slot kernel serves (see ed_matvec_multi.cu),
+// and the scratch memory that lets it run without allocating
+cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n, int nvec, ed_dtype dtype,
+                              void *scratch, size_t scratch_bytes, std::vector<char> &taken, cudaStream_t s);
+size_t slot_batch_bytes(const ed_sector *sectors, int n, int nvec, ed_dtype dtype);
 void set_inject_stall(bool on);
 int multi_policy_get();
 

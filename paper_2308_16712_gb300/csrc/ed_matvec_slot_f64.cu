@@ -1,0 +1,22 @@
+// ed_matvec_slot_f64.cu -- the slot-index matvec for f64 vectors: the choice of
+// search, and the variants that visit every element of the group.
+#include "ed_matvec_slot.cuh"
+
+namespace edk {
+cudaError_t slot1_f64_ring(const SlotArgs<1> &a, bool track, int el, cudaStream_t s);
+cudaError_t slot1_f64_torus(const SlotArgs<1> &a, bool track, int el, cudaStream_t s);
+cudaError_t slotn_f64_ring(const SlotArgs<kMaxSectors> &a, bool track, int el, cudaStream_t s);
+
+cudaError_t slot1_f64(const SlotArgs<1> &a, int search, bool track, int el, cudaStream_t s)
+{
+    return search == 1   ? slot1_f64_ring(a, track, el, s)
+           : search == 2 ? slot1_f64_torus(a, track, el, s)
+                         : slot_dispatch<double, false, 0, 1>(a, track, el, s);
+}
+
+// a batch on a torus takes the general search
+cudaError_t slotn_f64(const SlotArgs<kMaxSectors> &a, int search, bool track, int el, cudaStream_t s)
+{
+    return search == 1 ? slotn_f64_ring(a, track, el, s) : slot_dispatch<double, false, 0, kMaxSectors>(a, track, el, s);
+}
+}  // namespace edk

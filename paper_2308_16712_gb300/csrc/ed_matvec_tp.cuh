@@ -554,13 +554,8 @@ cudaError_t tp_launch(const TpArgs<kSec> &a, cudaStream_t stream)
     using V = TpVal<T, kC, NV>;
     auto kern = k_matvec_tp<W, T, kC, kTrack, kFact, kIdx, kSec, kPush, NV>;
     const size_t smem = tp_smem_bytes<W, T, V, kFact>(a.g, a.op, a.n_sectors, a.max_order);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTpThreads, smem);
+    int sms = 0, per_sm = 0;
+    const cudaError_t e = kernel_occupancy((const void *)kern, kTpThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
         return e;
     const uint64_t blocks_needed = (a.total_tiles + kTpWarps - 1) / kTpWarps;

@@ -2,13 +2,15 @@
 // arrays the library allocates itself: the solvers' work vectors, the basis
 // build's temporaries and the large arrays of a basis.  cudaMalloc / cudaFree
 // of gigabytes take milliseconds and synchronise the device; memory freed back
-// to this pool is kept (up to a release threshold, min(8 GiB, 1/16 of the
-// device memory), applied at synchronisation points) and handed out again by
+// to this pool is kept (up to a release threshold, 1/16 of the device memory,
+// applied at synchronisation points) and handed out again by
 // the next call without either cost.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
+#include <tuple>
 
 #include "ed_kernels.cuh"
 
@@ -38,7 +40,7 @@ cudaError_t device_pool(cudaMemPool_t *out)
             return e;
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
-        uint64_t keep = std::min<uint64_t>(8ull << 30, total_b / 16);
+        uint64_t keep = total_b / 16;
         if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
             cudaMemPoolDestroy(p);
             return e;
@@ -75,6 +77,35 @@ size_t ws_cached_bytes()
         cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
         return 0;
     return reserved > used ? (size_t)(reserved - used) : 0;
+}
+
+cudaError_t kernel_occupancy(const void *kern, int threads, size_t smem, int *sms, int *per_sm)
+{
+    static std::mutex m;
+    static std::map<std::tuple<int, const void *, size_t>, std::pair<int, int>> known;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess)
+        return e;
+    std::lock_guard<std::mutex> lock(m);
+    const auto key = std::make_tuple(dev, kern, smem);
+    auto it = known.find(key);
+    if (it == known.end()) {
+        int n = 0, k = 0, limit = 0;
+        // the limit only ever grows, so that launches of other sizes in flight keep theirs
+        cudaFuncAttributes fa;
+        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess)
+            return e;
+        limit = std::max(fa.maxDynamicSharedSizeBytes, (int)smem);
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, kern, threads, smem)) != cudaSuccess)
+            return e;
+        it = known.emplace(key, std::make_pair(n, k)).first;
+    }
+    *sms = it->second.first;
+    *per_sm = it->second.second;
+    return cudaSuccess;
 }
 
 }  // namespace edk

@@ -93,27 +93,28 @@ __host__ __device__ __forceinline__ W rotl_n(W x, int b, int n, W full)
 // P_2, P_4, P_8 by doubling, then the length bit by bit from 8 down to 1 (a
 // fixed number of steps for all lanes; the linear search P_{k+1} = P_k &
 // rot(P_k) takes as many as the longest run of the 32 lanes, about 9), longer
-// runs one at a time.  rot(x, k): x rotated down by k.
+// runs one at a time.  rot(x, k): x rotated down by k.  Only the bits of `keep`
+// count: those above may be wrong (they are, in a word repeated by shifting).
 template <typename X, typename F>
-__host__ __device__ __forceinline__ X longest_ones(X p1, int &g, F &&rot)
+__host__ __device__ __forceinline__ X longest_ones(X p1, X keep, int &g, F &&rot)
 {
     const X p2 = p1 & rot(p1, 1);
     const X p4 = p2 & rot(p2, 2);
     const X p8 = p4 & rot(p4, 4);
-    X cur = p8 ? p8 : ~X(0);
-    int len = p8 ? 8 : 0;
+    X cur = p8 & keep ? p8 : ~X(0);
+    int len = p8 & keep ? 8 : 0;
     X t = p4 & rot(cur, 4);
-    if (t) {
+    if (t & keep) {
         cur = t;
         len += 4;
     }
     t = p2 & rot(cur, 2);
-    if (t) {
+    if (t & keep) {
         cur = t;
         len += 2;
     }
     t = p1 & rot(cur, 1);
-    if (t) {
+    if (t & keep) {
         cur = t;
         len += 1;
     }
@@ -126,7 +127,7 @@ __host__ __device__ __forceinline__ X longest_ones(X p1, int &g, F &&rot)
 // structure (all bits equal; no two equal neighbours with spin inversion; no
 // zero without it) has one candidate word: bit 0 stands for it.
 template <typename W>
-__host__ __device__ __forceinline__ W longest_runs(W h, int n, int flip, W full, int &len)
+__host__ __device__ __forceinline__ W longest_runs(W h, uint64_t twice, int n, int flip, W full, int &len)
 {
     int g = 0;
     W found;
@@ -134,7 +135,7 @@ __host__ __device__ __forceinline__ W longest_runs(W h, int n, int flip, W full,
         if (n == 32) {
             const uint32_t b = flip ? ~(h ^ funnel_right(h, h, 1)) : ~h;
             auto rot = [](uint32_t x, int k) { return funnel_right(x, x, k); };
-            uint32_t cur = longest_ones(b, g, rot);
+            uint32_t cur = longest_ones(b, ~0u, g, rot);
             if (b == 0 || b == ~0u) {
                 cur = 1;
                 g = 0;
@@ -151,22 +152,21 @@ __host__ __device__ __forceinline__ W longest_runs(W h, int n, int flip, W full,
             return cur;
         }
     }
-    const W b = (flip ? ~(h ^ ((h >> 1) | (h << (n - 1)))) : ~h) & full;
-    if (b == 0 || b == full) {
-        len = 1;
-        return W(1);
-    }
     if (sizeof(W) == 4 || n <= 48) {
-        // b repeated with period n in a 64-bit word: a rotation down by k is a
-        // shift right by k, valid on the low n bits while the shifts of a chain
-        // add up to at most 64 - n (15 here, and at most n - 1 matter)
-        auto shr = [](uint64_t x, int k) { return x >> k; };
-        const uint64_t p = (uint64_t)b | ((uint64_t)b << n);
-        uint64_t cur = longest_ones(p, g, shr);
+        // h repeated with period n in a 64-bit word (`twice`): a rotation down by
+        // k is a shift right by k, valid on the low n bits while the shifts of
+        // a chain add up to at most 64 - n (16 here, and at most n matter)
+        const uint64_t keep = (uint64_t)full;
+        const uint64_t p = flip ? ~(twice ^ (twice >> 1)) : ~twice;
+        if (!(p & keep) || !(~p & keep)) {
+            len = 1;
+            return W(1);
+        }
+        uint64_t cur = longest_ones(p, keep, g, [](uint64_t x, int k) { return x >> k; });
         while (g >= 15) {
-            cur &= (uint64_t)full;
+            cur &= keep;
             cur |= cur << n;
-            const uint64_t t = p & (cur >> 1) & (uint64_t)full;
+            const uint64_t t = p & (cur >> 1) & keep;
             if (!t)
                 break;
             cur = t;
@@ -174,6 +174,11 @@ __host__ __device__ __forceinline__ W longest_runs(W h, int n, int flip, W full,
         }
         found = (W)cur & full;
     } else {
+        const W b = (flip ? ~(h ^ ((h >> 1) | (h << (n - 1)))) : ~h) & full;
+        if (b == 0 || b == full) {
+            len = 1;
+            return W(1);
+        }
         W cur = b;
         g = 1;
         while (true) {
@@ -189,6 +194,56 @@ __host__ __device__ __forceinline__ W longest_runs(W h, int n, int flip, W full,
     return found;
 }
 
+// Thins out candidates before they are formed one by one: of the runs whose
+// lowest bits are c, keeps those whose continuation can be the smallest.  Read
+// downwards from a run the next bit differs from it; of the kNarrow bits after
+// that, one after the other, candidates that continue with the run's own value
+// (a zero of the candidate word; any zero without spin inversion) win over the
+// others.  `down` gets the survivors read downwards, as lowest bit - kNarrow - 1;
+// `up` those read upwards (the mirrored candidates).  Each step is the same few
+// instructions for all lanes and halves the candidates beyond the first; the
+// loop over candidates then takes one pass for most warps instead of the four
+// or five of the lane with the most runs.  rot as in longest_ones; words
+// repeated with period n, valid on the bits of `keep`.
+constexpr int kNarrow = 4;
+template <typename X, typename F>
+__host__ __device__ __forceinline__ void narrow_runs(X h, X c, X keep, int len, int flip, bool mirrored, F &&rot,
+                                                     X &down, X &up)
+{
+    X d = rot(c, kNarrow + 1) & keep;
+    X ref = flip ? rot(h, kNarrow + 1) : X(0);
+#pragma unroll
+    for (int k = 1; k <= kNarrow; ++k) {
+        const X t = d & ~(rot(h, kNarrow - k) ^ ref);
+        d = t ? t : d;
+    }
+    down = d;
+    if (!mirrored)
+        return;
+    d = c & keep;
+    ref = flip ? h : X(0);
+    const X q = rot(h, len);
+#pragma unroll
+    for (int k = 1; k <= kNarrow; ++k) {
+        const X t = d & ~(rot(q, k) ^ ref);
+        d = t ? t : d;
+    }
+    up = d;
+}
+
+template <typename W>
+__host__ __device__ __forceinline__ int highest_set(W v)
+{
+#ifdef __CUDA_ARCH__
+    if constexpr (sizeof(W) == 4)
+        return 31 - __clz((int)v);
+    else
+        return 63 - __clzll((long long)v);
+#else
+    return 63 - __builtin_clzll((unsigned long long)v);
+#endif
+}
+
 // The word h twice in a row; get(s) = h rotated down by s (0 <= s < n).
 template <typename W> struct TwiceWord;
 template <> struct TwiceWord<uint32_t> {
@@ -199,6 +254,7 @@ template <> struct TwiceWord<uint32_t> {
         hi = n == 32 ? h : h >> (32 - n);
     }
     __host__ __device__ __forceinline__ uint32_t get(int s) const { return funnel_right(lo, hi, s) & full; }
+    __host__ __device__ __forceinline__ uint64_t low() const { return (uint64_t)hi << 32 | lo; }
 };
 template <> struct TwiceWord<uint64_t> {
     uint32_t w[4], full_hi;
@@ -216,6 +272,7 @@ template <> struct TwiceWord<uint64_t> {
         const uint32_t a = up ? w[1] : w[0], b = up ? w[2] : w[1], c = up ? w[3] : w[2];
         return ((uint64_t)(funnel_right(b, c, s) & full_hi) << 32) | funnel_right(a, b, s);
     }
+    __host__ __device__ __forceinline__ uint64_t low() const { return (uint64_t)w[1] << 32 | w[0]; }
 };
 
 // keep the smaller of best and q; complemented when its top bit is set and the
@@ -224,6 +281,11 @@ template <typename W, bool kTrack>
 __host__ __device__ __forceinline__ void take_candidate(W q, int gi, int n, int n_perm, int flip, W full, W &best,
                                                         int &gbest)
 {
+    if (!kTrack && sizeof(W) == 4) {
+        best = min(best, q);
+        best = flip ? min(best, (W)(q ^ full)) : best;
+        return;
+    }
     if (flip && ((q >> (n - 1)) & 1)) {
         q ^= full;
         gi += n_perm;
@@ -272,16 +334,50 @@ __host__ __device__ __forceinline__ void rep_search_rot1(W s, const uint8_t *kin
     int gb = 0, len;
     {
         const TwiceWord<W> two(s, n, full);
-        W runs = longest_runs(s, n, flip, full, len);
+        const W runs = longest_runs(s, two.low(), n, flip, full, len);
         const int base = g.cos_id * n, base_rev = g.cos_rev * n;
-        while (runs) {
-            const int p = lowest_set(runs);
-            runs &= runs - 1;
-            int t = p + len;  // rotated down by t, the run's top is bit n - 1
+        const bool mirrored = base_rev >= 0;
+        W down = runs, up = mirrored ? runs : W(0);
+        int below = 0;  // a bit of `down` stands for the run that many bits above
+        const int room = n < 64 - n ? n : 64 - n;  // bits by which a doubled word may be shifted
+        if (sizeof(W) == 4 && n == 32) {
+            uint32_t d, u;
+            narrow_runs((uint32_t)s, (uint32_t)runs, ~0u, len, flip, mirrored,
+                        [](uint32_t x, int k) { return funnel_right(x, x, k); }, d, u);
+            down = (W)d;
+            if (mirrored)
+                up = (W)u;
+            below = kNarrow + 1;
+        } else if (n <= 48 && kNarrow + 1 <= room) {
+            uint64_t d, u;
+            narrow_runs(two.low(), (uint64_t)runs | ((uint64_t)runs << n), (uint64_t)full, len, flip, mirrored,
+                        [](uint64_t x, int k) { return x >> k; }, d, u);
+            down = (W)d;
+            if (mirrored && len + kNarrow <= room)
+                up = (W)u;
+            below = kNarrow + 1;
+        }
+        auto take_down = [&]() {
+            const int p = highest_set(down);
+            down ^= W(1) << p;
+            int t = p + below + len;  // rotated down by t, the run's top is bit n - 1
+            t -= t >= n ? n : 0;
             t -= t >= n ? n : 0;
             take_candidate<W, kTrack>(two.get(t), base + (t ? n - t : 0), n, n_perm, flip, full, bst, gb);
-            if (base_rev >= 0)  // mirrored: rotated down by p and reversed
-                take_candidate<W, kTrack>(reverse_bits(two.get(p), n), base_rev + p, n, n_perm, flip, full, bst, gb);
+        };
+        auto take_up = [&]() {  // mirrored: rotated down by p and reversed
+            const int p = highest_set(up);
+            up ^= W(1) << p;
+            take_candidate<W, kTrack>(reverse_bits(two.get(p), n), base_rev + p, n, n_perm, flip, full, bst, gb);
+        };
+        take_down();  // there is always one; the loop is for the few words with more
+        if (mirrored)
+            take_up();
+        while (down | up) {
+            if (down)
+                take_down();
+            if (up)
+                take_up();
         }
     }
     for (int c = 0; c < g.n_cos; ++c) {
@@ -289,7 +385,7 @@ __host__ __device__ __forceinline__ void rep_search_rot1(W s, const uint8_t *kin
             continue;
         const W h = coset_image(s, (int)kinds[c], masks + c * kMaskStride, n);
         const TwiceWord<W> two(h, n, full);
-        W runs = longest_runs(h, n, flip, full, len);
+        W runs = longest_runs(h, two.low(), n, flip, full, len);
         while (runs) {
             const int p = lowest_set(runs);
             runs &= runs - 1;

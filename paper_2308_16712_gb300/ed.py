@@ -89,6 +89,8 @@ _SIGS = {
     "edx_lanczos_graph": (_i32, [_i32]),
     "edx_peak": (_d, [_i32, _P, _u64, ctypes.POINTER(_d), _P]),
     "edx_basis_bucket": (_i32, [_P, ctypes.POINTER(_i32), ctypes.POINTER(ctypes.c_uint32)]),
+    "edx_slot_min_dim": (None, [_u64]),
+    "edx_basis_slots": (_i32, [_P, ctypes.POINTER(_u64), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_count_nnz": (_i32, [_P, _P, ctypes.POINTER(ctypes.c_ulonglong)]),
     "edx_force_prefix_search": (None, [_i32]),
     "edx_kernel_policy": (None, [_i32]),
@@ -314,6 +316,19 @@ def index_policy(policy: str) -> None:
     index for large sectors), "hash" (always the hash index) or "bucket" (the
     bucketed index wherever its 64-bit entry can hold the key)."""
     _lib.edx_index_policy(INDEX_POLICIES[policy])
+
+
+def slot_min_dim(dim: int) -> None:
+    """Test hook: later basis builds make a slot index for sectors of at least
+    ``dim`` states (0: the library's own threshold)."""
+    _lib.edx_slot_min_dim(dim)
+
+
+def basis_slots(basis: Basis):
+    """(present, slots, weightless representatives) of a basis's slot index."""
+    n, g = _u64(0), ctypes.c_uint32(0)
+    r = _lib.edx_basis_slots(basis.handle, ctypes.byref(n), ctypes.byref(g))
+    return bool(r == 1), n.value, g.value
 
 
 def basis_bucket(basis: Basis):
