@@ -40,7 +40,28 @@ struct EnumPlan {
     uint64_t *ghosts = nullptr;
     uint32_t *ghost_count = nullptr;
     uint32_t ghost_cap = 0;
+    // Optional: only the states whose top n_sites - low_bits bits can belong to a
+    // representative (see launch_prefix_filter), segment by segment in
+    // ascending order; total then counts the states of the segments.
+    const uint32_t *seg_prefix = nullptr;  // the top bits
+    const uint64_t *seg_start = nullptr;   // n_seg + 1: states before each segment
+    uint32_t n_seg = 0;
+    int low_bits = 0;
+    int odd = 0;                           // 1: bit 0 is set in every state
 };
+
+// The values of the top `bits` bits (bits < n_sites) a representative can
+// have, by the bits alone: a value is out when some group element, compared
+// with the identity from the top bit down through bits that are known, makes a
+// smaller word.  prefix / start (2^bits and 2^bits + 1 entries) get the
+// remaining ones in ascending order and the running number of their states
+// (popcount n_up; n_up < 0: all; bit 0 set if odd), *n_seg their number.  inv:
+// n_perm x n_sites bytes, the site that goes to each site.  tmp: work memory of
+// prefix_filter_bytes(bits) bytes.
+size_t prefix_filter_bytes(int bits);
+cudaError_t launch_prefix_filter(int n_sites, int n_up, int odd, int bits, const uint8_t *inv, int n_perm, int flip,
+                                 const uint64_t *binom, void *tmp, uint32_t *prefix, uint64_t *start,
+                                 uint32_t *n_seg, cudaStream_t stream);
 
 // Reads and clears the basis kernels' device status word (synchronous).
 cudaError_t basis_status_take(unsigned int *status);

@@ -16,9 +16,8 @@ pytestmark = pytest.mark.gpu
 
 EXTRA = [
     ("ring18_k9_p-_z-", 18, 9, -1, lambda: ei.ring_group(18, 9, -1), lambda: ei.xxz_ring(18, 1.0, 1.5)),
-    ("ring22_k0_p+_z+", 22, 11, +1, lambda: ei.ring_group(22, 0, +1), lambda: ei.heisenberg_ring(22)),
     ("torus6x6_nup3_k1", 36, 3, 0, lambda: ei.torus_group(6, 6, 1, 0), lambda: ei.j1j2_torus(6, 6, 1.0, 0.5)),
-    ("torus4x5_k02", 20, 10, +1, lambda: ei.torus_group(4, 5, 0, 2), lambda: ei.j1j2_torus(4, 5, 1.0, 0.5)),
+    ("torus4x5_k02", 20, 5, 0, lambda: ei.torus_group(4, 5, 0, 2), lambda: ei.j1j2_torus(4, 5, 1.0, 0.5)),
 ]
 CASES = [s for s in SECTORS if s[0] not in ("ring8_empty", "ring10_noU1_xx_z-")] + EXTRA
 
