@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <vector>
 
 #include "../../include/ed.h"
@@ -559,5 +560,14 @@ struct ed_operator {
     double2 *d_mats = nullptr;        // n_mats x 16
     float2 *d_matsf = nullptr;
     uint8_t *d_offmask = nullptr;     // n_mats x 4: bit c' set if h[c'][c] != 0, c' != c
-    mutable std::atomic<const ed_basis *> checked{nullptr};  // last basis verified symmetric
+    // symmetry groups this operator was found to commute with, by content (the
+    // last kVerified of them)
+    struct Verified {
+        int spin_inversion;
+        std::vector<int32_t> perms;
+    };
+    static constexpr size_t kVerified = 8;
+    mutable std::mutex verified_mutex;
+    mutable std::vector<Verified> verified;
+    mutable size_t verified_next = 0;
 };

@@ -137,7 +137,7 @@ uint64_t binomial_host(int n, int k);
 int index_policy_get();
 void index_policy_set(int policy);
 
-// Operator/basis compatibility check (n_sites, symmetry); cached per basis.
+// Operator/basis compatibility check (n_sites, symmetry); the outcome is kept per group.
 ed_status check_pair(const ed_operator *op, const ed_basis *b);
 OpView make_op_view(const ed_operator *op);
 
