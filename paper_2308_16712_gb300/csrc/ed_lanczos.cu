@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "ed_kernels.cuh"
+#include "ed_tridiag.cuh"
 
 namespace edk {
 namespace {
@@ -506,143 +507,42 @@ __global__ void __launch_bounds__(kRedThreads) k_reorth_update(const typename Ve
         norm_part[blockIdx.x] = make_double2(k.s, k.c);
 }
 
-// ---- tridiagonal eigensolver (one thread) ------------------------------------
-// Number of eigenvalues of T (diag a, offdiag b) below x (Sturm sequence).
-__device__ int sturm_count(const double *a, const double *b, int m, double x)
-{
-    int cnt = 0;
-    double d = 1.0;
-    for (int i = 0; i < m; ++i) {
-        const double bb = i ? b[i] * b[i] : 0.0;
-        d = (a[i] - x) - (i ? bb / d : 0.0);
-        if (d == 0.0)
-            d = -1e-300;
-        if (d < 0.0)
-            ++cnt;
-    }
-    return cnt;
-}
-
+// ---- tridiagonal eigensolver -------------------------------------------------
 // Lowest eigenvalue and eigenvector of the leading m_eff x m_eff block, where
 // m_eff stops at the first beta that vanishes (invariant subspace).
-// a[0..m), beta[0..m]: beta[j] couples v_{j-1} and v_j (beta[0] unused).
-// One warp: multisection -- each lane evaluates the Sturm count at one of 32
-// interior points, which shrinks the bracket of the lowest eigenvalue 33-fold
-// per round -- then inverse iteration on lane 0.  Launch with 32 threads.
-__global__ void k_tridiag_lowest(const double *alpha, const double *beta, int m, double *y,
-                                 double *lambda_out, int *m_eff_out, double *work)
+// alpha[0..m), beta[0..m]: beta[j] couples v_{j-1} and v_j (beta[0] unused).
+// One block; work: 3 m doubles.
+__global__ void __launch_bounds__(kTriThreads) k_tridiag_lowest(const double *alpha, const double *beta, int m, double *y,
+                                                                double *lambda_out, int *m_eff_out, double *work)
 {
-    const int lane = threadIdx.x & 31;
-    int me = m;
-    double scale = 0.0, lo = 1e300, hi = -1e300;
-    if (lane == 0) {
-        for (int i = 0; i < m; ++i)
-            scale = fmax(scale, fabs(alpha[i]) + fabs(beta[i + 1]));
-        for (int i = 1; i < m; ++i)
-            if (!(beta[i] > 1e-13 * fmax(scale, 1e-300))) {
-                me = i;
-                break;
-            }
-        for (int i = 0; i < me; ++i) {  // Gershgorin interval
-            const double r = (i ? fabs(beta[i]) : 0.0) + (i + 1 < me ? fabs(beta[i + 1]) : 0.0);
-            lo = fmin(lo, alpha[i] - r);
-            hi = fmax(hi, alpha[i] + r);
-        }
-    }
-    me = __shfl_sync(0xffffffffu, me, 0);
-    scale = __shfl_sync(0xffffffffu, scale, 0);
-    lo = __shfl_sync(0xffffffffu, lo, 0);
-    hi = __shfl_sync(0xffffffffu, hi, 0);
-    for (int it = 0; it < 24; ++it) {
-        const double width = hi - lo;
-        if (!(width > 2e-16 * fmax(fabs(lo), fabs(hi))))
-            break;
-        const double x = lo + width * (double)(lane + 1) / 33.0;
-        const unsigned below = __ballot_sync(0xffffffffu, sturm_count(alpha, beta, me, x) >= 1);
-        // first lane whose point has an eigenvalue below it
-        const int f = below ? __ffs(below) - 1 : 32;
-        const double nlo = f == 0 ? lo : lo + width * (double)f / 33.0;
-        const double nhi = f == 32 ? hi : lo + width * (double)(f + 1) / 33.0;
-        lo = nlo;
-        hi = nhi;
-    }
-    if (lane != 0)
-        return;
-    const double lam = 0.5 * (lo + hi);
-    // inverse iteration: (T - lam I) z = y, LU without pivoting with guarded pivots
-    double *dd = work;  // pivots
-    const double eps = 1e-15 * fmax(scale, 1e-300);
-    for (int i = 0; i < me; ++i)
-        y[i] = 1.0;
-    for (int iter = 0; iter < 4; ++iter) {
-        double piv = alpha[0] - lam;
-        if (fabs(piv) < eps)
-            piv = eps;
-        dd[0] = piv;
-        for (int i = 1; i < me; ++i) {
-            const double l = beta[i] / dd[i - 1];
-            piv = (alpha[i] - lam) - l * beta[i];
-            if (fabs(piv) < eps)
-                piv = eps;
-            dd[i] = piv;
-            y[i] -= l * y[i - 1];
-        }
-        y[me - 1] /= dd[me - 1];
-        for (int i = me - 2; i >= 0; --i)
-            y[i] = (y[i] - beta[i + 1] * y[i + 1]) / dd[i];
-        double nrm = 0.0;
-        for (int i = 0; i < me; ++i)
-            nrm += y[i] * y[i];
-        nrm = sqrt(nrm);
-        for (int i = 0; i < me; ++i)
-            y[i] /= nrm;
-    }
-    for (int i = me; i < m; ++i)
+    __shared__ TriShared sm;
+    double scale;
+    const int me = tri_effective_size(alpha, beta, m, scale);
+    const double lam = tri_solve(alpha, beta, me, 0, sm, work);
+    tri_vector(alpha, beta, me, lam, scale, y, work + m);
+    for (int i = me + (int)threadIdx.x; i < m; i += kTriThreads)
         y[i] = 0.0;
-    *lambda_out = lam;
-    *m_eff_out = me;
+    if (threadIdx.x == 0) {
+        *lambda_out = lam;
+        *m_eff_out = me;
+    }
 }
 
 // Eigenvalue number blockIdx.x (0 = lowest) of the leading m_eff x m_eff block
-// (m_eff as found by k_tridiag_lowest), by the same 32-point multisection with
-// the criterion "at least blockIdx.x + 1 eigenvalues below x"; NaN beyond m_eff.
-// Launch with 32 threads per block, one block per eigenvalue.
-__global__ void k_tridiag_kth(const double *alpha, const double *beta, int m, const int *m_eff, double *out)
+// (m_eff as found by k_tridiag_lowest); NaN beyond m_eff.  One block per
+// eigenvalue; work: m doubles, which every block fills with the same values.
+__global__ void __launch_bounds__(kTriThreads) k_tridiag_kth(const double *alpha, const double *beta, int m,
+                                                             const int *m_eff, double *out, double *work)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ TriShared sm;
     const int e = blockIdx.x;
     const int me = *m_eff;
-    if (e >= me) {
-        if (lane == 0)
-            out[e] = __longlong_as_double(0x7ff8000000000000LL);
-        return;
-    }
-    double lo = 1e300, hi = -1e300;
-    if (lane == 0) {
-        for (int i = 0; i < me; ++i) {  // Gershgorin interval
-            const double r = (i ? fabs(beta[i]) : 0.0) + (i + 1 < me ? fabs(beta[i + 1]) : 0.0);
-            lo = fmin(lo, alpha[i] - r);
-            hi = fmax(hi, alpha[i] + r);
-        }
-    }
-    lo = __shfl_sync(0xffffffffu, lo, 0);
-    hi = __shfl_sync(0xffffffffu, hi, 0);
-    for (int it = 0; it < 24; ++it) {
-        const double width = hi - lo;
-        if (!(width > 2e-16 * fmax(fabs(lo), fabs(hi))))
-            break;
-        const double x = lo + width * (double)(lane + 1) / 33.0;
-        const unsigned below = __ballot_sync(0xffffffffu, sturm_count(alpha, beta, me, x) >= e + 1);
-        const int f = below ? __ffs(below) - 1 : 32;
-        const double nlo = f == 0 ? lo : lo + width * (double)f / 33.0;
-        const double nhi = f == 32 ? hi : lo + width * (double)(f + 1) / 33.0;
-        lo = nlo;
-        hi = nhi;
-    }
-    if (lane == 0)
-        out[e] = 0.5 * (lo + hi);
+    double lam = __longlong_as_double(0x7ff8000000000000LL);
+    if (e < me)
+        lam = tri_solve(alpha, beta, me, e, sm, work);
+    if (threadIdx.x == 0)
+        out[e] = lam;
 }
-
 
 // CUDA event pairs around every matvec launch; summed after the final sync.
 struct MatvecTimer {
@@ -787,7 +687,7 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
     ED_L_TRY(S.get(&alpha, mmax + 1));
     ED_L_TRY(S.get(&beta, mmax + 2));
     ED_L_TRY(S.get(&y, mmax + 1));
-    ED_L_TRY(S.get(&work, 2 * (mmax + 1)));
+    ED_L_TRY(S.get(&work, 3 * (mmax + 1)));
     ED_L_TRY(S.get(&scal, 8));
     ED_L_TRY(S.get(&m_eff, 1));
     ED_L_TRY(S.get(&part_a, nparts));
@@ -967,9 +867,9 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
     // main pass
     ED_L_TRY(run_any((const D *)x0, steps, f32, store ? V : nullptr, nullptr));
     ED_L_TRY(cudaMemsetAsync(y, 0, (mmax + 1) * sizeof(double), st));
-    k_tridiag_lowest<<<1, 32, 0, st>>>(alpha, beta, steps, y, scal + 0, m_eff, work); count_launch();
+    k_tridiag_lowest<<<1, kTriThreads, 0, st>>>(alpha, beta, steps, y, scal + 0, m_eff, work); count_launch();
     if (n_eig > 0) {
-        k_tridiag_kth<<<n_eig, 32, 0, st>>>(alpha, beta, steps, m_eff, d_eigs); count_launch();
+        k_tridiag_kth<<<n_eig, kTriThreads, 0, st>>>(alpha, beta, steps, m_eff, d_eigs, work); count_launch();
     }
     if (values_only) {
         // lowest Ritz value; residual estimate |beta_{m+1} y_m| of the recurrence
@@ -1033,7 +933,7 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
         ED_L_TRY(cudaMemsetAsync(beta, 0, (mmax + 2) * sizeof(double), st));
         ED_L_TRY(run_any(psi, mref, false, Vr, nullptr));
         ED_L_TRY(cudaMemsetAsync(y, 0, (mmax + 1) * sizeof(double), st));
-        k_tridiag_lowest<<<1, 32, 0, st>>>(alpha, beta, mref, y, scal + 1, m_eff, work); count_launch();
+        k_tridiag_lowest<<<1, kTriThreads, 0, st>>>(alpha, beta, mref, y, scal + 1, m_eff, work); count_launch();
         if (store_r) {
             k_combine<kC><<<vgrid, kRedThreads, 0, st>>>(psi, Vr, y, m_eff, n); count_launch();
         } else {

@@ -661,88 +661,105 @@ __global__ void k_dd_to_f64(const float *h, const float *l, double *x, uint64_t 
         x[i] = (double)h[i] + (double)l[i];
 }
 
-// Cholesky of the P x P symmetric matrix G (row-major): G = R^T R, R upper
-// triangular; Ri = R^-1 (upper).  False when a pivot is not positive enough
-// (rank loss: the block Krylov space stops growing).
+// Cholesky of the P x P symmetric matrix G (row-major) by one warp: G = R^T R, R
+// upper triangular; Ri = R^-1 (upper).  False when a pivot is not positive
+// enough (rank loss: the block Krylov space stops growing).  w: P x P doubles of
+// shared memory.  Right-looking: a pivot's square root and reciprocal are one
+// chain, everything else of a column is spread over the lanes.
 template <int P>
-__device__ bool chol_upper(const double *G, double *R, double *Ri)
+__device__ bool chol_upper(const double *G, double *R, double *Ri, double *w)
 {
+    const int lane = threadIdx.x & 31;
     double scale = 0.0;
     for (int a = 0; a < P; ++a)
         scale = fmax(scale, G[a * P + a]);
-    for (int e = 0; e < P * P; ++e) {
-        R[e] = 0.0;
+    for (int e = lane; e < P * P; e += 32) {
+        const int a = e / P, b = e % P;
+        w[e] = a <= b ? 0.5 * (G[e] + G[b * P + a]) : 0.0;
         Ri[e] = 0.0;
     }
+    __syncwarp();
+    double rinv[P];
     for (int a = 0; a < P; ++a) {
-        double d = G[a * P + a];
-        for (int k = 0; k < a; ++k)
-            d -= R[k * P + a] * R[k * P + a];
+        const double d = w[a * P + a];
         if (!(d > 1e-28 * scale) || !(scale > 0.0))
             return false;
         const double r = sqrt(d);
-        R[a * P + a] = r;
-        for (int b = a + 1; b < P; ++b) {
-            double s = 0.5 * (G[a * P + b] + G[b * P + a]);
-            for (int k = 0; k < a; ++k)
-                s -= R[k * P + a] * R[k * P + b];
-            R[a * P + b] = s / r;
+        rinv[a] = 1.0 / r;
+        __syncwarp();
+        for (int b = a + lane; b < P; b += 32)
+            w[a * P + b] = b == a ? r : w[a * P + b] * rinv[a];
+        __syncwarp();
+        for (int e = lane; e < P * P; e += 32) {
+            const int i = e / P, j = e % P;
+            if (i > a && j >= i)
+                w[e] = fma(-w[a * P + i], w[a * P + j], w[e]);
         }
+        __syncwarp();
     }
-    // inverse of the upper triangular R, column by column
-    for (int b = 0; b < P; ++b) {
-        Ri[b * P + b] = 1.0 / R[b * P + b];
-        for (int a = b - 1; a >= 0; --a) {
-            double s = 0.0;
-            for (int k = a + 1; k <= b; ++k)
-                s += R[a * P + k] * Ri[k * P + b];
-            Ri[a * P + b] = -s / R[a * P + a];
+    for (int e = lane; e < P * P; e += 32)
+        R[e] = w[e];
+    // inverse of the upper triangular R, a column per lane
+    if (lane < P) {
+        double col[P];
+#pragma unroll
+        for (int a = P - 1; a >= 0; --a) {
+            double t = a == lane ? 1.0 : 0.0;
+#pragma unroll
+            for (int k = a + 1; k < P; ++k)
+                t = fma(-w[a * P + k], col[k], t);
+            col[a] = a <= lane ? t * rinv[a] : 0.0;
         }
+#pragma unroll
+        for (int a = 0; a < P; ++a)
+            Ri[a * P + lane] = col[a];
     }
+    __syncwarp();
     return true;
 }
 
-// Small P x P steps, one thread.  Layout of `sm` (device scratch, P*P blocks):
+// Small P x P steps, one warp.  Layout of `sm` (device scratch, P*P blocks):
 // [0] C   [1] Cp   [2] G   [3] R1   [4] R1i   [5] G2   [6] R2   [7] R2i
 // which = 0: A_j = sym(C) -> A[j] (j = step index, 0-based);
 // which = 1: R1 = chol(G);  which = 2: R2 = chol(G2), B[j + 1] = R2 R1 (the
 // coupling to the next block; for j < 0 (the start block) nothing is stored).
 // A failed Cholesky stops the recurrence: *stop = 1, *m_eff = j + 1 blocks.
+// Latency-bound (square roots and divisions of one chain): spreading the rest
+// over the warp took a step from 30 to 12 us at P = 8.
 template <int P>
-__global__ void k_bl_small(double *sm, double *A, double *B, int j, int which, int *stop, int *m_eff)
+__global__ void __launch_bounds__(32) k_bl_small(double *sm, double *A, double *B, int j, int which, int *stop,
+                                                 int *m_eff)
 {
-    if (threadIdx.x != 0 || *stop)
+    __shared__ double w[P * P];
+    if (*stop)
         return;
+    const int lane = threadIdx.x;
     double *C = sm, *G = sm + 2 * P * P, *R1 = sm + 3 * P * P, *R1i = sm + 4 * P * P;
     double *G2 = sm + 5 * P * P, *R2 = sm + 6 * P * P, *R2i = sm + 7 * P * P;
     if (which == 0) {
-        for (int a = 0; a < P; ++a)
-            for (int b = 0; b < P; ++b)
-                A[(size_t)j * P * P + a * P + b] = 0.5 * (C[a * P + b] + C[b * P + a]);
+        for (int e = lane; e < P * P; e += 32)
+            A[(size_t)j * P * P + e] = 0.5 * (C[e] + C[e % P * P + e / P]);
         return;
     }
-    if (which == 1) {
-        if (!chol_upper<P>(G, R1, R1i)) {
+    const bool ok = which == 1 ? chol_upper<P>(G, R1, R1i, w) : chol_upper<P>(G2, R2, R2i, w);
+    if (!ok) {
+        if (lane == 0) {
             *stop = 1;
             *m_eff = j + 1;
         }
         return;
     }
-    if (!chol_upper<P>(G2, R2, R2i)) {
-        *stop = 1;
-        *m_eff = j + 1;
-        return;
-    }
-    if (j >= 0) {
+    if (which == 2 && j >= 0) {
         double *Bn = B + (size_t)(j + 1) * P * P;  // B = R2 R1 (upper triangular)
-        for (int a = 0; a < P; ++a)
-            for (int b = 0; b < P; ++b) {
-                double s = 0.0;
-                for (int k = a; k <= b; ++k)
-                    s += R2[a * P + k] * R1[k * P + b];
-                Bn[a * P + b] = b >= a ? s : 0.0;
-            }
-        *m_eff = j + 1;
+        for (int e = lane; e < P * P; e += 32) {
+            const int a = e / P, b = e % P;
+            double s = 0.0;
+            for (int k = a; k <= b; ++k)
+                s += w[a * P + k] * R1[k * P + b];
+            Bn[e] = b >= a ? s : 0.0;
+        }
+        if (lane == 0)
+            *m_eff = j + 1;
     }
 }
 
@@ -762,122 +779,236 @@ __device__ __forceinline__ double band_el(const double *A, const double *B, int 
 }
 
 // Number of eigenvalues of the leading nn x nn block of T below x: negative
-// pivots of the banded LDL^T of T - x I (Sylvester's law of inertia), with the
-// last P rows of L kept in a ring.
+// pivots of the banded LDL^T of T - x I (Sylvester's law of inertia).  ring: the
+// last P rows of L, and D, in shared memory, entry q of lane l at ring[q * 32 +
+// l].  One division per row (its pivot's reciprocal); P (P + 5) / 2
+// multiply-adds.
 template <int P>
-__device__ int band_count(const double *A, const double *B, int nn, double x, double tiny)
+__device__ int band_count(const double *A, const double *B, int nn, double x, double tiny, double *ring)
 {
-    double L[P + 1][P];  // L[k % (P+1)][k - l - 1] = L(k, l), l in [k - P, k)
-    double D[P + 1];
+    const int lane = threadIdx.x & 31;
+    auto L = [&](int row, int q) -> double & { return ring[(row * P + q) * 32 + lane]; };  // L(k, k-1-q), row = k % (P+1)
+    double *rd = ring + (P + 1) * P * 32 + lane;                                           // 1 / D(k) at [row * 32]
     int cnt = 0;
     for (int k = 0; k < nn; ++k) {
         const int ks = k % (P + 1);
         const int k0 = max(0, k - P);
-        for (int j = k0; j < k; ++j) {
+        double d = band_el<P>(A, B, k, k) - x;
+        double u[P];  // u[q] = L(k, k0+q) D(k0+q)
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const int j = k0 + q;
+            if (j >= k)
+                break;
             const int js = j % (P + 1);
             double s = band_el<P>(A, B, k, j);
-            for (int l = max(k0, j - P); l < j; ++l)
-                s -= L[ks][k - l - 1] * D[l % (P + 1)] * L[js][j - l - 1];
-            L[ks][k - j - 1] = s / D[js];
+#pragma unroll
+            for (int t = 0; t < q; ++t)
+                s = fma(-u[t], L(js, j - (k0 + t) - 1), s);  // L(j, k0+t)
+            u[q] = s;
+            const double l = s * rd[js * 32];
+            L(ks, k - j - 1) = l;
+            d = fma(-l, s, d);
         }
-        double d = band_el<P>(A, B, k, k) - x;
-        for (int l = k0; l < k; ++l)
-            d -= L[ks][k - l - 1] * L[ks][k - l - 1] * D[l % (P + 1)];
         if (fabs(d) < tiny)
             d = -tiny;
-        D[ks] = d;
+        rd[ks * 32] = 1.0 / d;
         cnt += d < 0.0;
     }
     return cnt;
 }
 
-// Eigenvalue number blockIdx.x (0 = lowest) of the leading m_eff P x m_eff P
-// block by 32-point multisection; block 0 also finds the eigenvector of the
-// lowest by inverse iteration (banded LDL^T with guarded pivots; scratch holds
-// nn (P + 1) doubles).  Launch with 32 threads per block.
+template <int P> constexpr size_t kBandRing = (size_t)((P + 1) * P + P + 1) * 32 * sizeof(double);
+
+// One round of the multisection for eigenvalues e = blockIdx.x (0 = lowest):
+// gridDim.y warps evaluate the count at 32 gridDim.y points of the bracket,
+// first[e] becomes the first point with more than e eigenvalues below it.  The
+// bracket (of round r) comes from the previous round's bracket and point, and
+// is kept for the next; round 0 starts from the Gershgorin interval.  The fp64
+// pipe of one SM passes a warp's multiply-add in 75 cycles, so a round gains by
+// spreading its points over SMs: 19456 points take as long as 32.
 template <int P>
-__global__ void k_band_eigs(const double *A, const double *B, const int *m_eff, double *eig, double *y,
-                            double *scratch)
+__global__ void __launch_bounds__(32) k_band_round(const double *A, const double *B, const int *m_eff, double *bracket,
+                                                   int *first, int ne, int round, int last)
 {
-    const int lane = threadIdx.x & 31;
+    extern __shared__ __align__(16) double ring[];
+    const int lane = threadIdx.x;
     const int nn = *m_eff * P;
-    const int e = blockIdx.x;
+    const int e = blockIdx.x, points = 32 * gridDim.y;
+    if (e >= nn)
+        return;
+    double lo = 1e300, hi = -1e300, scale = 0.0;
+    if (round == 0) {
+        for (int r = lane; r < nn; r += 32) {
+            double rad = 0.0;
+            for (int c = max(0, r - P); c <= min(nn - 1, r + P); ++c)
+                if (c != r)
+                    rad += fabs(band_el<P>(A, B, r, c));
+            const double d = band_el<P>(A, B, r, r);
+            lo = fmin(lo, d - rad);
+            hi = fmax(hi, d + rad);
+            scale = fmax(scale, fabs(d) + rad);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            scale = fmax(scale, __shfl_xor_sync(0xffffffffu, scale, o));
+        }
+    } else {
+        const double *p = bracket + ((size_t)(round - 1) * ne + e) * 3;
+        const int f = min(first[(size_t)(round - 1) * ne + e], points);
+        const double width = p[1] - p[0];
+        lo = f == 0 ? p[0] : p[0] + width * (double)f / (double)(points + 1);
+        hi = f >= points ? p[1] : p[0] + width * (double)(f + 1) / (double)(points + 1);
+        scale = p[2];
+    }
+    if (blockIdx.y == 0 && lane == 0) {
+        double *q = bracket + ((size_t)round * ne + e) * 3;
+        q[0] = lo;
+        q[1] = hi;
+        q[2] = scale;
+    }
+    int *out = first + (size_t)round * ne + e;
+    if (round == last || !(hi - lo > 2e-16 * fmax(fabs(lo), fabs(hi))))
+        return;  // only the bracket is wanted, or it is narrow enough already
+    const int at = blockIdx.y * 32 + lane;
+    const double x = lo + (hi - lo) * (double)(at + 1) / (double)(points + 1);
+    if (band_count<P>(A, B, nn, x, 1e-300 + 1e-30 * scale, ring) >= e + 1)
+        atomicMin(out, at);
+}
+
+// Eigenvalues from the last round, and the eigenvector of the lowest by inverse
+// iteration: one warp per eigenvalue, warp 0 goes on to the vector.  Factor
+// (LDL^T, guarded pivots): the columns' rank-one updates spread over the lanes in
+// a (P+1) x (P+1) window; the two triangular solves keep a sliding window of
+// partial results, one per lane.  scratch: nn (P + 1) doubles: L(k, k-1-q) at
+// k (P+1) + q, 1 / D(k) at k (P+1) + P.
+template <int P>
+__global__ void __launch_bounds__(32) k_band_finish(const double *A, const double *B, const int *m_eff,
+                                                    const double *bracket, int ne, int rounds, double *eig, double *y,
+                                                    double *scratch)
+{
+    __shared__ double win[(P + 1) * (P + 1)];
+    const int lane = threadIdx.x;
+    const int nn = *m_eff * P, e = blockIdx.x;
     if (e >= nn) {
         if (lane == 0)
             eig[e] = __longlong_as_double(0x7ff8000000000000LL);
         return;
     }
-    double lo = 1e300, hi = -1e300, scale = 0.0;
-    for (int r = 0; r < nn; ++r) {  // Gershgorin interval
-        double rad = 0.0;
-        for (int c = max(0, r - P); c <= min(nn - 1, r + P); ++c)
-            if (c != r)
-                rad += fabs(band_el<P>(A, B, r, c));
-        const double d = band_el<P>(A, B, r, r);
-        lo = fmin(lo, d - rad);
-        hi = fmax(hi, d + rad);
-        scale = fmax(scale, fabs(d) + rad);
-    }
-    const double tiny = 1e-300 + 1e-30 * scale;
-    for (int it = 0; it < 64; ++it) {
-        const double width = hi - lo;
-        if (!(width > 2e-16 * fmax(fabs(lo), fabs(hi))))
-            break;
-        const double x = lo + width * (double)(lane + 1) / 33.0;
-        const unsigned below = __ballot_sync(0xffffffffu, band_count<P>(A, B, nn, x, tiny) >= e + 1);
-        const int f = below ? __ffs(below) - 1 : 32;
-        const double nlo = f == 0 ? lo : lo + width * (double)f / 33.0;
-        const double nhi = f == 32 ? hi : lo + width * (double)(f + 1) / 33.0;
-        lo = nlo;
-        hi = nhi;
-    }
-    if (lane != 0)
-        return;
-    const double lam = 0.5 * (lo + hi);
-    eig[e] = lam;
+    const double *br = bracket + ((size_t)rounds * ne + e) * 3;
+    const double lam = 0.5 * (br[0] + br[1]), scale = br[2];
+    if (lane == 0)
+        eig[e] = lam;
     if (e != 0 || !y)
         return;
-    // inverse iteration: banded LDL^T of T - lam I stored in full (row k:
-    // L(k, k-1-q) at scratch[k (P+1) + q], D(k) at scratch[k (P+1) + P])
+    constexpr int S = P + 1;
+    const unsigned kAll = 0xffffffffu;
     const double eps = 1e-15 * fmax(scale, 1e-300);
     double *F = scratch;
+    // window: rows and columns k .. k+P, index (r % S, c % S), lower triangle
+    for (int q = lane; q < S * S; q += 32) {
+        const int r = q / S, c = q % S;
+        win[q] = r >= c && r < nn ? band_el<P>(A, B, r, c) - (r == c ? lam : 0.0) : 0.0;
+    }
+    __syncwarp();
     for (int k = 0; k < nn; ++k) {
-        const int k0 = max(0, k - P);
-        for (int j = k0; j < k; ++j) {
-            double s = band_el<P>(A, B, k, j);
-            for (int l = max(k0, j - P); l < j; ++l)
-                s -= F[(size_t)k * (P + 1) + (k - l - 1)] * F[(size_t)l * (P + 1) + P] *
-                     F[(size_t)j * (P + 1) + (j - l - 1)];
-            F[(size_t)k * (P + 1) + (k - j - 1)] = s / F[(size_t)j * (P + 1) + P];
-        }
-        double d = band_el<P>(A, B, k, k) - lam;
-        for (int l = k0; l < k; ++l) {
-            const double Lkl = F[(size_t)k * (P + 1) + (k - l - 1)];
-            d -= Lkl * Lkl * F[(size_t)l * (P + 1) + P];
-        }
+        const int kc = k % S;
+        double d = win[kc * S + kc];
         if (fabs(d) < eps)
             d = d < 0.0 ? -eps : eps;
-        F[(size_t)k * (P + 1) + P] = d;
+        const double r = 1.0 / d;
+        double l = 0.0;
+        if (lane >= 1 && lane <= P && k + lane < nn) {
+            l = win[(k + lane) % S * S + kc] * r;
+            F[(size_t)(k + lane) * S + lane - 1] = l;
+        }
+        if (lane == 0)
+            F[(size_t)k * S + P] = r;
+        for (int q = lane; q < P * P; q += 32) {
+            const int i = 1 + q / P, j = 1 + q % P;  // entry (k+i, k+j), j <= i
+            if (j <= i && k + i < nn) {
+                double &t = win[(k + i) % S * S + (k + j) % S];
+                t = fma(-win[(k + i) % S * S + kc] * r, win[(k + j) % S * S + kc], t);
+            }
+        }
+        __syncwarp();
+        const int nr = k + S;  // the row that enters, in place of row k
+        for (int q = lane; q < S; q += 32) {
+            const int c = nr - q;  // columns nr-P .. nr
+            win[kc * S + c % S] = nr < nn ? band_el<P>(A, B, nr, c) - (c == nr ? lam : 0.0) : 0.0;
+        }
+        __syncwarp();
     }
-    for (int k = 0; k < nn; ++k)
+    for (int k = lane; k < nn; k += 32)
         y[k] = 1.0;
+    __syncwarp();
     for (int iter = 0; iter < 4; ++iter) {
-        for (int k = 0; k < nn; ++k)  // L u = y
-            for (int l = max(0, k - P); l < k; ++l)
-                y[k] -= F[(size_t)k * (P + 1) + (k - l - 1)] * y[l];
-        for (int k = 0; k < nn; ++k)  // D
-            y[k] /= F[(size_t)k * (P + 1) + P];
-        for (int k = nn - 1; k >= 0; --k)  // L^T z = u
-            for (int r = k + 1; r <= min(nn - 1, k + P); ++r)
-                y[k] -= F[(size_t)r * (P + 1) + (r - k - 1)] * y[r];
-        double nrm = 0.0;
-        for (int k = 0; k < nn; ++k)
-            nrm += y[k] * y[k];
-        nrm = sqrt(nrm);
-        for (int k = 0; k < nn; ++k)
-            y[k] /= nrm;
+        // L u = y: lane q holds the partial entry k + q
+        double w = lane <= P && lane < nn ? y[lane] : 0.0;
+        for (int k = 0; k < nn; ++k) {
+            const double v = __shfl_sync(kAll, w, 0);
+            const bool in = lane >= 1 && lane <= P && k + lane < nn;
+            const double l = in ? F[(size_t)(k + lane) * S + lane - 1] : 0.0;
+            const double enter = lane == P && k + S < nn ? y[k + S] : 0.0;
+            w = fma(-l, v, w);
+            if (lane == 0)
+                y[k] = v * F[(size_t)k * S + P];  // and D
+            w = __shfl_down_sync(kAll, w, 1);
+            if (lane == P)
+                w = enter;
+        }
+        __syncwarp();
+        // L^T z = u: lane q holds the partial entry k - q
+        w = lane <= P && nn - 1 - lane >= 0 ? y[nn - 1 - lane] : 0.0;
+        double s2 = 0.0;
+        for (int k = nn - 1; k >= 0; --k) {
+            const double v = __shfl_sync(kAll, w, 0);
+            const bool in = lane >= 1 && lane <= P && k - lane >= 0;
+            const double l = in ? F[(size_t)k * S + lane - 1] : 0.0;
+            const double enter = lane == P && k - S >= 0 ? y[k - S] : 0.0;
+            w = fma(-l, v, w);
+            s2 = fma(v, v, s2);
+            if (lane == 0)
+                y[k] = v;
+            w = __shfl_down_sync(kAll, w, 1);
+            if (lane == P)
+                w = enter;
+        }
+        __syncwarp();
+        const double r = 1.0 / sqrt(s2);
+        for (int k = lane; k < nn; k += 32)
+            y[k] *= r;
+        __syncwarp();
     }
 }
+
+// Lowest ne eigenvalues of T (and the lowest one's eigenvector into y, if given):
+// rounds of 32 points per warp, as many warps per eigenvalue as the GPU holds at
+// one per SM sub-partition.
+constexpr int kBandWarps = 608;
+template <int P>
+cudaError_t band_eigs(const double *A, const double *B, const int *m_eff, int ne, double *eig, double *y, double *scratch,
+                      double *bracket, int *first, int max_rounds, cudaStream_t st)
+{
+    const int warps = std::max(1, kBandWarps / ne);
+    int rounds = 1;  // 54 bits of the Gershgorin interval
+    while (rounds < max_rounds - 1 && rounds * std::log2(32.0 * warps + 1.0) < 54.0)
+        ++rounds;
+    cudaError_t e = cudaFuncSetAttribute(k_band_round<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBandRing<P>);
+    if (e == cudaSuccess)  // a point beyond every grid: none found
+        e = cudaMemsetAsync(first, 0x7f, (size_t)max_rounds * ne * sizeof(int), st);
+    if (e != cudaSuccess)
+        return e;
+    for (int r = 0; r <= rounds; ++r) {  // the last one only forms the bracket
+        k_band_round<P><<<dim3(ne, warps), 32, kBandRing<P>, st>>>(A, B, m_eff, bracket, first, ne, r, rounds);
+        count_launch();
+    }
+    k_band_finish<P><<<ne, 32, 0, st>>>(A, B, m_eff, bracket, ne, rounds, eig, y, scratch);
+    count_launch();
+    return cudaGetLastError();
+}
+constexpr int kBandMaxRounds = 14;  // 32 points per round: 5.04 bits each, and the last bracket
 
 struct Pool {
     cudaStream_t st;
@@ -990,6 +1121,10 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     ED_BL_TRY(S.get(&y, (size_t)(steps + 1) * P));
     ED_BL_TRY(S.get(&eig, std::max(n_eig, 1)));
     ED_BL_TRY(S.get(&scr, (size_t)(steps + 1) * P * (P + 1)));
+    double *bracket = nullptr;  // the eigensolver's brackets and points
+    int *bfirst = nullptr;
+    ED_BL_TRY(S.get(&bracket, (size_t)kBandMaxRounds * std::max(n_eig, 1) * 3));
+    ED_BL_TRY(S.get(&bfirst, (size_t)kBandMaxRounds * std::max(n_eig, 1)));
     ED_BL_TRY(S.get(&part, (size_t)grid * 2 * P * P));
     ED_BL_TRY(S.get(&tickets, 4));
     ED_BL_TRY(S.get(&flags, 3));
@@ -1103,8 +1238,7 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
         return ED_ERR_INVALID_ARG;  // the start block has lower rank than nvec
     ED_BL_TRY(cudaMemcpyAsync(flags + 2, flags + 1, sizeof(int), cudaMemcpyDeviceToDevice, st));
     const int ne = std::max(n_eig, 1);
-    k_band_eigs<P><<<ne, 32, 0, st>>>(A, B, flags + 1, eig, y, scr); count_launch();
-    ED_BL_TRY(cudaGetLastError());
+    ED_BL_TRY(band_eigs<P>(A, B, flags + 1, ne, eig, y, scr, bracket, bfirst, kBandMaxRounds, st));
     std::vector<double> eh(ne);
     ED_BL_TRY(cudaMemcpyAsync(eh.data(), eig, ne * sizeof(double), cudaMemcpyDeviceToHost, st));
     *res_out = 0.0;

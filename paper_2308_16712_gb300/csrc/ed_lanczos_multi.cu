@@ -22,6 +22,7 @@
 
 #include "ed_kernels.cuh"
 #include "ed_matvec_multi_impl.cuh"
+#include "ed_tridiag.cuh"
 
 namespace edk {
 namespace {
@@ -269,97 +270,28 @@ __global__ void __launch_bounds__(kThr) k_seg_resid(Seg sg, const typename El<C>
 __global__ void k_step_set(int *step, int v) { *step = v; }
 __global__ void k_step_inc(int *step) { *step += 1; }
 
-// Sturm count: eigenvalues below x of the m x m tridiagonal (a, b)
-__device__ int sturm_cnt(const double *a, const double *b, int m, double x)
+// One block per sector: lowest eigenvalue of the sector's tridiagonal matrix and
+// its eigenvector, cut at the first vanishing beta; work: 3 * stride doubles
+// per sector.
+__global__ void __launch_bounds__(kTriThreads) k_seg_tridiag(const double *alpha, const double *beta, int stride, int m,
+                                                             double *y, double *lam_out, int *m_eff, double *work)
 {
-    int cnt = 0;
-    double d = 1.0;
-    for (int i = 0; i < m; ++i) {
-        d = (a[i] - x) - (i ? b[i] * b[i] / d : 0.0);
-        if (d == 0.0)
-            d = -1e-300;
-        cnt += d < 0.0;
-    }
-    return cnt;
-}
-
-// One warp per sector: lowest eigenvalue of the sector's tridiagonal matrix
-// (32-point multisection of the Gershgorin interval with Sturm counts) and its
-// eigenvector (inverse iteration), cut at the first vanishing beta.
-__global__ void k_seg_tridiag(const double *alpha, const double *beta, int stride, int m, double *y,
-                              double *lam_out, int *m_eff, double *work)
-{
+    __shared__ TriShared sm;
     const int s = blockIdx.x;
-    const int lane = threadIdx.x & 31;
     const double *a = alpha + (size_t)s * stride;
     const double *b = beta + (size_t)s * stride;
     double *ys = y + (size_t)s * stride;
-    double *dd = work + (size_t)s * stride;
-    int me = m;
-    double scl = 0.0, lo = 1e300, hi = -1e300;
-    if (lane == 0) {
-        for (int i = 0; i < m; ++i)
-            scl = fmax(scl, fabs(a[i]) + fabs(b[i + 1]));
-        for (int i = 1; i < m; ++i)
-            if (!(b[i] > 1e-13 * fmax(scl, 1e-300))) {
-                me = i;
-                break;
-            }
-        for (int i = 0; i < me; ++i) {
-            const double r = (i ? fabs(b[i]) : 0.0) + (i + 1 < me ? fabs(b[i + 1]) : 0.0);
-            lo = fmin(lo, a[i] - r);
-            hi = fmax(hi, a[i] + r);
-        }
-    }
-    me = __shfl_sync(0xffffffffu, me, 0);
-    scl = __shfl_sync(0xffffffffu, scl, 0);
-    lo = __shfl_sync(0xffffffffu, lo, 0);
-    hi = __shfl_sync(0xffffffffu, hi, 0);
-    for (int it = 0; it < 24; ++it) {
-        const double wd = hi - lo;
-        if (!(wd > 2e-16 * fmax(fabs(lo), fabs(hi))))
-            break;
-        const double x = lo + wd * (double)(lane + 1) / 33.0;
-        const unsigned below = __ballot_sync(0xffffffffu, sturm_cnt(a, b, me, x) >= 1);
-        const int f = below ? __ffs(below) - 1 : 32;
-        const double nlo = f == 0 ? lo : lo + wd * (double)f / 33.0;
-        const double nhi = f == 32 ? hi : lo + wd * (double)(f + 1) / 33.0;
-        lo = nlo;
-        hi = nhi;
-    }
-    if (lane != 0)
-        return;
-    const double lam = 0.5 * (lo + hi);
-    const double eps = 1e-15 * fmax(scl, 1e-300);
-    for (int i = 0; i < me; ++i)
-        ys[i] = 1.0;
-    for (int iter = 0; iter < 4; ++iter) {
-        double piv = a[0] - lam;
-        if (fabs(piv) < eps)
-            piv = eps;
-        dd[0] = piv;
-        for (int i = 1; i < me; ++i) {
-            const double l = b[i] / dd[i - 1];
-            piv = (a[i] - lam) - l * b[i];
-            if (fabs(piv) < eps)
-                piv = eps;
-            dd[i] = piv;
-            ys[i] -= l * ys[i - 1];
-        }
-        ys[me - 1] /= dd[me - 1];
-        for (int i = me - 2; i >= 0; --i)
-            ys[i] = (ys[i] - b[i + 1] * ys[i + 1]) / dd[i];
-        double nrm = 0.0;
-        for (int i = 0; i < me; ++i)
-            nrm += ys[i] * ys[i];
-        nrm = sqrt(nrm);
-        for (int i = 0; i < me; ++i)
-            ys[i] /= nrm;
-    }
-    for (int i = me; i < m; ++i)
+    double *ws = work + (size_t)s * 3 * stride;
+    double scl;
+    const int me = tri_effective_size(a, b, m, scl);
+    const double lam = tri_solve(a, b, me, 0, sm, ws);
+    tri_vector(a, b, me, lam, scl, ys, ws + stride);
+    for (int i = me + (int)threadIdx.x; i < m; i += kTriThreads)
         ys[i] = 0.0;
-    lam_out[(size_t)s * stride] = lam;
-    m_eff[s] = me;
+    if (threadIdx.x == 0) {
+        lam_out[(size_t)s * stride] = lam;
+        m_eff[s] = me;
+    }
 }
 
 // device buffers, graphs and the capture stream, released on every exit path
@@ -467,8 +399,9 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         LM_TRY(O.get(&x32, total));
         LM_TRY(O.get(&w32, total));
     }
-    for (double **p : {&alpha, &beta, &y, &work, &lam, &nrm, &num, &den, &res})
+    for (double **p : {&alpha, &beta, &y, &lam, &nrm, &num, &den, &res})
         LM_TRY(O.get(p, sc));
+    LM_TRY(O.get(&work, 3 * sc));
     LM_TRY(O.get(&m_eff, ns));
     LM_TRY(O.get(&step, 1));
     LM_TRY(O.get(&part, nblk));
@@ -659,7 +592,7 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
     };
     auto tridiag = [&](int m) -> cudaError_t {
         LM_CHK(cudaMemsetAsync(y, 0, sc * sizeof(double), st));
-        k_seg_tridiag<<<ns, 32, 0, st>>>(alpha, beta, stride, m, y, lam, m_eff, work); count_launch();
+        k_seg_tridiag<<<ns, kTriThreads, 0, st>>>(alpha, beta, stride, m, y, lam, m_eff, work); count_launch();
         return cudaGetLastError();
     };
     // m steps from start, then psi = the lowest Ritz vector of every sector
