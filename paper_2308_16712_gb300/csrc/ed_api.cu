@@ -143,16 +143,32 @@ uint64_t binomial(int n, int k)
     return (uint64_t)r;
 }
 
-template <typename T>
-cudaError_t upload(T **dst, const T *src, size_t count)
-{
-    cudaError_t e = cudaMalloc((void **)dst, std::max<size_t>(count, 1) * sizeof(T));
-    if (e != cudaSuccess)
+// Small host tables collected into one image, so that a handle costs one device
+// allocation and one copy: a dozen cudaMalloc / cudaMemcpy pairs took a third of
+// the build of a small sector.
+struct TableImage {
+    std::vector<unsigned char> bytes;
+    std::vector<std::pair<void **, size_t>> slots;  // pointers to set, offsets
+    template <typename T>
+    void add(T **dst, const T *src, size_t count)
+    {
+        const size_t at = (bytes.size() + 255) / 256 * 256;
+        bytes.resize(at + std::max<size_t>(count, 1) * sizeof(T));
+        if (count)
+            std::memcpy(bytes.data() + at, src, count * sizeof(T));
+        slots.push_back({(void **)dst, at});
+    }
+    cudaError_t upload(void **base, cudaStream_t stream) const
+    {
+        cudaError_t e = edk::ws_alloc(base, bytes.size(), stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(*base, bytes.data(), bytes.size(), cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess)
+            for (const auto &s : slots)
+                *s.first = (unsigned char *)*base + s.second;
         return e;
-    if (count)
-        e = cudaMemcpy(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice);
-    return e;
-}
+    }
+};
 
 // Factored form of the lattice group: the largest cyclic subgroup acting as a
 // rotation of the n-bit word (site i -> i + d mod n, smallest such d) and one
@@ -327,7 +343,8 @@ bool g_force_all_rotations = false;  // test hook: factored search over every ro
 // index; 2 = the bucketed index wherever its entry fits in 64 bits.
 int g_index_policy = 0;
 // Sectors of at least this many states get a slot index.
-uint64_t g_slot_min_dim = 32768;
+constexpr uint64_t kSlotMinDim = 1;
+uint64_t g_slot_min_dim = kSlotMinDim;
 constexpr uint64_t kBucketAutoDim = 1ULL << 23;
 
 // Bucketed index over the basis (see find_bucketed): 2^bbits >= dim / 1.8
@@ -404,13 +421,7 @@ void free_basis(ed_basis *b)
     // every launch that may still read the arrays has finished before they
     // go back to the pool (the large ones) or to the device
     cudaDeviceSynchronize();
-    cudaFree(b->d_cos_kind);
-    cudaFree(b->d_cos_masks32);
-    cudaFree(b->d_cos_masks64);
-    cudaFree(b->d_fchi);
-    cudaFree(b->d_fchif);
-    cudaFree(b->d_fchi_one);
-    cudaFree(b->d_blk_tab);
+    edk::ws_free(b->d_tables, 0);
     edk::ws_free(b->d_states, 0);
     edk::ws_free(b->d_norms, 0);
     edk::ws_free(b->d_keys, 0);
@@ -420,11 +431,6 @@ void free_basis(ed_basis *b)
     edk::ws_free(b->d_stash, 0);
     edk::free_slot_index(b);
     edk::ws_free(b->d_tab, 0);
-    cudaFree(b->d_masks32);
-    cudaFree(b->d_masks64);
-    cudaFree(b->d_chi);
-    cudaFree(b->d_chif);
-    cudaFree(b->d_chi_one);
     delete b;
 }
 
@@ -856,8 +862,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
             edk::ws_free(d_ghost_n, stream);     \
             edk::ws_free(d_offsets, stream);     \
             edk::ws_free(d_tmp, stream);         \
-            cudaFree(d_binom);                   \
-            cudaFree(d_flag);                    \
+            edk::ws_free(d_flag, stream);        \
             return _e == cudaErrorMemoryAllocation ? ED_ERR_OOM : ED_ERR_CUDA; \
         }                                        \
     } while (0)
@@ -865,12 +870,14 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     uint64_t *d_ghosts = nullptr, *d_start = nullptr;
     uint32_t *d_prefix = nullptr;
     uint64_t *d_offsets = nullptr, *d_tmp = nullptr, *d_binom = nullptr;
-    int *d_flag = nullptr;
-    ED_B_TRY(upload(&b->d_masks32, m32.data(), m32.size()));
-    ED_B_TRY(upload(&b->d_masks64, m64.data(), m64.size()));
-    ED_B_TRY(upload(&b->d_chi, chi.data(), chi.size()));
-    ED_B_TRY(upload(&b->d_chif, chif.data(), chif.size()));
-    ED_B_TRY(upload(&b->d_chi_one, one.data(), one.size()));
+    uint8_t *d_inv = nullptr;
+    int *d_flag = nullptr;  // [0] not ascending, largest bucket of [1] the prefix table, [2] the hash index, [3] slots failed
+    TableImage tables;
+    tables.add(&b->d_masks32, m32.data(), m32.size());
+    tables.add(&b->d_masks64, m64.data(), m64.size());
+    tables.add(&b->d_chi, chi.data(), chi.size());
+    tables.add(&b->d_chif, chif.data(), chif.size());
+    tables.add(&b->d_chi_one, one.data(), one.size());
     {
         Factorization F;
         if (factorize(n_sites, n_elems, perms, F)) {
@@ -886,7 +893,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
                 std::vector<uint32_t> tab = block_table(F.d, rows, false);
                 const std::vector<uint32_t> inv = block_table(F.d, rows, true);
                 tab.insert(tab.end(), inv.begin(), inv.end());
-                ED_B_TRY(upload(&b->d_blk_tab, tab.data(), tab.size()));
+                tables.add(&b->d_blk_tab, tab.data(), tab.size());
                 b->blk_rows = rows;
                 b->blk_bits = rows * F.d;
             }
@@ -933,12 +940,12 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
                 if ((one[src / 32] >> (src % 32)) & 1u)
                     fone[g / 32] |= 1u << (g % 32);
             }
-            ED_B_TRY(upload(&b->d_cos_kind, F.kind.data(), F.kind.size()));
-            ED_B_TRY(upload(&b->d_cos_masks32, cm32.data(), cm32.size()));
-            ED_B_TRY(upload(&b->d_cos_masks64, cm64.data(), cm64.size()));
-            ED_B_TRY(upload(&b->d_fchi, fchi.data(), fchi.size()));
-            ED_B_TRY(upload(&b->d_fchif, fchif.data(), fchif.size()));
-            ED_B_TRY(upload(&b->d_fchi_one, fone.data(), fone.size()));
+            tables.add(&b->d_cos_kind, F.kind.data(), F.kind.size());
+            tables.add(&b->d_cos_masks32, cm32.data(), cm32.size());
+            tables.add(&b->d_cos_masks64, cm64.data(), cm64.size());
+            tables.add(&b->d_fchi, fchi.data(), fchi.size());
+            tables.add(&b->d_fchif, fchif.data(), fchif.size());
+            tables.add(&b->d_fchi_one, fone.data(), fone.size());
             b->fact = true;
             b->rot_L = F.L;
             b->rot_d = F.d;
@@ -951,7 +958,13 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     for (int n = 0; n <= 64; ++n)
         for (int k = 0; k <= 64; ++k)
             binom[n * 65 + k] = binomial(n, k);
-    ED_B_TRY(upload(&d_binom, binom.data(), binom.size()));
+    tables.add(&d_binom, binom.data(), binom.size());
+    std::vector<uint8_t> inv((size_t)n_elems * n_sites);  // the site that goes to each site
+    for (int g = 0; g < n_elems; ++g)
+        for (int i = 0; i < n_sites; ++i)
+            inv[(size_t)g * n_sites + perms[(size_t)g * n_sites + i]] = (uint8_t)i;
+    tables.add(&d_inv, inv.data(), inv.size());
+    ED_B_TRY(tables.upload(&b->d_tables, stream));
     edk::EnumPlan plan;
     plan.n_sites = n_sites;
     plan.n_up = n_up;
@@ -965,23 +978,14 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     if (plan.total >= (1ULL << 20) && n_elems > 1) {
         const int bits = std::min(22, n_sites - 14);
         const int odd = n_up > 0 && b->fact && b->rot_d == 1 ? 1 : 0;
-        std::vector<uint8_t> inv((size_t)n_elems * n_sites);
-        for (int g = 0; g < n_elems; ++g)
-            for (int i = 0; i < n_sites; ++i)
-                inv[(size_t)g * n_sites + perms[(size_t)g * n_sites + i]] = (uint8_t)i;
-        uint8_t *d_inv = nullptr;
         void *d_work = nullptr;
         uint32_t n_seg = 0;
         uint64_t total = 0;
-        cudaError_t pe = edk::ws_alloc((void **)&d_inv, inv.size(), stream);
-        if (pe == cudaSuccess)
-            pe = edk::ws_alloc(&d_work, edk::prefix_filter_bytes(bits), stream);
+        cudaError_t pe = edk::ws_alloc(&d_work, edk::prefix_filter_bytes(bits), stream);
         if (pe == cudaSuccess)
             pe = edk::ws_alloc((void **)&d_prefix, ((1ULL << bits) + 1) * sizeof(uint32_t), stream);
         if (pe == cudaSuccess)
             pe = edk::ws_alloc((void **)&d_start, ((1ULL << bits) + 1) * sizeof(uint64_t), stream);
-        if (pe == cudaSuccess)
-            pe = cudaMemcpyAsync(d_inv, inv.data(), inv.size(), cudaMemcpyHostToDevice, stream);
         if (pe == cudaSuccess)
             pe = edk::launch_prefix_filter(n_sites, n_up, odd, bits, d_inv, n_elems, spin_inversion != 0, d_binom,
                                            d_work, d_prefix, d_start, d_prefix + (1ULL << bits), stream);
@@ -991,7 +995,6 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
             pe = cudaMemcpyAsync(&total, d_start + (1ULL << bits), sizeof(total), cudaMemcpyDeviceToHost, stream);
         if (pe == cudaSuccess)
             pe = cudaStreamSynchronize(stream);
-        edk::ws_free(d_inv, stream);
         edk::ws_free(d_work, stream);
         ED_B_TRY(pe);
         plan.total = total;
@@ -1021,7 +1024,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         }
         (void)cudaGetLastError();
     }
-    if (!count_only && states / b->order >= edk::slot_min_dim() / 2) {
+    if (!count_only) {
         // the weightless representatives, for the slot index: they are fixed by
         // some element, a vanishing share of all at the sizes where it is built
         const uint64_t cap = std::min<uint64_t>(1ULL << 24, states / b->order / 8 + 65536);
@@ -1048,7 +1051,6 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         free_basis(b);
         edk::ws_free(d_counts, stream); edk::ws_free(d_offsets, stream); edk::ws_free(d_tmp, stream);
         edk::ws_free(d_prefix, stream); edk::ws_free(d_start, stream);
-        cudaFree(d_binom);
         return ED_OK;
     }
     if (dim >= (1ULL << 32)) {
@@ -1056,7 +1058,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         edk::ws_free(d_counts, stream); edk::ws_free(d_flags, stream); edk::ws_free(d_offsets, stream);
         edk::ws_free(d_ghosts, stream); edk::ws_free(d_ghost_n, stream);
         edk::ws_free(d_prefix, stream); edk::ws_free(d_start, stream);
-        edk::ws_free(d_tmp, stream); cudaFree(d_binom);
+        edk::ws_free(d_tmp, stream);
         return ED_ERR_UNSUPPORTED;
     }
     b->dim = dim;
@@ -1068,6 +1070,8 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     d_prefix = nullptr;
     d_start = nullptr;
 
+    ED_B_TRY(edk::ws_alloc((void **)&d_flag, 4 * sizeof(int), stream));
+    ED_B_TRY(cudaMemsetAsync(d_flag, 0, 4 * sizeof(int), stream));
     if (plan.ghosts && dim >= edk::slot_min_dim() && n_ghost <= plan.ghost_cap) {
         // the list shrunk to its length, owned by the index
         uint64_t *list = nullptr;
@@ -1075,7 +1079,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         if (ok && n_ghost)
             ok = cudaMemcpyAsync(list, d_ghosts, n_ghost * sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream) ==
                  cudaSuccess;
-        ok = ok && edk::build_slot_index(b, list, n_ghost, stream);
+        ok = ok && edk::build_slot_index(b, list, n_ghost, d_flag + 3, stream);
         if (!ok) {
             (void)cudaGetLastError();
             edk::ws_free(list, stream);
@@ -1104,19 +1108,8 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     b->tab_size = (uint64_t)n_exp << mb;
     ED_B_TRY(edk::ws_alloc((void **)&b->d_tab, (b->tab_size + 1) * sizeof(uint32_t), stream));
     ED_B_TRY(edk::launch_prefix_table(b->index_view(), b->d_tab, stream));
-    ED_B_TRY(cudaMalloc(&d_flag, 2 * sizeof(int)));
-    ED_B_TRY(cudaMemsetAsync(d_flag, 0, 2 * sizeof(int), stream));
     ED_B_TRY(edk::launch_check_sorted(b->d_states, dim, d_flag, stream));
     ED_B_TRY(edk::launch_max_bucket(b->d_tab, b->tab_size, reinterpret_cast<uint32_t *>(d_flag + 1), stream));
-    int flag[2] = {0, 0};
-    ED_B_TRY(cudaMemcpyAsync(flag, d_flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, stream));
-    ED_B_TRY(cudaStreamSynchronize(stream));
-    b->max_bucket = (uint32_t)flag[1];
-    {
-        unsigned int dev_status = 0;
-        ED_B_TRY(edk::basis_status_take(&dev_status));
-        flag[0] |= (int)dev_status;
-    }
     bool bucketed = false;
     // index kind: the test policy, else the autotuner's choice for sectors
     // like this one, else the bucketed index from kBucketAutoDim states on
@@ -1167,21 +1160,12 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         if (he == cudaSuccess)
             he = edk::launch_hash_fill(b->d_states, b->d_norms, dim, hb, d_hcount, b->d_hent, b->hwide,
                                        b->norm_bits, stream);
-        uint32_t hmax = 0;
-        uint32_t *d_hmax = reinterpret_cast<uint32_t *>(d_flag);
         if (he == cudaSuccess)
-            he = cudaMemsetAsync(d_hmax, 0, sizeof(uint32_t), stream);
-        if (he == cudaSuccess)
-            he = edk::launch_max_bucket(b->d_htab, T, d_hmax, stream);
-        if (he == cudaSuccess)
-            he = cudaMemcpyAsync(&hmax, d_hmax, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
-        if (he == cudaSuccess)
-            he = cudaStreamSynchronize(stream);
+            he = edk::launch_max_bucket(b->d_htab, T, reinterpret_cast<uint32_t *>(d_flag + 2), stream);
         edk::ws_free(d_hcount, stream);
         edk::ws_free(d_hoff, stream);
         edk::ws_free(d_htmp, stream);
         ED_B_TRY(he);
-        b->hash_max_bucket = hmax;
         // packed keys (state << 16 | norm) for the products' row loads and the
         // prefix-table search: one 8-byte load instead of two streams.  The
         // bucketed index goes without them (rows then read states and norms):
@@ -1190,6 +1174,18 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
             ED_B_TRY(edk::ws_alloc((void **)&b->d_keys, dim * sizeof(uint64_t), stream));
             ED_B_TRY(edk::launch_pack_keys(b->d_states, b->d_norms, dim, b->d_keys, stream));
         }
+    }
+    int flag[4] = {0, 0, 0, 0};
+    ED_B_TRY(cudaMemcpyAsync(flag, d_flag, sizeof(flag), cudaMemcpyDeviceToHost, stream));
+    ED_B_TRY(cudaStreamSynchronize(stream));
+    b->max_bucket = (uint32_t)flag[1];
+    b->hash_max_bucket = (uint32_t)flag[2];
+    if (flag[3])
+        edk::free_slot_index(b);
+    {
+        unsigned int dev_status = 0;
+        ED_B_TRY(edk::basis_status_take(&dev_status));
+        flag[0] |= (int)dev_status;
     }
     {
         int k = 1;  // steps that reduce the largest bucket to one entry, plus the final probe
@@ -1201,8 +1197,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     edk::ws_free(d_flags, stream);
     edk::ws_free(d_offsets, stream);
     edk::ws_free(d_tmp, stream);
-    cudaFree(d_binom);
-    cudaFree(d_flag);
+    edk::ws_free(d_flag, stream);
 #undef ED_B_TRY
     if (flag[0]) {
         free_basis(b);
@@ -1292,13 +1287,14 @@ ed_status ed_operator_create(int n_sites, int n_terms, const double *coeff, cons
     ed_operator *op = build_operator_host(n_sites, n_terms, coeff, sites, local);
     if (!op)
         return ED_ERR_INVALID_ARG;
-    cudaError_t e = upload(&op->d_fams, op->h_fams.data(), op->h_fams.size());
-    if (e == cudaSuccess)
-        e = upload(&op->d_mats, op->h_mats.data(), op->h_mats.size());
-    if (e == cudaSuccess)
-        e = upload(&op->d_matsf, op->h_matsf.data(), op->h_matsf.size());
-    if (e == cudaSuccess)
-        e = upload(&op->d_offmask, op->h_offmask.data(), op->h_offmask.size());
+    TableImage tables;
+    tables.add(&op->d_fams, op->h_fams.data(), op->h_fams.size());
+    tables.add(&op->d_mats, op->h_mats.data(), op->h_mats.size());
+    tables.add(&op->d_matsf, op->h_matsf.data(), op->h_matsf.size());
+    tables.add(&op->d_offmask, op->h_offmask.data(), op->h_offmask.size());
+    cudaError_t e = tables.upload(&op->d_tables, 0);
+    if (e == cudaSuccess)  // any stream may use the operator
+        e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         ed_operator_destroy(op);
@@ -1313,10 +1309,7 @@ void ed_operator_destroy(ed_operator *op)
     if (!op)
         return;
     cudaDeviceSynchronize();
-    cudaFree(op->d_fams);
-    cudaFree(op->d_mats);
-    cudaFree(op->d_matsf);
-    cudaFree(op->d_offmask);
+    edk::ws_free(op->d_tables, 0);
     delete op;
 }
 
@@ -1430,7 +1423,7 @@ void edx_index_policy(int policy) { g_index_policy = policy; }
 
 // Test hook: later basis builds make a slot index for sectors of at least this
 // many states (0: the library's own threshold).
-void edx_slot_min_dim(uint64_t dim) { g_slot_min_dim = dim ? dim : 32768; }
+void edx_slot_min_dim(uint64_t dim) { g_slot_min_dim = dim ? dim : kSlotMinDim; }
 
 // Diagnostics hook: whether a basis has a slot index, its slots and the
 // weightless representatives among its keys.

@@ -500,6 +500,7 @@ struct ed_basis {
     std::vector<double> chars;   // n_perm x 2
     uint64_t dim = 0;
     // device arrays
+    void *d_tables = nullptr;  // one allocation with the group tables below (masks, characters, cosets)
     uint64_t *d_states = nullptr;
     uint16_t *d_norms = nullptr;
     uint64_t *d_keys = nullptr;  // state << 16 | norm, n_sites <= 48
@@ -555,7 +556,8 @@ struct ed_operator {
     std::vector<double2> h_mats;
     std::vector<float2> h_matsf;
     std::vector<uint8_t> h_offmask;
-    // device tables
+    // device tables, in one allocation
+    void *d_tables = nullptr;
     edk::OpFamily *d_fams = nullptr;  // rotation families of the terms
     double2 *d_mats = nullptr;        // n_mats x 16
     float2 *d_matsf = nullptr;

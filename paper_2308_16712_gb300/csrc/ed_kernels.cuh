@@ -149,7 +149,8 @@ cudaError_t launch_count_nnz(const OpView &op, const GroupView &g, const IndexVi
 cudaError_t launch_matvec(const OpView &op, const GroupView &g, const IndexView &ix, bool track,
                           const void *x, void *y, int nvec, ed_dtype dtype, cudaStream_t stream);
 // A product variant: kernel 0 = the library's rule (use_term_parallel),
-// 1 = row-per-lane, 2 = term-parallel (where it applies); prune -1 = the
+// 1 = row-per-lane, 2 = term-parallel (where it applies), 4 = the rule without
+// the slot kernel; prune -1 = the
 // group's own setting, 0 = every rotation, 1 = the pruned search (rotation
 // step one site only).
 struct MatvecVariant {
@@ -163,7 +164,7 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
 // ---- slot index (ed_slots.cu) and the product over it (ed_matvec_slot.cuh) --------
 // Sectors of at least this many states get a slot index (test hook: any size).
 uint64_t slot_min_dim();
-bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, cudaStream_t stream);
+bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, cudaStream_t stream);
 void free_slot_index(ed_basis *b);
 // Layout of a row of the slotted copy: scalars of a row, scalars per access, row stride.
 struct SlotRow {
@@ -177,10 +178,20 @@ inline size_t slot_scratch_bytes(const SlotView &v, int nvec, ed_dtype dtype)
 {
     return slot_copy_bytes(v, nvec, dtype) + kSlotQueueBytes;
 }
-cudaError_t launch_slot_fill(const IndexView &ix, const void *x, void *xs, int nvec, ed_dtype dtype,
-                             unsigned long long *queue, cudaStream_t s);
+// One sector's part of a fill: x (rows of nvec values) into xs.
+struct SlotFill {
+    SlotView v;
+    const uint64_t *states;
+    const uint16_t *norms;
+    uint64_t dim;
+    const void *x;
+    void *xs;
+};
+constexpr int kSlotMaxBatch = 160;
+cudaError_t launch_slot_fill(const SlotFill *sec, int n, int nvec, ed_dtype dtype, unsigned long long *queue,
+                             cudaStream_t s);
 // Whether the slot kernel serves products of this operator over this basis.
-bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, ed_dtype dtype);
+bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, int nvec, ed_dtype dtype);
 
 // Multiprocessors of the current device and resident blocks of a kernel on one
 // of them at this block size and dynamic shared memory (set as its limit);

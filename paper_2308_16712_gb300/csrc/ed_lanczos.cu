@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "ed_kernels.cuh"
+#include "ed_lanczos_step.cuh"
 #include "ed_tridiag.cuh"
 
 namespace edk {
@@ -67,7 +68,7 @@ __device__ KSum block_ksum(KSum k)
     __syncthreads();
     if (wid == 0) {
         k = lane < kRedThreads / 32 ? KSum{sm_s[lane], sm_c[lane]} : KSum{0.0, 0.0};
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = kRedThreads / 64; o > 0; o >>= 1) {  // wider merges would add zeros
             KSum other{__shfl_down_sync(0xffffffffu, k.s, o), __shfl_down_sync(0xffffffffu, k.c, o)};
             k = ksum_merge(k, other);
         }
@@ -149,6 +150,16 @@ __device__ double sum_partials_l2(const double2 *part, int nparts)
     for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
         const double2 p = __ldcg(part + i);
         k = ksum_merge(k, KSum{p.x, p.y});
+    }
+    if (nparts <= 32) {  // one warp holds them all: the same merges without the zeros of the others
+        if (threadIdx.x < 32)
+            for (int o = 16; o > 0; o >>= 1) {
+                if (o >= nparts)
+                    continue;
+                KSum other{__shfl_down_sync(0xffffffffu, k.s, o), __shfl_down_sync(0xffffffffu, k.c, o)};
+                k = ksum_merge(k, other);
+            }
+        return k.s + k.c;
     }
     k = block_ksum(k);
     return k.s + k.c;
@@ -425,6 +436,27 @@ __global__ void k_finish_residual(const double2 *res_part, const double2 *den_pa
         *out = sqrt(fmax(r, 0.0) / d);
 }
 
+// dot, update and normalisation of a step in one block (ed_lanczos_step.cuh);
+// with a step index jp, alpha, beta and the store are offset by *jp, which is
+// then advanced
+template <bool kC>
+__global__ void __launch_bounds__(kFusedThreads) k_step_fused(typename Vec<kC>::D *w, const typename Vec<kC>::D *v,
+                                                              const typename Vec<kC>::D *vp,
+                                                              typename Vec<kC>::D *vn, uint64_t n, double *alpha,
+                                                              double *beta, typename Vec<kC>::D *store, int *jp)
+{
+    using D = typename Vec<kC>::D;
+    using F = typename Vec<kC>::F;
+    const int j = jp ? *jp : 0;
+    lanczos_step<D, F, D>(n, w, w, v, vp, vn, (F *)nullptr, store ? store + (uint64_t)(j + 1) * n : nullptr,
+                          (F *)nullptr, alpha + j, beta + j);
+    if (jp) {
+        __syncthreads();  // every thread has read *jp
+        if (threadIdx.x == 0)
+            *jp = j + 1;
+    }
+}
+
 // ---- full reorthogonalisation against the kept Krylov vectors ----------------
 struct Part4 {  // compensated real and imaginary parts of one block's partial
     double rs, rc, is, ic;
@@ -576,6 +608,7 @@ struct MatvecTimer {
 // Steps replayed from a CUDA graph: -1 = for sectors of at most
 // kGraphMaxDim states (launch-bound; larger sectors spend microseconds per
 // launch against milliseconds per kernel), 0 = never, 1 = always.
+constexpr uint64_t kSlotMixedMinDim = 1ULL << 23;
 int g_lanczos_graph = -1;
 constexpr uint64_t kGraphMaxDim = 1ULL << 22;
 
@@ -659,6 +692,7 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
     if (reorth && !store)
         return ED_ERR_UNSUPPORTED;
 
+    const bool fused = !reorth && n <= kFusedMax;  // the vector part of an fp64 step in one block
     const bool graph = !reorth && !push && (g_lanczos_graph == 1 || (g_lanczos_graph < 0 && n <= kGraphMaxDim));
     Scratch S(st);
     Graphs GR;
@@ -722,6 +756,14 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
     }
     auto variant = [&](ed_dtype dt) {
         MatvecVariant v = tuned_variant(b, 1, dt);
+        // The fp32 recurrence loses orthogonality after some 50 steps (fp64: 80),
+        // and from then on the Ritz vector's sign follows the rounding of every
+        // product: below kSlotMixedMinDim states the products of that mode keep
+        // the order of sums they always had, at 8 % more time (ring N=32).
+        // So do those of reorthogonalised runs, whose time the vectors dominate
+        // and whose end (a vanishing beta) is a matter of rounding, too.
+        if (v.kernel == 0 && (reorth || (dt == dt32 && n < kSlotMixedMinDim)))
+            v.kernel = 4;
         v.scratch = slot_ws;
         v.scratch_bytes = slot_bytes;
         return v;
@@ -758,12 +800,22 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
                 e = timed_matvec(x32, w32, dt32);
                 if (e != cudaSuccess)
                     return e;
+            } else if ((e = H64(v, w)) != cudaSuccess) {
+                return e;
+            }
+            D *vn = Vs ? Vs + (uint64_t)(j + 1) * n : (vp ? vp : ring[1]);
+            if (fused && !use_f32) {
+                k_step_fused<kC><<<1, kFusedThreads, 0, st>>>(w, v, vp, vn, n, alpha + j, beta + j, nullptr, nullptr);
+                count_launch();
+                vp = v;
+                v = vn;
+                continue;
+            }
+            if (use_f32) {
                 k_dot_part<kC, true><<<nparts, kRedThreads, 0, st>>>(v, w32, n, part_a, tickets, alpha + j); count_launch();
                 k_update<kC, true><<<nparts, kRedThreads, 0, st>>>(w32, w, v, vp, n, alpha + j, beta + j, part_b,
                                                                     tickets + 1, beta + j + 1); count_launch();
             } else {
-                if ((e = H64(v, w)) != cudaSuccess)
-                    return e;
                 k_dot_part<kC, false><<<nparts, kRedThreads, 0, st>>>(v, w, n, part_a, tickets, alpha + j); count_launch();
                 k_update<kC, false><<<nparts, kRedThreads, 0, st>>>(w, w, v, vp, n, alpha + j, beta + j, part_b,
                                                                      tickets + 1, beta + j + 1); count_launch();
@@ -776,7 +828,6 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
                 }
                 k_norm_final<<<1, kRedThreads, 0, st>>>(part_b, nparts, beta + j + 1); count_launch();
             }
-            D *vn = Vs ? Vs + (uint64_t)(j + 1) * n : (vp ? vp : ring[1]);
             k_normalize<kC><<<vgrid, kRedThreads, 0, st>>>(w, vn, use_f32 ? x32 : nullptr, n, beta + j + 1); count_launch();
             vp = v;
             v = vn;
@@ -813,6 +864,11 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
                 if ((e2 = launch_matvec_v(ov, gv, iv, track, v, w, 1, dt64, variant(dt64), s)) !=
                     cudaSuccess)
                     return e2;
+                if (fused) {
+                    k_step_fused<kC><<<1, kFusedThreads, 0, s>>>(w, v, vp, vn, n, alpha, beta, Vs, jdev);
+                    count_launch();
+                    return cudaGetLastError();
+                }
                 k_dot_part<kC, false><<<nparts, kRedThreads, 0, s>>>(v, w, n, part_a, tickets, alpha, jdev); count_launch();
                 k_update<kC, false><<<nparts, kRedThreads, 0, s>>>(w, w, v, vp, n, alpha, beta, part_b,
                                                                     tickets + 1, beta + 1, jdev); count_launch();

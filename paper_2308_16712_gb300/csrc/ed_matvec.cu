@@ -71,29 +71,35 @@ cudaError_t launch_matvec(const OpView &op, const GroupView &g, const IndexView 
 // ---- the slot kernel -----------------------------------------------------------
 namespace {
 
-// log2 of the rows of a tile: as many as keep a tile's terms within the list,
-// and fewer where the sector would not give every resident warp a tile
-// (152 x 32 warps).  A function of the sector and the operator only: it fixes
-// the order of the sums.
-int slot_log_rows(const OpView &op, uint64_t dim)
-{
-    int lg = 4;
-    while (lg > 0 && (op.max_terms << lg) > kSlTerms)
-        --lg;
-    while (lg > 0 && (dim >> lg) < 152 * 32)
-        --lg;
-    return lg;
-}
+constexpr uint64_t kSlotBlockMinDim = 1024;
 
 int slot_search(const GroupView &g) { return g.fact ? g.prune : 0; }
 
 }  // namespace
 
-bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, ed_dtype dtype)
+// Lanes of a row: as few as keep the terms of 32 / lanes rows within the list.
+int slot_log_group(const OpView &op)
+{
+    int lg = 1;
+    while (lg < 5 && (op.max_terms << (5 - lg)) > kSlTerms)
+        ++lg;
+    return lg;
+}
+
+// Tiles a warp takes from the queue at a time: one, unless there are so many that
+// the end of the launch is still balanced with several (at 8 chunks per warp ring
+// N=32 fp32 lost 4 %).
+int slot_chunk(uint64_t tiles) { return (int)std::max<uint64_t>(1, std::min<uint64_t>(8, tiles / (152 * 40 * 128))); }
+
+bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, int nvec, ed_dtype dtype)
 {
     if (!ix.slots.pilots || !op.exchange_only || op.max_terms > kSlTerms)
         return false;
     if (g_kernel_policy != 0 && g_kernel_policy != 3)
+        return false;
+    // blocks of vectors over the smallest sectors stay with the row-per-lane
+    // kernel, whose columns are those of its single products bit for bit
+    if (nvec > 1 && ix.dim < kSlotBlockMinDim && g_kernel_policy != 3)
         return false;
     // the coefficient table: in shared memory, its entries counted in 16 bits
     const int order = track ? g.order : 1;
@@ -104,7 +110,7 @@ bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, boo
 }
 
 SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix, const void *x, const void *xs,
-                       void *y)
+                       void *y, bool alone)
 {
     SlotSector d;
     d.v = ix.slots;
@@ -117,7 +123,11 @@ SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix
     d.y = y;
     d.dim = ix.dim;
     d.tile_begin = 0;
-    d.log_rows = slot_log_rows(op, ix.dim);
+    // rows of a tile: all the lanes have room for; fewer where a sector alone
+    // would not give every resident warp (152 x 32) a tile
+    d.log_rows = 5 - slot_log_group(op);
+    while (alone && d.log_rows > 0 && (ix.dim >> d.log_rows) < 152 * 32)
+        --d.log_rows;
     d.flip = g.flip;
     return d;
 }
@@ -128,7 +138,8 @@ static cudaError_t launch_slot(const OpView &op, const GroupView &g, const Index
                                void *y, void *xs, int nvec, ed_dtype dtype, cudaStream_t stream)
 {
     unsigned long long *queue = (unsigned long long *)((char *)xs + slot_copy_bytes(ix.slots, nvec, dtype));
-    cudaError_t e = launch_slot_fill(ix, x, xs, nvec, dtype, queue, stream);
+    const SlotFill fill{ix.slots, ix.states, ix.norms, ix.dim, x, xs};
+    cudaError_t e = launch_slot_fill(&fill, 1, nvec, dtype, queue, stream);
     if (e != cudaSuccess)
         return e;
     const SlotRow row = slot_row(nvec, dtype);
@@ -145,8 +156,10 @@ static cudaError_t launch_slot(const OpView &op, const GroupView &g, const Index
         ++a.log_parts;
     a.beyond_l2 = slot_copy_bytes(ix.slots, nvec, dtype) > kSlotL2Bytes;
     a.ctl = BatchCtl{queue, nullptr, nullptr};
-    a.sec[0] = slot_sector(op, g, ix, x, xs, y);
+    a.log_group = slot_log_group(op);
+    a.sec[0] = slot_sector(op, g, ix, x, xs, y, true);
     a.total_tiles = slot_tiles(a.sec[0]);
+    a.chunk = slot_chunk(a.total_tiles);
     const int search = slot_search(g);
     switch (dtype) {
     case ED_F64: return slot1_f64(a, search, track, row.el, stream);
@@ -165,7 +178,7 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
     // the slot kernel wherever the sector has a slot index and memory for the
     // slotted copy can be had (ring N=32 fp32 / N=36 fp64 / 6x6 torus
     // complex128: see ed_matvec_slot.cuh); else the kernels below
-    if (v.kernel == 0 && slot_applies(op, g, ix, track, dtype)) {
+    if (v.kernel == 0 && slot_applies(op, g, ix, track, nvec, dtype)) {
         const size_t bytes = slot_scratch_bytes(ix.slots, nvec, dtype);
         void *xs = v.scratch_bytes >= bytes ? v.scratch : nullptr;
         void *own = nullptr;
@@ -190,7 +203,7 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
     const bool tp_ok = (ix.htab || ix.bkt) && (nvec == 1 || block8) && op.exchange_only;
     const bool rule = block8 ? (g_kernel_policy == 2 || (g_kernel_policy == 0 && dtype == ED_F32))
                              : use_term_parallel(nvec, op, dtype, g.n_sites);
-    const bool tp = tp_ok && (v.kernel == 2 || (v.kernel == 0 && rule));
+    const bool tp = tp_ok && (v.kernel == 2 || ((v.kernel == 0 || v.kernel == 4) && rule));
     if (tp) {
         const TpArgs<1> t = single_tp_args(op, g, ix, x, y);
         const int k = tp_index_kind(t.sec[0]);

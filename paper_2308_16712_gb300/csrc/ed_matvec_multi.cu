@@ -113,6 +113,8 @@ cudaError_t multi_c64(const MultiArgs &a, bool track, cudaStream_t s) { return m
 // only for a single sector that needs it): filled right before they are read,
 // they are still in L2 where they fit.  `taken` marks the sectors done here;
 // the rest, also when no scratch memory can be had, are left to the caller.
+static_assert(kSlotMaxBatch >= kMaxSectors, "a fill takes a whole batch");
+
 size_t slot_batch_bytes(const ed_sector *sectors, int n, int nvec, ed_dtype dtype)
 {
     size_t largest = 0, total = 0;
@@ -134,7 +136,7 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
         for (int k = 0; k < n; ++k) {
             const ed_basis *b = sectors[k].basis;
             if (b->dim && !taken[k] && (track != 0) == !b->trivial_chars &&
-                slot_applies(op, b->group_view(), b->index_view(), track != 0, dtype))
+                slot_applies(op, b->group_view(), b->index_view(), track != 0, nvec, dtype))
                 todo.push_back(k);
         }
         std::stable_sort(todo.begin(), todo.end(),
@@ -171,22 +173,25 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
                 ++a.log_parts;
             uint64_t tiles = 0;
             size_t at = 0;
-            cudaError_t e = cudaSuccess;
-            for (size_t q = i; q < j && e == cudaSuccess; ++q) {
+            std::vector<SlotFill> fill;
+            for (size_t q = i; q < j; ++q) {
                 const ed_sector &sec = sectors[todo[q]];
                 const IndexView iv = sec.basis->index_view();
-                e = launch_slot_fill(iv, sec.d_x, xs + at, nvec, dtype, q == i ? queue : nullptr, s);
+                fill.push_back(SlotFill{iv.slots, iv.states, iv.norms, iv.dim, sec.d_x, xs + at});
                 SlotSector &d = a.sec[q - i];
-                d = slot_sector(op, sec.basis->group_view(), iv, sec.d_x, xs + at, sec.d_y);
+                d = slot_sector(op, sec.basis->group_view(), iv, sec.d_x, xs + at, sec.d_y, j - i == 1);
                 d.tile_begin = tiles;
                 tiles += slot_tiles(d);
                 at += slot_copy_bytes(iv.slots, nvec, dtype);
                 a.max_order = std::max(a.max_order, sec.basis->order);
                 taken[todo[q]] = 1;
             }
+            a.log_group = slot_log_group(op);
+            a.chunk = slot_chunk(tiles);
             a.order = track ? a.max_order : 1;
             a.beyond_l2 = bytes > kSlotL2Bytes;
             a.total_tiles = tiles;
+            cudaError_t e = launch_slot_fill(fill.data(), (int)fill.size(), nvec, dtype, queue, s);
             if (e == cudaSuccess)
                 e = batch_gate(&a.ctl);
             a.ctl.queue = queue;

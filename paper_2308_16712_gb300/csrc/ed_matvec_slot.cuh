@@ -10,17 +10,17 @@
 //
 // Work decomposition.  The grid is persistent; a warp takes a tile of R = 1 ..
 // 16 consecutive rows (about 300 terms) and goes through three phases:
-//   A  32 / R lanes per row share the row's bond families: they form the
-//      diagonal, count the antiparallel bonds, and (after a warp scan) list
-//      them in shared memory, the terms of a row contiguous;
+//   A  a group of lanes per row (2 for a ring, 8 for a J1-J2 torus, see
+//      slot_log_group) shares the row's bond families: they form the diagonal,
+//      count the antiparallel bonds, and (after a warp scan) list them in
+//      shared memory, the terms of a row contiguous;
 //   B  one term per lane and round: the flipped state, its representative, its
 //      slot and its coefficient index go back to the list.  Every lane has
 //      work in every round but the tile's last; the pilot is read one round
 //      ahead of its use;
-//   C  the rows are summed from the list: a group of 32 / R lanes per row
-//      splits the row's terms (and, for several vectors, its columns), each
-//      lane gathers with 4 reads in flight and accumulates in registers; a
-//      shuffle tree joins the group.
+//   C  the rows are summed from the list: the row's lanes split its terms (and,
+//      for several vectors, its columns), each lane gathers with 4 reads in
+//      flight and accumulates in registers; a shuffle tree joins the group.
 // Summing in phase C takes one addition per term and vector spread over all
 // lanes.  The segmented warp scan of the term-parallel kernel it replaces took
 // 5 shuffles and 5 additions per round of 32 terms and vector (and 4 fp64
@@ -30,9 +30,9 @@
 // entries are one real number it is factored out of the sum, and no
 // multiplication is left when the characters are 1.
 //
-// The order of every sum depends only on the sector, the operator and the
-// number of vectors: results are deterministic, and the same for a sector alone
-// or in a batch.
+// The order of every sum depends only on the operator, the type and the number of
+// vectors, not on R: results are deterministic, and the same for a sector alone
+// (small R, when it is small: one round of terms per tile) or in a batch.
 #pragma once
 
 #include "ed_matvec_tp.cuh"
@@ -73,6 +73,8 @@ struct SlotArgs {
     int order;                // characters per coefficient table row: 1 when all are 1
     int scalars, stride;      // per row: scalars of a vector row, of a row of xs
     int log_parts;            // lanes that share a row's scalars
+    int log_group;            // lanes of a row: 32 >> log2 of the most rows a tile may have
+    int chunk;                // tiles taken from the queue at a time
     int beyond_l2;            // the slotted copies exceed L2: gather past L1
     uint64_t total_tiles;
     BatchCtl ctl;             // tile queue (zeroed by the fill), status word and gate
@@ -209,15 +211,21 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
     const bool plain = !kTrack && uniform;  // no coefficients at all
     const uint64_t keep = policy_keep();
     const uint32_t mat0 = sm_fam[0].mat, delta0 = sm_fam[0].delta;  // operators of one family
-    const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
 
     // Tiles from a queue: dealt statically, the warps of an SM drift apart (the
     // scheduler favours some) and a third of them had finished for most of the
     // launch (ring N=36: 45 % of the warp slots in use on average, 62 % resident).
-    uint64_t taken = 0;
-    for (uint64_t tile = next_tile(a.ctl, taken, gw, nw); tile < a.total_tiles;
-         tile = next_tile(a.ctl, taken, gw, nw)) {
+    uint64_t tile = 0, tile_end = 0;
+    while (true) {
+        if (tile == tile_end) {
+            unsigned long long t = 0;
+            if (lane == 0)
+                t = atomicAdd(a.ctl.queue, (unsigned long long)a.chunk);
+            tile = __shfl_sync(kAll, t, 0);
+            tile_end = min(tile + (uint64_t)a.chunk, a.total_tiles);
+            if (tile >= a.total_tiles)
+                break;
+        }
         int sec = 0;
         if (kBatch) {  // last sector with tile_begin <= tile (warp-uniform)
             int lo = 0, hi = a.n_sectors - 1;
@@ -234,11 +242,13 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
         const int flip = sd.flip;
         const int log_rows = sd.log_rows;
         const uint64_t row0 = (tile - sd.tile_begin) << log_rows;
+        ++tile;
 
         // ---- A: the rows and their terms ----
-        const int per_row = 32 >> log_rows;  // lanes per row
-        const int my = lane >> (5 - log_rows), sub = lane & (per_row - 1);
-        const bool valid = row0 + my < sd.dim;
+        const int per_row = 1 << a.log_group;  // lanes per row
+        const int rows = 1 << log_rows;
+        const int my = lane >> a.log_group, sub = lane & (per_row - 1);
+        const bool valid = my < rows && row0 + my < sd.dim;
         W r = 0;
         uint32_t nt = 0;
         Cplx<T> d = {T(0), T(0)};
@@ -272,14 +282,14 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
                 incl += v;
         }
         const uint32_t total = __shfl_sync(kAll, incl, 31);
-        if (sub == 0) {
+        if (sub == 0 && my < rows) {
             ws.r[my] = r;
             ws.off[my] = incl - nt;
             ws.diag[my] = d;
             ws.rinv[my] = valid ? sm_isq[__ldg(sd.norms + row0 + my)] : T(0);
         }
         if (lane == 31)
-            ws.off[1 << log_rows] = total;
+            ws.off[rows] = total;
         if (nt) {
             uint32_t k = incl - nt;
             for (int it = sub; it < n_items; it += per_row) {
@@ -346,7 +356,7 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
 
         // ---- C: gather and sum ----
         const int parts = 1 << a.log_parts;                       // lanes that share a row's scalars
-        const int log_split = max(0, 5 - log_rows - a.log_parts); // lanes that share a part's terms
+        const int log_split = max(0, a.log_group - a.log_parts);  // lanes that share a part's terms
         const int split = 1 << log_split;
         const int part = lane & (parts - 1);
         const int sp = (lane >> a.log_parts) & (split - 1);
@@ -357,13 +367,15 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
         T *y = reinterpret_cast<T *>(sd.y);
         const bool whole = a.scalars % EL == 0;
         const int group = a.log_parts + log_split;
-        for (int rr = lane >> group; rr < (1 << log_rows); rr += 32 >> group) {
+        for (int first = 0; first < rows; first += 32 >> group) {  // same trip count for all lanes
+            const int rr = first + (lane >> group);
+            const bool mine = rr < rows && e0 < a.scalars;
             T acc[EL];
 #pragma unroll
             for (int e = 0; e < EL; ++e)
                 acc[e] = T(0);
-            const uint32_t k1 = ws.off[rr + 1];
-            if (e0 < a.scalars) {
+            if (mine) {
+                const uint32_t k1 = ws.off[rr + 1];
                 for (uint32_t k = ws.off[rr] + sp; k < k1; k += 4 * split) {
                     Vec v[4];
                     uint32_t ci[4];
@@ -423,7 +435,7 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
 #pragma unroll
                 for (int e = 0; e < EL; ++e)
                     acc[e] += __shfl_xor_sync(kAll, acc[e], o << a.log_parts);
-            if (sp == 0 && e0 < a.scalars && row0 + rr < sd.dim) {
+            if (sp == 0 && mine && row0 + rr < sd.dim) {
                 const uint64_t at = (row0 + rr) * (uint32_t)a.scalars + e0;
                 Vec xv;
                 if (whole) {
@@ -506,9 +518,12 @@ cudaError_t slot_dispatch(const SlotArgs<kSec> &a, bool track, int el, cudaStrea
     return cudaErrorInvalidValue;
 }
 
-// ed_matvec.cu: a sector's descriptor (tile_begin 0) and its number of tiles
+// ed_matvec.cu: lanes of a row (log2), a sector's descriptor (tile_begin 0) and its
+// number of tiles; alone: tiles small enough to occupy the GPU
+int slot_log_group(const OpView &op);
 SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix, const void *x, const void *xs,
-                       void *y);
+                       void *y, bool alone);
+int slot_chunk(uint64_t tiles);
 uint64_t slot_tiles(const SlotSector &d);
 
 // one sector / a batch, per dtype and search, in the ed_matvec_slot_*.cu units

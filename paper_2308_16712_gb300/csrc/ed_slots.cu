@@ -157,6 +157,8 @@ __global__ void __launch_bounds__(kSlotThreads) k_slot_pilots(const uint2 *list,
     __syncthreads();
     for (int k = kMaxBucketKeys; k >= 0; --k) {
         const uint32_t first = k == (int)kMaxBucketKeys ? 0u : b.of_size[k + 1], end = b.of_size[k];
+        if (first == end)
+            continue;
         for (uint32_t q = first + tid; q < end; q += kSlotThreads) {
             const uint32_t e = b.order[q], s0 = b.start[e];
             uint32_t pilot = 0;
@@ -211,30 +213,53 @@ __global__ void __launch_bounds__(kSlotThreads) k_slot_pilots(const uint2 *list,
     }
 }
 
-// xs[slot(state_i)] = sqrt(n_i) x_i: one thread per EL scalars of a row, `lanes`
-// threads per row (a power of two; those beyond the row's scalars idle).  One
-// random write per row against some twenty random reads per row of the product
-// that follows; the state and norm streams are coalesced.  Also zeroes the tile
-// queue of that product.
-template <typename T, int EL>
-__global__ void __launch_bounds__(256) k_slot_fill(const SlotView v, const uint64_t *states, const uint16_t *norms,
-                                                   uint64_t dim, const T *x, int scalars, T *xs, int stride,
-                                                   int log_lanes, unsigned long long *queue)
+// xs[slot(state_i)] = sqrt(n_i) x_i for one sector or several: one thread per EL
+// scalars of a row, 2^log_lanes threads per row (those beyond the row's scalars
+// idle).  One random write per row against some twenty random reads per row of
+// the product that follows; the state and norm streams are coalesced.  Also
+// zeroes the tile queue of that product.
+template <int kSec>
+struct FillArgs {
+    int n_sectors, scalars, stride, log_lanes;
+    unsigned long long *queue;
+    SlotFill sec[kSec];
+    uint32_t first_block[kSec + 1];  // blocks of each sector
+};
+
+template <typename T, int EL, int kSec>
+__global__ void __launch_bounds__(256) k_slot_fill(const __grid_constant__ FillArgs<kSec> a)
 {
-    if (queue && blockIdx.x == 0 && threadIdx.x == 0)
-        *queue = 0;
-    const int part = ((int)threadIdx.x & ((1 << log_lanes) - 1)) * EL;
-    const uint64_t step = ((uint64_t)gridDim.x * blockDim.x) >> log_lanes;
+    if (a.queue && blockIdx.x == 0 && threadIdx.x == 0)
+        *a.queue = 0;
+    int sec = 0;
+    if (kSec > 1) {  // last sector whose blocks begin at or below this one
+        int lo = 0, hi = a.n_sectors - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.first_block[mid] <= blockIdx.x)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        sec = lo;
+    }
+    const SlotFill &f = a.sec[sec];
+    const uint32_t block = blockIdx.x - a.first_block[sec], blocks = a.first_block[sec + 1] - a.first_block[sec];
+    const int scalars = a.scalars;
+    const int part = ((int)threadIdx.x & ((1 << a.log_lanes) - 1)) * EL;
+    const uint64_t step = ((uint64_t)blocks * blockDim.x) >> a.log_lanes;
     const bool whole = scalars % EL == 0;
-    for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> log_lanes; i < dim + v.n_ghost; i += step) {
-        const bool ghost = i >= dim;
-        const uint64_t s = ghost ? v.ghosts[i - dim] : __ldcs(states + i);
+    const T *x = reinterpret_cast<const T *>(f.x);
+    T *xs = reinterpret_cast<T *>(f.xs);
+    for (uint64_t i = ((uint64_t)block * blockDim.x + threadIdx.x) >> a.log_lanes; i < f.dim + f.v.n_ghost; i += step) {
+        const bool ghost = i >= f.dim;
+        const uint64_t s = ghost ? f.v.ghosts[i - f.dim] : __ldcs(f.states + i);
         T w = T(0);
         if (!ghost) {
-            const uint32_t n = __ldcs(norms + i);
+            const uint32_t n = __ldcs(f.norms + i);
             w = n == 1 ? T(1) : sqrt((T)n);
         }
-        const uint64_t at = (uint64_t)slot_of(s, v) * stride + part;
+        const uint64_t at = (uint64_t)slot_of(s, f.v) * a.stride + part;
         if (part >= scalars)
             continue;
         struct __align__(sizeof(T) * EL) Vec { T e[EL]; } r;
@@ -256,19 +281,40 @@ __global__ void __launch_bounds__(256) k_slot_fill(const SlotView v, const uint6
     }
 }
 
-template <typename T, int EL>
-cudaError_t fill_launch(const IndexView &ix, const void *x, void *xs, const SlotRow &r, unsigned long long *queue,
-                        cudaStream_t s)
+template <typename T, int EL, int kSec>
+cudaError_t fill_launch(const SlotFill *sec, int n, const SlotRow &r, unsigned long long *queue, cudaStream_t s)
 {
-    int lg = 0;
-    while ((1 << lg) * EL < r.scalars)
-        ++lg;
-    const uint64_t threads = (ix.dim + ix.slots.n_ghost) << lg;
-    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((threads + 255) / 256, 152 * 64));
-    k_slot_fill<T, EL><<<grid, 256, 0, s>>>(ix.slots, ix.states, ix.norms, ix.dim, (const T *)x, r.scalars, (T *)xs,
-                                            r.stride, lg, queue);
+    static thread_local FillArgs<kSec> a;  // host staging; copied at launch
+    a.n_sectors = n;
+    a.scalars = r.scalars;
+    a.stride = r.stride;
+    a.log_lanes = 0;
+    while ((1 << a.log_lanes) * EL < r.scalars)
+        ++a.log_lanes;
+    a.queue = queue;
+    uint32_t blocks = 0;
+    for (int k = 0; k < n; ++k) {
+        a.sec[k] = sec[k];
+        a.first_block[k] = blocks;
+        const uint64_t threads = (sec[k].dim + sec[k].v.n_ghost) << a.log_lanes;
+        blocks += (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((threads + 255) / 256, 152 * 64));
+    }
+    a.first_block[n] = blocks;
+    k_slot_fill<T, EL, kSec><<<blocks, 256, 0, s>>>(a);
     count_launch();
     return cudaGetLastError();
+}
+
+template <int kSec>
+cudaError_t fill_dispatch(const SlotFill *sec, int n, const SlotRow &r, ed_dtype dtype, unsigned long long *queue,
+                          cudaStream_t s)
+{
+    if (dtype == ED_F64 || dtype == ED_C128)
+        return r.el == 1 ? fill_launch<double, 1, kSec>(sec, n, r, queue, s)
+                         : fill_launch<double, 2, kSec>(sec, n, r, queue, s);
+    return r.el == 1   ? fill_launch<float, 1, kSec>(sec, n, r, queue, s)
+           : r.el == 2 ? fill_launch<float, 2, kSec>(sec, n, r, queue, s)
+                       : fill_launch<float, 4, kSec>(sec, n, r, queue, s);
 }
 
 }  // namespace
@@ -301,61 +347,65 @@ size_t slot_copy_bytes(const SlotView &v, int nvec, ed_dtype dtype)
     return (v.n_slots * slot_row(nvec, dtype).stride * (dtype == ED_F64 || dtype == ED_C128 ? 8 : 4) + 255) / 256 * 256;
 }
 
-cudaError_t launch_slot_fill(const IndexView &ix, const void *x, void *xs, int nvec, ed_dtype dtype,
-                             unsigned long long *queue, cudaStream_t s)
+cudaError_t launch_slot_fill(const SlotFill *sec, int n, int nvec, ed_dtype dtype, unsigned long long *queue,
+                             cudaStream_t s)
 {
     const SlotRow r = slot_row(nvec, dtype);
-    if (dtype == ED_F64 || dtype == ED_C128)
-        return r.el == 1 ? fill_launch<double, 1>(ix, x, xs, r, queue, s) : fill_launch<double, 2>(ix, x, xs, r, queue, s);
-    return r.el == 1   ? fill_launch<float, 1>(ix, x, xs, r, queue, s)
-           : r.el == 2 ? fill_launch<float, 2>(ix, x, xs, r, queue, s)
-                       : fill_launch<float, 4>(ix, x, xs, r, queue, s);
+    return n == 1 ? fill_dispatch<1>(sec, n, r, dtype, queue, s) : fill_dispatch<kSlotMaxBatch>(sec, n, r, dtype, queue, s);
 }
 
 // Builds the slot index over the basis states and the weightless
 // representatives (ghosts: ownership passes to the basis on success).  False,
-// with nothing kept, when memory is short, the slots exceed 32 bits or no
-// pilots were found; the products then use the other index kinds.
-bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, cudaStream_t stream)
+// with nothing kept, when memory is short or the slots exceed 32 bits; *err
+// (device, zero) becomes 1 when no pilots were found: the caller then takes the
+// index back.  The products then use the other index kinds.
+bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, cudaStream_t stream)
 {
     if (!b->dim)
         return false;
-    uint64_t top = 0;  // the last state; weightless ones beyond it share the last cell
-    cudaError_t e = cudaMemcpyAsync(&top, b->d_states + b->dim - 1, sizeof(top), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(stream);
+    cudaError_t e = cudaSuccess;
     SlotView v{};
     v.ghosts = ghosts;
     v.n_ghost = n_ghost;
     int lg = 0;  // log2 of the cells: some 65536 states each, at most 8192 (64 KB of table)
     while (lg < 13 && (b->dim >> 17) >> lg)
         ++lg;
-    const int bits = top ? 64 - __builtin_clzll(top) : 1;
-    v.shift = std::min(63, std::max(0, bits - lg));
-    v.n_cells = (uint32_t)(top >> v.shift) + 1;
-    std::vector<uint32_t> count(v.n_cells), part_cell;
-    std::vector<uint2> cells(v.n_cells);
-    uint32_t *d_count = nullptr;
-    if (e == cudaSuccess)
-        e = ws_alloc((void **)&d_count, v.n_cells * sizeof(uint32_t), stream);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(d_count, 0, v.n_cells * sizeof(uint32_t), stream);
-    if (e == cudaSuccess) {
-        const uint64_t n = std::max<uint64_t>(v.n_cells, std::min<uint64_t>(n_ghost, 1 << 18));
-        k_cell_count<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(v, b->d_states, b->dim, d_count);
-        count_launch();
-        e = cudaMemcpyAsync(count.data(), d_count, v.n_cells * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
+    v.shift = 63;
+    v.n_cells = 1;
+    std::vector<uint32_t> count(1, (uint32_t)(b->dim + n_ghost)), part_cell;
+    if (lg) {
+        uint64_t top = 0;  // the last state; weightless ones beyond it share the last cell
+        e = cudaMemcpyAsync(&top, b->d_states + b->dim - 1, sizeof(top), cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess)
+            e = cudaStreamSynchronize(stream);
+        const int bits = top ? 64 - __builtin_clzll(top) : 1;
+        v.shift = std::min(63, std::max(0, bits - lg));
+        v.n_cells = (uint32_t)(top >> v.shift) + 1;
+        count.resize(v.n_cells);
+        uint32_t *d_count = nullptr;
+        if (e == cudaSuccess)
+            e = ws_alloc((void **)&d_count, v.n_cells * sizeof(uint32_t), stream);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(d_count, 0, v.n_cells * sizeof(uint32_t), stream);
+        if (e == cudaSuccess) {
+            const uint64_t n = std::max<uint64_t>(v.n_cells, std::min<uint64_t>(n_ghost, 1 << 18));
+            k_cell_count<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(v, b->d_states, b->dim, d_count);
+            count_launch();
+            e = cudaMemcpyAsync(count.data(), d_count, v.n_cells * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream);
+        }
+        if (e == cudaSuccess)
+            e = cudaStreamSynchronize(stream);
+        ws_free(d_count, stream);
     }
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(stream);
-    ws_free(d_count, stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
+    std::vector<uint2> cells(v.n_cells);
     uint64_t parts = 0;
+    const uint32_t part_keys = b->dim + n_ghost <= kSlotSmallMax ? kSlotSmallKeys : kSlotPartKeys;
     for (uint32_t c = 0; c < v.n_cells; ++c) {
-        const uint64_t p = ((uint64_t)count[c] + kSlotPartKeys - 1) / kSlotPartKeys;
+        const uint64_t p = ((uint64_t)count[c] + part_keys - 1) / part_keys;
         // a cell without keys is never asked for; its entry stays in bounds
         cells[c] = p ? make_uint2((uint32_t)(parts << kSlotLogB), (uint32_t)(p << kSlotLogB)) : make_uint2(0, 1);
         part_cell.insert(part_cell.end(), p, c);
@@ -369,27 +419,25 @@ bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, cudaStrea
         exc_n *= 2;
     uint8_t *pilots = nullptr;
     uint2 *exc = nullptr, *list = nullptr, *d_cells = nullptr;
-    uint32_t *cursor = nullptr, *d_part = nullptr;
+    uint32_t *cursor = nullptr;
     e = ws_alloc((void **)&pilots, parts << kSlotLogB, stream);
     if (e == cudaSuccess)
         e = ws_alloc((void **)&exc, exc_n * sizeof(uint2), stream);
+    // cells, and behind them the cell of each partition (build only)
+    cells.resize(v.n_cells + (parts + 1) / 2);
+    std::memcpy(cells.data() + v.n_cells, part_cell.data(), parts * sizeof(uint32_t));
     if (e == cudaSuccess)
-        e = ws_alloc((void **)&d_cells, v.n_cells * sizeof(uint2), stream);
-    if (e == cudaSuccess)
-        e = ws_alloc((void **)&d_part, parts * sizeof(uint32_t), stream);
+        e = ws_alloc((void **)&d_cells, cells.size() * sizeof(uint2), stream);
     if (e == cudaSuccess)
         e = ws_alloc((void **)&list, n_slots * sizeof(uint2), stream);
     if (e == cudaSuccess)
-        e = ws_alloc((void **)&cursor, (parts + 1) * sizeof(uint32_t), stream);  // + the error flag
+        e = ws_alloc((void **)&cursor, parts * sizeof(uint32_t), stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_cells, cells.data(), v.n_cells * sizeof(uint2), cudaMemcpyHostToDevice, stream);
+        e = cudaMemcpyAsync(d_cells, cells.data(), cells.size() * sizeof(uint2), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_part, part_cell.data(), parts * sizeof(uint32_t), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(cursor, 0, (parts + 1) * sizeof(uint32_t), stream);
+        e = cudaMemsetAsync(cursor, 0, parts * sizeof(uint32_t), stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(exc, 0xFF, exc_n * sizeof(uint2), stream);
-    int *err = reinterpret_cast<int *>(cursor + parts);
     v.pilots = pilots;
     v.cells = d_cells;
     v.exc = exc;
@@ -399,23 +447,18 @@ bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, cudaStrea
         const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((keys + 255) / 256, 152 * 32));
         k_slot_scatter<<<grid, 256, 0, stream>>>(v, b->d_states, b->dim, cursor, list, err);
         count_launch();
-        e = cudaFuncSetAttribute(k_slot_pilots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SlotBuild));
+        int sms = 0, per_sm = 0;
+        e = kernel_occupancy((const void *)k_slot_pilots, kSlotThreads, sizeof(SlotBuild), &sms, &per_sm);
     }
     if (e == cudaSuccess) {
-        k_slot_pilots<<<(unsigned)parts, kSlotThreads, sizeof(SlotBuild), stream>>>(list, cursor, d_part, d_cells, pilots,
+        k_slot_pilots<<<(unsigned)parts, kSlotThreads, sizeof(SlotBuild), stream>>>(list, cursor, (const uint32_t *)(d_cells + v.n_cells), d_cells, pilots,
                                                                                    exc, exc_n - 1, err);
         count_launch();
         e = cudaGetLastError();
     }
-    int failed = 0;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&failed, err, sizeof(int), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(stream);
     ws_free(list, stream);
     ws_free(cursor, stream);
-    ws_free(d_part, stream);
-    if (e != cudaSuccess || failed) {
+    if (e != cudaSuccess) {
         (void)cudaGetLastError();
         ws_free(pilots, stream);
         ws_free(exc, stream);

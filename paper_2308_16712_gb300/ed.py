@@ -420,15 +420,14 @@ def matvec_push(op: Operator, basis: Basis, x, y, stream=None):
            "edx_matvec_push")
 
 
-KERNEL_POLICIES = {"auto": 0, "rowwise": 1, "term_parallel": 2}
+KERNEL_POLICIES = {"auto": 0, "rowwise": 1, "term_parallel": 2, "slots": 3}
 
 
 def kernel_policy(policy: str) -> None:
-    """Testing aid: which matvec kernel serves one vector (or a real block of 8)
-    of an exchange-only operator: "auto" (one vector: term-parallel in single
-    precision and for more than 32 sites, row-per-lane otherwise; blocks of 8
-    vectors: term-parallel in fp32, row-per-lane in fp64), "rowwise" or
-    "term_parallel" (both precisions).  Affects later launches."""
+    """Testing aid: which matvec kernel serves an exchange-only operator: "auto"
+    (the slot kernel where the basis has a slot index, except for blocks of
+    vectors over fewer than 1024 states), "slots" (there, too), "rowwise", or
+    "term_parallel" (one vector or a real block of 8).  Affects later launches."""
     _lib.edx_kernel_policy(KERNEL_POLICIES[policy])
 
 

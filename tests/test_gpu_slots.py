@@ -25,9 +25,9 @@ CASES = [s for s in SECTORS if s[0] not in ("ring8_empty", "ring10_noU1_xx_z-")]
 @pytest.fixture(autouse=True)
 def slots_everywhere():
     torch, ed = gpu()
-    ed.slot_min_dim(1)
+    ed.kernel_policy("slots")
     yield
-    ed.slot_min_dim(0)
+    ed.kernel_policy("auto")
     ed.force_generic(False)
 
 
