@@ -17,8 +17,8 @@
 // (ed_lanczos), as in the single-vector fp32-matvec mode.
 //
 // Every reduction over the rows is a per-block partial in a fixed tile order,
-// merged by the last block to finish in block order with compensated (TwoSum)
-// merges, so both passes reproduce every coefficient bit for bit.  The
+// merged in a fixed order with compensated (TwoSum) merges (k_merge_partials),
+// so both passes reproduce every coefficient bit for bit.  The
 // per-element arithmetic is double-float on the fp32 pipe (see dd_acc); the
 // coefficient matrices, the tile sums and all merges are fp64.
 #include <cuda_runtime.h>
@@ -51,33 +51,27 @@ __device__ __forceinline__ KS ks_merge(KS a, KS b)
     return r;
 }
 
-__device__ bool last_block(unsigned int *ticket)
+// out[e] = the blocks' partials part[b * E + e] merged, one warp per entry e
+// (grid E): lane l takes blocks l, l + 32, ... in order, then a tree over the
+// lanes.  A merge is a chain of six fp64 additions, some 500 cycles; the last
+// block of the Gram kernels used to take all 608 of an entry one after the
+// other, 0.2 ms at the end of every such kernel, more than the rows of ring N=32
+// took.  Ring N=32, 8 vectors: Gram 0.49 -> 0.28 ms, update 0.57 -> 0.36 ms.
+__global__ void __launch_bounds__(32) k_merge_partials(const double2 *part, int blocks, double *out, const int *stop)
 {
-    __shared__ bool last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (*stop)
+        return;
+    const int e = blockIdx.x, E = gridDim.x;
+    KS k{0.0, 0.0};
+#pragma unroll 4
+    for (int b = threadIdx.x; b < blocks; b += 32) {
+        const double2 p = part[(size_t)b * E + e];
+        k = ks_merge(k, KS{p.x, p.y});
     }
-    __syncthreads();
-    return last;
-}
-
-// out[e] = merged block partials part[b * E + e], b in block order (the last
-// block to finish runs this; every partial is visible after the ticket)
-__device__ void merge_partials(const double2 *part, int E, double *out, unsigned int *ticket)
-{
-    for (int e = threadIdx.x; e < E; e += blockDim.x) {
-        KS k{0.0, 0.0};
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            const double2 p = __ldcg(part + (size_t)b * E + e);
-            k = ks_merge(k, KS{p.x, p.y});
-        }
-        out[e] = k.s + k.c;
-    }
-    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1)
+        k = ks_merge(k, KS{__shfl_down_sync(0xffffffffu, k.s, o), __shfl_down_sync(0xffffffffu, k.c, o)});
     if (threadIdx.x == 0)
-        *ticket = 0;
+        out[e] = k.s + k.c;
 }
 
 // ---- double-float arithmetic on the fp32 pipe --------------------------------
@@ -264,10 +258,9 @@ __device__ __forceinline__ void gram_tile(const float *sxh, const float *sxl, co
 }
 
 // Per-block partials of the Gram entries: the slices' fp64 accumulators merged
-// in slice order (compensated) through shared memory; the last block to
-// finish merges the blocks into out.
+// in slice order (compensated) through shared memory.
 template <int P, int NM>
-__device__ void gram_finish(GramAcc &acc, double *red, double2 *part, unsigned int *ticket, double *out)
+__device__ void gram_finish(GramAcc &acc, double *red, double2 *part)
 {
     using L = GramLayout<P, NM>;
     const int grp = threadIdx.x % L::kGroups, sl = threadIdx.x / L::kGroups;
@@ -286,17 +279,14 @@ __device__ void gram_finish(GramAcc &acc, double *red, double2 *part, unsigned i
             t = ks_add(t, red[(q * L::kGroups + g) * 4 + k]);
         part[(size_t)blockIdx.x * L::E + e] = make_double2(t.s, t.c);
     }
-    if (last_block(ticket))
-        merge_partials(part, L::E, out, ticket);
 }
 
-// Gram of NM double-float blocks X_m against Y (kind YK as in Prefetch):
-// out[m][a][b] = sum_i X_m[i][a] Y[i][b].
+// Gram of NM double-float blocks X_m against Y (kind YK as in Prefetch), block
+// partials of [m][a][b] = sum_i X_m[i][a] Y[i][b].
 template <int P, int NM, int YK>
 __global__ void __launch_bounds__(kBlThreads) k_dd_gram(const float *X0h, const float *X0l, const float *X1h,
                                                         const float *X1l, const void *Yh, const float *Yl,
-                                                        uint64_t n, double2 *part, unsigned int *ticket,
-                                                        double *out, const int *stop)
+                                                        uint64_t n, double2 *part, const int *stop)
 {
     if (*stop)
         return;
@@ -327,7 +317,7 @@ __global__ void __launch_bounds__(kBlThreads) k_dd_gram(const float *X0h, const 
         gram_tile<P, NM, YK != 0, kXStride<P>>(sxh, sxl, syh, syl, acc);
         __syncthreads();
     }
-    gram_finish<P, NM>(acc, red, part, ticket, out);
+    gram_finish<P, NM>(acc, red, part);
 }
 
 // ---- row-per-thread kernels: update and Cholesky QR ---------------------------
@@ -451,7 +441,7 @@ __device__ __forceinline__ void gram_tile_sym(const float *sh, const float *sl, 
 // As gram_finish, for the symmetric layout: entry (a, b) with a/2 > b/2 is
 // the transposed entry of group (b/2, a/2), so the result is exactly symmetric.
 template <int P>
-__device__ void gram_finish_sym(GramAcc &acc, double *red, double2 *part, unsigned int *ticket, double *out)
+__device__ void gram_finish_sym(GramAcc &acc, double *red, double2 *part)
 {
     using L = SymLayout<P>;
     const int grp = threadIdx.x % L::kGroups, slc = threadIdx.x / L::kGroups;
@@ -472,20 +462,17 @@ __device__ void gram_finish_sym(GramAcc &acc, double *red, double2 *part, unsign
             t = ks_add(t, red[(q * L::kGroups + g) * 4 + k]);
         part[(size_t)blockIdx.x * P * P + e] = make_double2(t.s, t.c);
     }
-    if (last_block(ticket))
-        merge_partials(part, P * P, out, ticket);
 }
 
 // W = Y - X0 C0 - X1 C1 (C fp64, P x P row-major per matrix: W[i][b] -=
 // sum_a X[i][a] C[a][b]), written as a double-float block; W may alias X1 or
 // Y (each row is read completely by its thread before that thread writes it).
-// With G: the Gram of W.
+// With gram: block partials of the Gram of W.
 template <int P, int NM, int YK>
 __global__ void __launch_bounds__(kBlThreads) k_dd_update(const float *X0h, const float *X0l, const float *X1h,
                                                           const float *X1l, const void *Yh, const float *Yl,
                                                           const double *C, float *Wh, float *Wl, uint64_t n,
-                                                          double2 *part, unsigned int *ticket, double *G,
-                                                          const int *stop)
+                                                          double2 *part, int gram, const int *stop)
 {
     if (*stop)
         return;
@@ -532,7 +519,7 @@ __global__ void __launch_bounds__(kBlThreads) k_dd_update(const float *X0h, cons
             for (int b = 0; b < P; ++b)
                 wh[b] = wl[b] = 0.f;
         }
-        if (G) {
+        if (gram) {
 #pragma unroll
             for (int b = 0; b < P; ++b) {
                 swh[threadIdx.x * L::kStride + b] = wh[b];
@@ -543,18 +530,17 @@ __global__ void __launch_bounds__(kBlThreads) k_dd_update(const float *X0h, cons
             __syncthreads();
         }
     }
-    if (G)
-        gram_finish_sym<P>(acc, red, part, ticket, G);
+    if (gram)
+        gram_finish_sym<P>(acc, red, part);
 }
 
 // Cholesky QR steps on the block W (double-float, in place).  kApply = false:
-// Z = W R1i (R1i fp64 upper triangular, row-major) and the Gram of Z into G2;
+// Z = W R1i (R1i fp64 upper triangular, row-major), block partials of its Gram;
 // kApply = true: W = W (R1i R2i), the product of the two upper triangular
 // inverses formed in fp64 (CholQR2 applied at once).
 template <int P, bool kApply>
 __global__ void __launch_bounds__(kBlThreads) k_dd_qr(float *Wh, float *Wl, const double *R1i, const double *R2i,
-                                                      uint64_t n, double2 *part, unsigned int *ticket,
-                                                      double *G2, const int *stop)
+                                                      uint64_t n, double2 *part, const int *stop)
 {
     if (*stop)
         return;
@@ -618,7 +604,7 @@ __global__ void __launch_bounds__(kBlThreads) k_dd_qr(float *Wh, float *Wl, cons
         }
     }
     if (!kApply)
-        gram_finish_sym<P>(acc, red, part, ticket, G2);
+        gram_finish_sym<P>(acc, red, part);
 }
 
 // psi (double-float, dim) += V_j s_j  (s_j = y[j P .. j P + P) in fp64); psi
@@ -1042,11 +1028,11 @@ struct Pool {
 // number of earlier blocks (1 or 2) the new one is orthogonalised against.
 template <int P>
 void launch_gram(int nm, int yk, const float *X0h, const float *X0l, const float *X1h, const float *X1l,
-                 const void *Yh, const float *Yl, uint64_t n, int grid, double2 *part, unsigned int *ticket,
-                 double *out, const int *stop, cudaStream_t st)
+                 const void *Yh, const float *Yl, uint64_t n, int grid, double2 *part, double *out, const int *stop,
+                 cudaStream_t st)
 {
 #define ED_DD_GRAM(NM, YK) \
-    k_dd_gram<P, NM, YK><<<grid, kBlThreads, 0, st>>>(X0h, X0l, X1h, X1l, Yh, Yl, n, part, ticket, out, stop)
+    k_dd_gram<P, NM, YK><<<grid, kBlThreads, 0, st>>>(X0h, X0l, X1h, X1l, Yh, Yl, n, part, stop)
     if (nm == 1) {
         if (yk == 0) ED_DD_GRAM(1, 0); else if (yk == 1) ED_DD_GRAM(1, 1); else ED_DD_GRAM(1, 2);
     } else {
@@ -1054,16 +1040,17 @@ void launch_gram(int nm, int yk, const float *X0h, const float *X0l, const float
     }
 #undef ED_DD_GRAM
     count_launch();
+    k_merge_partials<<<nm * P * P, 32, 0, st>>>(part, grid, out, stop); count_launch();
 }
 
 template <int P>
 void launch_update(int nm, int yk, const float *X0h, const float *X0l, const float *X1h, const float *X1l,
                    const void *Yh, const float *Yl, const double *C, float *Wh, float *Wl, uint64_t n, int grid,
-                   double2 *part, unsigned int *ticket, double *G, const int *stop, cudaStream_t st)
+                   double2 *part, double *G, const int *stop, cudaStream_t st)
 {
 #define ED_DD_UPD(NM, YK)                                                                                  \
-    k_dd_update<P, NM, YK><<<grid, kBlThreads, 0, st>>>(X0h, X0l, X1h, X1l, Yh, Yl, C, Wh, Wl, n, part, ticket, \
-                                                        G, stop)
+    k_dd_update<P, NM, YK><<<grid, kBlThreads, 0, st>>>(X0h, X0l, X1h, X1l, Yh, Yl, C, Wh, Wl, n, part, \
+                                                        G ? 1 : 0, stop)
     if (nm == 1) {
         if (yk == 0) ED_DD_UPD(1, 0); else if (yk == 1) ED_DD_UPD(1, 1); else ED_DD_UPD(1, 2);
     } else {
@@ -1071,6 +1058,9 @@ void launch_update(int nm, int yk, const float *X0h, const float *X0l, const flo
     }
 #undef ED_DD_UPD
     count_launch();
+    if (G) {
+        k_merge_partials<<<P * P, 32, 0, st>>>(part, grid, G, stop); count_launch();
+    }
 }
 
 template <int P>
@@ -1103,7 +1093,6 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     double *V64 = nullptr, *W64 = nullptr, *A = nullptr, *B = nullptr, *sm = nullptr;
     double *y = nullptr, *eig = nullptr, *scr = nullptr;
     double2 *part = nullptr;
-    unsigned int *tickets = nullptr;
     int *flags = nullptr;  // [0] stop, [1] m_eff (running), [2] m_eff of the main pass
     ED_BL_TRY(S.get(&Vh, (size_t)nblocks * blk));
     ED_BL_TRY(S.get(&Vl, (size_t)nblocks * blk));
@@ -1126,9 +1115,7 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     ED_BL_TRY(S.get(&bracket, (size_t)kBandMaxRounds * std::max(n_eig, 1) * 3));
     ED_BL_TRY(S.get(&bfirst, (size_t)kBandMaxRounds * std::max(n_eig, 1)));
     ED_BL_TRY(S.get(&part, (size_t)grid * 2 * P * P));
-    ED_BL_TRY(S.get(&tickets, 4));
     ED_BL_TRY(S.get(&flags, 3));
-    ED_BL_TRY(cudaMemsetAsync(tickets, 0, 4 * sizeof(unsigned int), st));
     ED_BL_TRY(cudaMemsetAsync(A, 0, (size_t)(steps + 1) * P * P * sizeof(double), st));
     ED_BL_TRY(cudaMemsetAsync(B, 0, (size_t)(steps + 2) * P * P * sizeof(double), st));
 
@@ -1164,10 +1151,11 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
 
     // Cholesky QR (twice) of the block (wh, wl) in place; R1 already in sm
     auto qr = [&](float *wh, float *wl, int j) {
-        k_dd_qr<P, false><<<rgrid, kBlThreads, 0, st>>>(wh, wl, R1i, nullptr, n, part, tickets + 2, G2, stop);
+        k_dd_qr<P, false><<<rgrid, kBlThreads, 0, st>>>(wh, wl, R1i, nullptr, n, part, stop);
         count_launch();
+        k_merge_partials<<<P * P, 32, 0, st>>>(part, rgrid, G2, stop); count_launch();
         k_bl_small<P><<<1, 32, 0, st>>>(sm, A, B, j, 2, stop, flags + 1); count_launch();
-        k_dd_qr<P, true><<<rgrid, kBlThreads, 0, st>>>(wh, wl, R1i, R2i, n, part, tickets + 2, nullptr, stop);
+        k_dd_qr<P, true><<<rgrid, kBlThreads, 0, st>>>(wh, wl, R1i, R2i, n, part, stop);
         count_launch();
     };
 
@@ -1177,7 +1165,7 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
         if (e != cudaSuccess)
             return e;
         k_f64_to_dd<<<vgrid, 256, 0, st>>>(x0, bh(0), bl(0), blk); count_launch();
-        launch_gram<P>(1, 2, bh(0), bl(0), nullptr, nullptr, bh(0), bl(0), n, grid, part, tickets, G, stop, st);
+        launch_gram<P>(1, 2, bh(0), bl(0), nullptr, nullptr, bh(0), bl(0), n, grid, part, G, stop, st);
         k_bl_small<P><<<1, 32, 0, st>>>(sm, A, B, -1, 1, stop, flags + 1); count_launch();
         qr(bh(0), bl(0), -1);
         for (int j = 0; j < steps; ++j) {
@@ -1203,19 +1191,19 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
             if ((e = mark()) != cudaSuccess)
                 return e;
             const int nm = j ? 2 : 1;
-            launch_gram<P>(nm, yk, Vjh, Vjl, Vph, Vpl, Yh, nullptr, n, grid, part, tickets, C, stop, st);
+            launch_gram<P>(nm, yk, Vjh, Vjl, Vph, Vpl, Yh, nullptr, n, grid, part, C, stop, st);
             k_bl_small<P><<<1, 32, 0, st>>>(sm, A, B, j, 0, stop, flags + 1); count_launch();
-            launch_update<P>(nm, yk, Vjh, Vjl, Vph, Vpl, Yh, nullptr, C, Wh, Wl, n, rgrid, part, tickets + 1,
+            launch_update<P>(nm, yk, Vjh, Vjl, Vph, Vpl, Yh, nullptr, C, Wh, Wl, n, rgrid, part,
                              reorth ? nullptr : G, stop, st);
             if (reorth) {  // against every kept block, block modified Gram-Schmidt, twice
                 for (int rep = 0; rep < 2; ++rep)
                     for (int i = 0; i <= j; ++i) {
-                        launch_gram<P>(1, 2, bh(i), bl(i), nullptr, nullptr, Wh, Wl, n, grid, part, tickets, C,
+                        launch_gram<P>(1, 2, bh(i), bl(i), nullptr, nullptr, Wh, Wl, n, grid, part, C,
                                        stop, st);
                         launch_update<P>(1, 2, bh(i), bl(i), nullptr, nullptr, Wh, Wl, C, Wh, Wl, n, rgrid, part,
-                                         tickets + 1, nullptr, stop, st);
+                                         nullptr, stop, st);
                     }
-                launch_gram<P>(1, 2, Wh, Wl, nullptr, nullptr, Wh, Wl, n, grid, part, tickets, G, stop, st);
+                launch_gram<P>(1, 2, Wh, Wl, nullptr, nullptr, Wh, Wl, n, grid, part, G, stop, st);
             }
             k_bl_small<P><<<1, 32, 0, st>>>(sm, A, B, j, 1, stop, flags + 1); count_launch();
             qr(Wh, Wl, j);
