@@ -21,6 +21,12 @@
 // lanes idling while others start rows or walk their term lists), and the
 // summation order depends only on the tile layout: deterministic, and
 // identical for a sector alone or inside a batch of sectors.
+//
+// Small sectors (at most kTpSmallTiles tiles, fp32) take a block per tile
+// instead of a warp: its eight warps lay the tile out alike, share its rounds,
+// and one adds the rounds' sums in their order, so the result keeps every bit.
+// A product is then some two rounds long instead of ten: ring N=20 (2518 states)
+// 29 -> 11 us.
 #pragma once
 
 #include <type_traits>
@@ -31,6 +37,8 @@ namespace edk {
 
 constexpr int kTpThreads = 256;
 constexpr int kTpWarps = kTpThreads / 32;
+constexpr uint64_t kTpSmallTiles = 608;  // resident at once, four blocks per SM
+constexpr int kTpSmallTerms = 64;        // rounds of a tile, at most (32 rows x 64 terms)
 
 template <int kSec>
 struct TpArgs {
@@ -236,11 +244,12 @@ constexpr int kTpMinBlocks = NV > 1 ? 4 : (sizeof(W) == 4 && kIdx != 2 ? 8 : 5);
 // 16-byte entries, 2 bucketed index (find_bucketed).  NV > 1: a real block of
 // NV interleaved vectors (one search and lookup per term serves them all).
 template <typename W, typename T, bool kC, bool kTrack, bool kFact, int kIdx, int kSec, bool kPush = false,
-          int NV = 1>
-__global__ void __launch_bounds__(kTpThreads, kTpMinBlocks<W, kIdx, NV>)
+          int NV = 1, bool kSmall = false>
+__global__ void __launch_bounds__(kTpThreads, kSmall ? 4 : kTpMinBlocks<W, kIdx, NV>)
     k_matvec_tp(const __grid_constant__ TpArgs<kSec> a)
 {
     static_assert(NV == 1 || (!kC && !kPush), "blocks: real, pull form");
+    static_assert(!kSmall || (NV == 1 && !kPush && kSec == 1), "one vector, one sector, pull form");
     using V = TpVal<T, kC, NV>;
     using E = std::conditional_t<kIdx == 1, ulonglong2, uint2>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -298,9 +307,10 @@ __global__ void __launch_bounds__(kTpThreads, kTpMinBlocks<W, kIdx, NV>)
     const uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
 
+    V *sm_part = reinterpret_cast<V *>(smem + tp_terms_offset<W, T, V>(off[7]) + (size_t)kTpWarps * 32 * tstride);
     uint64_t taken = 0;
-    for (uint64_t tile = next_tile(a.ctl, taken, gw, nw); tile < a.total_tiles;
-         tile = next_tile(a.ctl, taken, gw, nw)) {
+    auto take = [&]() { return kSmall ? (taken++) * gridDim.x + blockIdx.x : next_tile(a.ctl, taken, gw, nw); };
+    for (uint64_t tile = take(); tile < a.total_tiles; tile = take()) {
         int sec = 0;
         if (kSec > 1) {  // last sector with tile_begin <= tile (warp-uniform)
             int lo = 0, hi = a.n_sectors - 1;
@@ -398,7 +408,7 @@ __global__ void __launch_bounds__(kTpThreads, kTpMinBlocks<W, kIdx, NV>)
         const E *__restrict__ hent = reinterpret_cast<const E *>(sd.hent);
         const uint32_t *__restrict__ htab = sd.htab;
         const int hbits = sd.hbits, norm_bits = sd.norm_bits;
-        for (uint32_t base = 0; base < total; base += 32) {
+        for (uint32_t base = kSmall ? (threadIdx.x & ~31u) : 0u; base < total; base += kSmall ? kTpThreads : 32) {
             // rows whose terms start in this round, and the row carried in
             const bool starts = nt > 0 && offl >= base && offl < base + 32;
             if (starts)
@@ -536,13 +546,28 @@ __global__ void __launch_bounds__(kTpThreads, kTpMinBlocks<W, kIdx, NV>)
                         val = vadd(val, up);
                 }
                 const bool seg_end = act && (lane == 31 || t + 1 == total || ((M >> (lane + 1)) & 1u));
-                if (seg_end)
-                    ws.acc[rho] = vadd(ws.acc[rho], val);
+                if (seg_end) {
+                    if constexpr (kSmall)
+                        sm_part[base + rho] = val;  // round base / 32, row rho
+                    else
+                        ws.acc[rho] = vadd(ws.acc[rho], val);
+                }
             }
             __syncwarp();
         }
-        if (!kPush && valid)
+        if constexpr (kSmall) {
+            __syncthreads();
+            if (threadIdx.x < 32 && valid) {
+                V sum = ws.acc[lane];
+                if (nt)
+                    for (uint32_t q = offl >> 5; q <= (offl + nt - 1) >> 5; ++q)
+                        sum = vadd(sum, sm_part[q * 32 + lane]);
+                store_cs(reinterpret_cast<V *>(sd.y) + row, sum);
+            }
+            __syncthreads();
+        } else if (!kPush && valid) {
             store_cs(reinterpret_cast<V *>(sd.y) + row, ws.acc[lane]);
+        }
         __syncwarp();
     }
 }
@@ -552,8 +577,20 @@ template <typename W, typename T, bool kC, bool kTrack, bool kFact, int kIdx, in
 cudaError_t tp_launch(const TpArgs<kSec> &a, cudaStream_t stream)
 {
     using V = TpVal<T, kC, NV>;
-    auto kern = k_matvec_tp<W, T, kC, kTrack, kFact, kIdx, kSec, kPush, NV>;
     const size_t smem = tp_smem_bytes<W, T, V, kFact>(a.g, a.op, a.n_sectors, a.max_order);
+    if constexpr (kSec == 1 && !kPush && NV == 1 && sizeof(T) == 4) {
+        if (a.total_tiles <= kTpSmallTiles && a.op.max_terms <= kTpSmallTerms) {
+            auto small = k_matvec_tp<W, T, kC, kTrack, kFact, kIdx, kSec, kPush, NV, true>;
+            const size_t bytes = smem + (size_t)a.op.max_terms * 32 * sizeof(V);
+            int sms = 0, per_sm = 0;
+            const cudaError_t e = kernel_occupancy((const void *)small, kTpThreads, bytes, &sms, &per_sm);
+            if (e != cudaSuccess)
+                return e;
+            small<<<(unsigned)a.total_tiles, kTpThreads, bytes, stream>>>(a); count_launch();
+            return cudaGetLastError();
+        }
+    }
+    auto kern = k_matvec_tp<W, T, kC, kTrack, kFact, kIdx, kSec, kPush, NV>;
     int sms = 0, per_sm = 0;
     const cudaError_t e = kernel_occupancy((const void *)kern, kTpThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
