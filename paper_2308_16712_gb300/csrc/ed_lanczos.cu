@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag_lowest(const double *al
     double scale;
     const int me = tri_effective_size(alpha, beta, m, scale);
     const double lam = tri_solve(alpha, beta, me, 0, sm, work);
-    tri_vector(alpha, beta, me, lam, scale, y, work + m);
+    tri_vector(alpha, beta, me, lam, scale, y, sm, work + m);
     for (int i = me + (int)threadIdx.x; i < m; i += kTriThreads)
         y[i] = 0.0;
     if (threadIdx.x == 0) {

@@ -56,7 +56,7 @@ __device__ __forceinline__ KS ks_merge(KS a, KS b)
 // lanes.  A merge is a chain of six fp64 additions, some 500 cycles; the last
 // block of the Gram kernels used to take all 608 of an entry one after the
 // other, 0.2 ms at the end of every such kernel, more than the rows of ring N=32
-// took.  Ring N=32, 8 vectors: Gram 0.49 -> 0.28 ms, update 0.57 -> 0.36 ms.
+// took.  Ring N=32, 8 vectors: Gram 0.49 -> 0.29 ms, update 0.57 -> 0.40 ms.
 __global__ void __launch_bounds__(32) k_merge_partials(const double2 *part, int blocks, double *out, const int *stop)
 {
     if (*stop)

@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kTriThreads) k_seg_tridiag(const double *alpha
     double scl;
     const int me = tri_effective_size(a, b, m, scl);
     const double lam = tri_solve(a, b, me, 0, sm, ws);
-    tri_vector(a, b, me, lam, scl, ys, ws + stride);
+    tri_vector(a, b, me, lam, scl, ys, sm, ws + stride);
     for (int i = me + (int)threadIdx.x; i < m; i += kTriThreads)
         ys[i] = 0.0;
     if (threadIdx.x == 0) {

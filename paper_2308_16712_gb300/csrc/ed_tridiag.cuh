@@ -3,21 +3,22 @@
 // iteration, one block per matrix: shared by the single- and many-sector Lanczos
 // solvers.
 //
-// Bound by the latency of one chain of fp64 operations per step (a division
-// takes some 900 cycles on this GPU, a fused multiply-add some 80), not by
-// throughput: a count is one block-wide evaluation at kTriThreads points, so a
-// round brackets an eigenvalue 257 times more narrowly instead of 33 times,
-// the counts use the division-free form of the sequence, and the pivots of the
-// inverse iteration are divided out once instead of in each of its passes.
-// Matrix of 100 steps: 1.08 -> 0.15 ms; of 50: 0.32 -> 0.08 ms.
+// Bound by chains of fp64 operations (a division takes some 900 cycles on this
+// GPU, a multiply-add some 80, and an SM sub-partition starts one for a warp
+// every 75), not by work: a count is one block-wide evaluation with one warp per
+// sub-partition, so a round brackets an eigenvalue 129 times more narrowly
+// instead of 33 times; the counts use the division-free form of the sequence;
+// the pivots of the inverse iteration are divided out once instead of in each of
+// its passes; and its chains run on shared memory.  Matrices of 50 and of 6 steps
+// together: 0.65 -> 0.21 ms (0.29 with 256 threads and the chains in memory).
 #pragma once
 
 #include <cuda_runtime.h>
 
 namespace edk {
 
-constexpr int kTriThreads = 256;
-constexpr int kTriShared = 1024;  // matrices up to this size are counted from shared memory
+constexpr int kTriThreads = 128;
+constexpr int kTriShared = 768;  // matrices up to this size are worked on in shared memory
 
 // Number of eigenvalues below x: sign changes of p_0 = 1, p_1 = a_0 - x,
 // p_{i+1} = (a_i - x) p_i - b_i^2 p_{i-1} (b2[i] = b_i^2 couples i-1 and i),
@@ -126,6 +127,7 @@ __device__ __forceinline__ void tri_interval(const double *a, const double *b, i
 
 struct TriShared {
     double a[kTriShared], b2[kTriShared];
+    double b[kTriShared], y[kTriShared], l[kTriShared], rd[kTriShared];
 };
 
 // Eigenvalue k of the leading me x me matrix; sm holds its entries when they fit
@@ -145,13 +147,20 @@ __device__ __forceinline__ double tri_solve(const double *a, const double *b, in
     return tri_eigenvalue(fits ? sm.a : a, q, me, k, lo, hi);
 }
 
-// y[0..me) = normalised eigenvector for the eigenvalue lam by inverse iteration
+// y_out[0..me) = normalised eigenvector for the eigenvalue lam by inverse iteration
 // (four passes from the all-ones vector; LU without pivoting, guarded pivots);
-// work: 2 me doubles.  The chains run in one thread.
-__device__ __forceinline__ void tri_vector(const double *a, const double *b, int me, double lam, double scale, double *y,
-                                           double *work)
+// work: 2 me doubles, used when sm has no room.  The chains run in one thread.
+__device__ __forceinline__ void tri_vector(const double *a, const double *b_in, int me, double lam, double scale,
+                                           double *y_out, TriShared &sm, double *work)
 {
-    double *rd = work, *l = work + me;  // reciprocal pivots, multipliers
+    const bool fits = me <= kTriShared;
+    double *rd = fits ? sm.rd : work, *l = fits ? sm.l : work + me;  // reciprocal pivots, multipliers
+    double *y = fits ? sm.y : y_out;
+    const double *b = fits ? sm.b : b_in;
+    if (fits)
+        for (int i = threadIdx.x; i < me; i += kTriThreads)
+            sm.b[i] = b_in[i];
+    __syncthreads();
     const double eps = 1e-15 * fmax(scale, 1e-300);
     if (threadIdx.x == 0) {
         double piv = a[0] - lam;
@@ -193,6 +202,9 @@ __device__ __forceinline__ void tri_vector(const double *a, const double *b, int
             y[i] *= r;
         __syncthreads();
     }
+    if (fits)
+        for (int i = threadIdx.x; i < me; i += kTriThreads)
+            y_out[i] = y[i];
 }
 
 }  // namespace edk
