@@ -98,6 +98,64 @@ __device__ __forceinline__ int rep_norm_fact(W s, const uint8_t *kinds, const W 
     return rep ? (ok ? stab : -1) : 0;
 }
 
+// Not decided by rep_norm_rot1.
+constexpr int kNormOpen = -2;
+
+// Same test for the translations of a ring: s is a representative if no coset
+// image has a smaller minimum (rep_search_rot1, one coset at a time), and only
+// the identity fixes it if no other coset reaches s, no rotation by n / p (p a
+// prime factor of n, plan.turn) does, and the half turn does not complement it:
+// any further element of the stabiliser has one of these as a power.  The few
+// states with more symmetry are left to rep_norm_fact (kNormOpen).  known: s is
+// a representative.  Bound by integer issue slots like the search: some 250
+// instructions against 3000 for the 72 images of ring N=36 (a warp always holds
+// a state for which every image counts): both passes of its basis 37 -> 10 ms.
+template <typename W>
+__device__ __forceinline__ int rep_norm_rot1(W s, const uint8_t *kinds, const W *masks, const uint32_t *one,
+                                             const GroupView &g, const EnumPlan &plan, W full, bool known)
+{
+    const int n = g.n_sites;
+    GroupView ring = g;  // the rotations alone
+    ring.cos_rev = -1;
+    ring.n_cos = 0;
+    bool alone = true;
+    for (int c = 0; c < g.n_cos; ++c) {
+        const bool id = c == g.cos_id;
+        if (id && known)
+            continue;
+        W best;
+        int gbest;
+        rep_search_rot1<W, false>(coset_image(s, (int)kinds[c], masks + c * kMaskStride, n), kinds, masks, ring,
+                                  g.flip, full, best, gbest);
+        if (best < s)
+            return 0;
+        alone = alone && (id || best != s);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        alone = alone && (!plan.turn[i] || rotl_n(s, plan.turn[i], n, full) != s);
+    if (g.flip && n % 2 == 0)
+        alone = alone && rotl_n(s, n / 2, n, full) != (W)(s ^ full);
+    return !alone ? kNormOpen : chi_is_one(one, g.cos_id * n) ? 1 : -1;
+}
+
+// Same test for the translations of a torus, over the candidates of
+// rep_search_blocks: every element that makes the minimum is one of them.
+template <typename W>
+__device__ __forceinline__ int rep_norm_blocks(W s, const W *masks, const uint32_t *one, const GroupView &g, W full)
+{
+    int stab = 0;
+    bool ok = true;
+    const bool rep = blocks_candidates<W>(s, masks, g, g.flip, full, [&](W q, int gi) {
+        if (q == s) {
+            ++stab;
+            ok = ok && chi_is_one(one, gi);
+        }
+        return q >= s;
+    });
+    return rep ? (ok ? stab : -1) : 0;
+}
+
 __host__ __device__ inline size_t enum_smem_bytes(const GroupView &g, size_t wbytes, bool fact)
 {
     const int nm = fact ? g.n_cos : g.n_perm;
@@ -186,6 +244,18 @@ __global__ void __launch_bounds__(kEnumThreads) k_enumerate(EnumPlan plan, Group
             sm_kind[e] = g.cos_kind[e];
     __syncthreads();
     const W full = (W)g.full;
+    auto norm_of = [&](W s, bool known) {
+        if constexpr (kFact) {
+            int nrm = kNormOpen;
+            if (g.prune == 1)
+                nrm = rep_norm_rot1<W>(s, sm_kind, sm_masks, sm_one, g, plan, full, known);
+            else if (g.prune == 2)
+                nrm = rep_norm_blocks<W>(s, sm_masks, sm_one, g, full);
+            return nrm != kNormOpen ? nrm : rep_norm_fact<W>(s, sm_kind, sm_masks, sm_one, g, full);
+        } else {
+            return rep_norm<W>(s, sm_masks, sm_one, g.n_perm, g.flip, full);
+        }
+    };
     for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < plan.n_chunks;
          c += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t r0 = c * plan.chunk;
@@ -198,17 +268,14 @@ __global__ void __launch_bounds__(kEnumThreads) k_enumerate(EnumPlan plan, Group
         uint32_t word = 0;
         for (uint64_t q = 0; q < cnt; ++q) {
             const uint64_t s = walk.state();
-            int nrm;
+            int nrm = 0;
             if (kWrite && cflags) {  // only the states the count pass kept
                 if ((q & 31) == 0)
                     word = cflags[q >> 5];
-                nrm = (word >> (q & 31)) & 1u
-                          ? (kFact ? rep_norm_fact<W>((W)s, sm_kind, sm_masks, sm_one, g, full)
-                                   : rep_norm<W>((W)s, sm_masks, sm_one, g.n_perm, g.flip, full))
-                          : 0;
+                if ((word >> (q & 31)) & 1u)
+                    nrm = norm_of((W)s, true);
             } else {
-                nrm = kFact ? rep_norm_fact<W>((W)s, sm_kind, sm_masks, sm_one, g, full)
-                            : rep_norm<W>((W)s, sm_masks, sm_one, g.n_perm, g.flip, full);
+                nrm = norm_of((W)s, false);
             }
             if (!kWrite && nrm < 0 && plan.ghosts) {
                 const uint32_t at = atomicAdd(plan.ghost_count, 1u);
@@ -258,10 +325,17 @@ cudaError_t enum_launch(const EnumPlan &plan, const GroupView &g, uint32_t *coun
 }
 
 template <bool kWrite>
-cudaError_t enum_dispatch(const EnumPlan &plan, const GroupView &g, uint32_t *counts,
+cudaError_t enum_dispatch(EnumPlan plan, const GroupView &g, uint32_t *counts,
                           const uint64_t *offsets, uint64_t *states, uint16_t *norms,
                           cudaStream_t stream)
 {
+    int m = plan.n_sites, at = 0;
+    for (int p = 2; p <= m; ++p) {  // at most three prime factors up to 64 sites
+        if (m % p == 0)
+            plan.turn[at++] = plan.n_sites / p;
+        while (m % p == 0)
+            m /= p;
+    }
     const bool u1 = plan.n_up >= 0;
 #define ED_ENUM(W, U1)                                                                           \
     return g.fact ? enum_launch<W, U1, kWrite, true>(plan, g, counts, offsets, states, norms, stream) \

@@ -48,6 +48,7 @@ struct EnumPlan {
     uint32_t n_seg = 0;
     int low_bits = 0;
     int odd = 0;                           // 1: bit 0 is set in every state
+    int turn[3] = {0, 0, 0};               // set by the launch: n_sites / p for its prime factors p
 };
 
 // The values of the top `bits` bits (bits < n_sites) a representative can

@@ -420,9 +420,11 @@ __host__ __device__ __forceinline__ uint32_t read_table(const uint32_t *p)
 #endif
 }
 
-template <typename W, bool kTrack>
-__host__ __device__ __forceinline__ void rep_search_blocks(W s, const W *masks, const GroupView &g, int flip, W full,
-                                                           W &best, int &gbest)
+// Visits those candidates, f(image, factored index), until f returns false;
+// returns whether it never did.
+template <typename W, typename F>
+__host__ __device__ __forceinline__ bool blocks_candidates(W s, const W *masks, const GroupView &g, int flip, W full,
+                                                           F &&f)
 {
     const uint32_t *tab = g.blk_tab + (flip ? 1u << g.blk_bits : 0u);
     const int n = g.n_sites, d = g.rot_d, L = g.rot_L;
@@ -435,8 +437,7 @@ __host__ __device__ __forceinline__ void rep_search_blocks(W s, const W *masks, 
         low = k < low ? k : low;
         at |= (k == low ? 1u : 0u) << z;
     }
-    W bst = ~W(0);
-    int gb = 0, b = 0;
+    int b = 0;
     uint32_t who = 0;
     while (who | at) {
         if (!who) {
@@ -448,20 +449,34 @@ __host__ __device__ __forceinline__ void rep_search_blocks(W s, const W *masks, 
         }
         const int t = lowest_set(who);
         who &= who - 1;
-        const bool f = t >= d;
-        const int a = f ? t - d : t;
+        const bool inv = t >= d;
+        const int a = inv ? t - d : t;
         W q = rotl_n(rotate_blocks(s, masks + a * kMaskStride), b * d, n, full);
-        if (f)
+        if (inv)
             q ^= full;
+        if (!f(q, a * L + b + (inv ? g.n_perm : 0)))
+            return false;
+    }
+    return true;
+}
+
+template <typename W, bool kTrack>
+__host__ __device__ __forceinline__ void rep_search_blocks(W s, const W *masks, const GroupView &g, int flip, W full,
+                                                           W &best, int &gbest)
+{
+    W bst = ~W(0);
+    int gb = 0;
+    blocks_candidates<W>(s, masks, g, flip, full, [&](W q, int gi) {
         if (kTrack) {
             if (q < bst) {
                 bst = q;
-                gb = a * L + b + (f ? g.n_perm : 0);
+                gb = gi;
             }
         } else {
             bst = q < bst ? q : bst;
         }
-    }
+        return true;
+    });
     best = bst;
     gbest = gb;
 }
