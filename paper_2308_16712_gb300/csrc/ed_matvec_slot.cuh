@@ -81,10 +81,15 @@ struct SlotArgs {
     SlotSector sec[kSec];     // read from the launch parameters (constant bank)
 };
 
+// A warp's shared memory: this, the term list (phase A: site | row << 6 |
+// (2 family + c) << 10, phase B: slot), and the terms' coefficient indices unless
+// the sum has none.  The list is sized for the operator, because what is left of
+// an SM's 256 KB is its L1, and every gather on its way occupies a line there:
+// with a list of 640 terms and indices for all (196 KB at five or six blocks)
+// the 6x6 torus complex128 took 372 instead of 207 ms, ring N=32 fp32 1.07
+// instead of 0.96; six blocks of ring N=32's 48 products of 8 vectors 74 -> 47 ms.
 template <typename W, typename T>
-struct SlotWarp {
-    uint32_t term[kSlTerms];            // phase A: site | row << 6 | (2 family + c) << 10; phase B: slot
-    uint16_t coef[kSlTerms];
+struct __align__(16) SlotWarp {
     W r[kSlMaxRows];
     uint32_t off[kSlMaxRows + 1];
     T rinv[kSlMaxRows];
@@ -122,19 +127,38 @@ __host__ __device__ inline void slot_smem_layout(const GroupView &g, const OpVie
     off[6] = align16(off[5] + (size_t)(max_order + 1) * sizeof(T));              // warps
 }
 
+__host__ __device__ inline uint32_t slot_list_terms(const OpView &op, int log_group)
+{
+    return (uint32_t)op.max_terms << (5 - log_group);
+}
+
+template <typename W, typename T>
+__host__ __device__ inline size_t slot_warp_bytes(const OpView &op, int log_group, bool plain)
+{
+    const size_t terms = slot_list_terms(op, log_group);
+    return align16(sizeof(SlotWarp<W, T>) + terms * 4 + (plain ? 0 : terms * 2));
+}
+
 template <typename W, typename T, bool kFact>
 __host__ __device__ inline size_t slot_smem_bytes(const GroupView &g, const OpView &op, int order, int max_order,
-                                                  bool batch)
+                                                  int log_group, bool batch, bool plain)
 {
     size_t off[7];
     slot_smem_layout<W, T, kFact>(g, op, order, max_order, batch, off);
-    return off[6] + kSlWarps * sizeof(SlotWarp<W, T>);
+    return off[6] + kSlWarps * slot_warp_bytes<W, T>(op, log_group, plain);
 }
 
 // kSearch: 0 every element of the group (factored or not), 1 ring runs, 2 torus
 // row keys.  EL: scalars per lane and access.
+// Blocks per SM, by registers: a word of 32 bits and single precision fit 32 of
+// them (a few spill; ring N=32 fp32 0.96 -> 0.90 ms), in double precision that
+// costs more than the warps give (lanczos of ring N=32 fp64 115 -> 130 ms), and a
+// sixth block for 64-bit words changes nothing (they wait for DRAM).
+template <typename W, typename T, bool kTrack>
+constexpr int kSlBlocks = sizeof(W) == 8 ? 5 : sizeof(T) == 4 && !kTrack ? 8 : 6;
+
 template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int kSec>
-__global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_slot(const __grid_constant__ SlotArgs<kSec> a)
+__global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack>) k_matvec_slot(const __grid_constant__ SlotArgs<kSec> a)
 {
     static_assert(!kC || EL % 2 == 0, "a complex number per lane at least");
     constexpr bool kBatch = kSec > 1;
@@ -152,7 +176,12 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
     uint8_t *sm_off = smem + off[3] + slot_table_bytes<T>(a.op, a.order, kBatch);
     uint8_t *sm_kind = smem + off[4];
     T *sm_isq = reinterpret_cast<T *>(smem + off[5]);
-    SlotWarp<W, T> &ws = reinterpret_cast<SlotWarp<W, T> *>(smem + off[6])[threadIdx.x >> 5];
+    const bool uniform = a.op.uniform != 0;
+    const bool plain = !kTrack && uniform;  // no coefficients at all
+    SlotWarp<W, T> &ws = *reinterpret_cast<SlotWarp<W, T> *>(
+        smem + off[6] + (threadIdx.x >> 5) * slot_warp_bytes<W, T>(a.op, a.log_group, plain));
+    uint32_t *term = reinterpret_cast<uint32_t *>(&ws + 1);
+    uint16_t *coef = reinterpret_cast<uint16_t *>(term + slot_list_terms(a.op, a.log_group));
     {
         const int nm = fact ? a.g.n_cos : a.g.n_perm;
         const W *gm;
@@ -207,8 +236,6 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
     const W full = (W)a.g.full;
     const int lane = threadIdx.x & 31;
     const bool real_op = a.op.real != 0;
-    const bool uniform = a.op.uniform != 0;
-    const bool plain = !kTrack && uniform;  // no coefficients at all
     const uint64_t keep = policy_keep();
     const uint32_t mat0 = sm_fam[0].mat, delta0 = sm_fam[0].delta;  // operators of one family
 
@@ -300,7 +327,7 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
                 W bits = config_mask(r, rot_down(r, (int)fm.delta, n, full), (W)fm.mask, cc);
                 const uint32_t code = (uint32_t)my << 6 | (uint32_t)it << 10;
                 while (bits) {
-                    ws.term[k++] = code | (uint32_t)lowest_bit(bits);
+                    term[k++] = code | (uint32_t)lowest_bit(bits);
                     bits &= bits - 1;
                 }
             }
@@ -315,7 +342,7 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
             const SlotKey key_p = key;
             const uint32_t bucket_p = bucket, pilot_p = pilot;
             if (t < total) {
-                const uint32_t code = ws.term[t];
+                const uint32_t code = term[t];
                 uint32_t mat = mat0, delta = delta0;
                 if (n_items > 2) {
                     mat = sm_fam[code >> 11].mat;
@@ -343,14 +370,14 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
                     rep_search<W, kTrack>(s, sm_masks, a.g.n_perm, flip, full, best, gbest);
                 }
                 if (!plain)
-                    ws.coef[t] = (uint16_t)((uniform ? 0u : (mat * 2 + ((code >> 10) & 1u)) * (uint32_t)a.order) +
+                    coef[t] = (uint16_t)((uniform ? 0u : (mat * 2 + ((code >> 10) & 1u)) * (uint32_t)a.order) +
                                             (uint32_t)gbest);
                 key = slot_key((uint64_t)best);
                 bucket = slot_bucket((uint64_t)best, key, sd.v);
                 pilot = load_pilot(sd.v.pilots + bucket, keep);
             }
             if (base && t - 32 < total)
-                ws.term[t - 32] = slot_finish(key_p, bucket_p, pilot_p, sd.v);
+                term[t - 32] = slot_finish(key_p, bucket_p, pilot_p, sd.v);
         }
         __syncwarp();
 
@@ -383,12 +410,12 @@ __global__ void __launch_bounds__(kSlThreads, sizeof(W) == 4 ? 6 : 5) k_matvec_s
                     for (int u = 0; u < 4; ++u) {
                         const uint32_t q = k + u * split;
                         if (q < k1) {
-                            const T *from = xs + (uint64_t)ws.term[q] * (uint32_t)a.stride;
+                            const T *from = xs + (uint64_t)term[q] * (uint32_t)a.stride;
                             if (a.beyond_l2)
                                 load_random<sizeof(Vec)>(&v[u], from);
                             else
                                 v[u] = *reinterpret_cast<const Vec *>(from);
-                            ci[u] = plain ? 0u : ws.coef[q];
+                            ci[u] = plain ? 0u : coef[q];
                         } else {
                             ci[u] = 0;
 #pragma unroll
@@ -481,9 +508,10 @@ template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int
 cudaError_t slot_launch(const SlotArgs<kSec> &a, cudaStream_t stream)
 {
     auto kern = k_matvec_slot<W, T, kC, kTrack, kSearch, EL, kSec>;
+    const bool plain = !kTrack && a.op.uniform;
     const size_t smem = kSearch > 0 || a.g.fact
-                            ? slot_smem_bytes<W, T, true>(a.g, a.op, a.order, a.max_order, kSec > 1)
-                            : slot_smem_bytes<W, T, false>(a.g, a.op, a.order, a.max_order, kSec > 1);
+                            ? slot_smem_bytes<W, T, true>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain)
+                            : slot_smem_bytes<W, T, false>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain);
     int sms = 0, per_sm = 0;
     const cudaError_t e = kernel_occupancy((const void *)kern, kSlThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
