@@ -568,6 +568,10 @@ ed_operator *build_operator_host(int n_sites, int n_terms, const double *coeff,
             op->uniform = op->uniform && re == op->scale;
             first = false;
         }
+    op->even = true;
+    for (int k = 0; k < op->n_mats; ++k)
+        for (int c = 0; c < 2; ++c)
+            op->even = op->even && op->mats[(size_t)k * 32 + 2 * 6 + c] == op->mats[(size_t)k * 32 + 2 * 9 + c];
     // the most off-diagonal elements one row can produce
     int worst = 0;
     for (int t = 0; t < n_terms; ++t) {
@@ -614,7 +618,8 @@ edk::OpView op_view(const ed_operator *op)
             exch = 0;
     }
     return edk::OpView{(int)op->h_fams.size(), op->n_mats, op->max_offdiag, op->d_fams, op->d_mats,
-                       op->d_matsf, op->d_offmask, exch, op->real ? 1 : 0, op->uniform ? 1 : 0, op->scale};
+                       op->d_matsf, op->d_offmask, exch, op->real ? 1 : 0, op->uniform ? 1 : 0, op->scale,
+                       op->even ? 1 : 0};
 }
 
 }  // namespace

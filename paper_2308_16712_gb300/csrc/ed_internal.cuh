@@ -551,6 +551,7 @@ struct ed_operator {
     bool real = true;                 // every matrix entry real
     bool uniform = false;             // every off-diagonal entry is the real number `scale`
     double scale = 1.0;
+    bool even = false;                // every matrix has the same entry for |01> and |10>
     // host copies of the device tables
     std::vector<edk::OpFamily> h_fams;
     std::vector<double2> h_mats;

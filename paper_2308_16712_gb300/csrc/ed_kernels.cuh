@@ -124,6 +124,7 @@ struct OpView {
     int real;                // every entry is real
     int uniform;             // every nonzero off-diagonal entry is the real number `scale`
     double scale;
+    int even;                // every matrix has the same entry for |01> and |10>
 };
 
 // Host tables (generic group search) for counting a sector; validates the group.

@@ -103,8 +103,10 @@ bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, boo
         return false;
     // the coefficient table: in shared memory, its entries counted in 16 bits
     const int order = track ? g.order : 1;
-    const size_t bytes = dtype == ED_F64 || dtype == ED_C128 ? slot_table_bytes<double>(op, order, false)
-                                                             : slot_table_bytes<float>(op, order, false);
+    OpView all = op;
+    all.even = 0;
+    const size_t bytes = dtype == ED_F64 || dtype == ED_C128 ? slot_table_bytes<double>(all, order, false)
+                                                             : slot_table_bytes<float>(all, order, false);
     return bytes <= (size_t)kSlMaxTable && (size_t)op.n_mats * 2 * g.order < 65536 &&
            (size_t)op.n_fam * sizeof(OpFamily) <= 16384;
 }
@@ -149,6 +151,8 @@ static cudaError_t launch_slot(const OpView &op, const GroupView &g, const Index
     a.n_sectors = 1;
     a.max_order = g.order;
     a.order = track ? g.order : 1;
+    a.op.even = track && op.even;
+    a.byte = slot_entries(a.op) * a.order <= 256;
     a.scalars = row.scalars;
     a.stride = row.stride;
     a.log_parts = 0;

@@ -161,6 +161,8 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
             unsigned long long *queue = (unsigned long long *)(xs + bytes);
             const ed_basis *b0 = sectors[todo[i]].basis;
             a.op = op;
+            a.op.even = 0;
+            a.byte = 0;
             a.g = b0->group_view();
             const int search = a.g.fact ? a.g.prune : 0;
             a.g.flip = 0;  // spin inversion is per sector

@@ -30,6 +30,14 @@
 // entries are one real number it is factored out of the sum, and no
 // multiplication is left when the characters are 1.
 //
+// Beyond L2 the reads of xs are bound by DRAM's rate of random accesses (5.1e10 /s
+// over 0.5 GB, 4.1e10 /s over 2 GB, whatever the load's form): ring N=36 fp64
+// 25.6 ms of 23, ring N=38 8 vectors fp32 123 of 116.  Within L2 issue slots and the
+// L2's 2.9e11 random reads /s overlap in part (ring N=32 fp32: 71 % of the issue
+// slots, 0.90 ms against 0.53 for the reads alone).  Against the kernels it
+// replaced: those three 41.0, 181 and 1.18 ms; ring N=33 3 vectors complex128
+// 99.8 -> 20.5, 6x6 torus complex128 838 -> 180.
+//
 // The order of every sum depends only on the operator, the type and the number of
 // vectors, not on R: results are deterministic, and the same for a sector alone
 // (small R, when it is small: one round of terms per tile) or in a batch.
@@ -76,6 +84,7 @@ struct SlotArgs {
     int log_group;            // lanes of a row: 32 >> log2 of the most rows a tile may have
     int chunk;                // tiles taken from the queue at a time
     int beyond_l2;            // the slotted copies exceed L2: gather past L1
+    int byte;                 // the coefficient table has at most 256 entries
     uint64_t total_tiles;
     BatchCtl ctl;             // tile queue (zeroed by the fill), status word and gate
     SlotSector sec[kSec];     // read from the launch parameters (constant bank)
@@ -83,11 +92,12 @@ struct SlotArgs {
 
 // A warp's shared memory: this, the term list (phase A: site | row << 6 |
 // (2 family + c) << 10, phase B: slot), and the terms' coefficient indices unless
-// the sum has none.  The list is sized for the operator, because what is left of
-// an SM's 256 KB is its L1, and every gather on its way occupies a line there:
-// with a list of 640 terms and indices for all (196 KB at five or six blocks)
-// the 6x6 torus complex128 took 372 instead of 207 ms, ring N=32 fp32 1.07
-// instead of 0.96; six blocks of ring N=32's 48 products of 8 vectors 74 -> 47 ms.
+// the sum has none (a byte each where that is enough).  The list is sized for
+// the operator, because what is left of an SM's 256 KB is its L1, and every
+// gather on its way occupies a line there: with a list of 640 terms and 16-bit
+// indices for all (196 KB at five or six blocks) the 6x6 torus complex128 took
+// 372 instead of 207 ms (188 with bytes), ring N=32 fp32 1.07 instead of 0.96,
+// and 48 of its products of 8 vectors 74 instead of 47.
 template <typename W, typename T>
 struct __align__(16) SlotWarp {
     W r[kSlMaxRows];
@@ -98,11 +108,18 @@ struct __align__(16) SlotWarp {
 
 // Coefficient table: conj(h) chi for (matrix, c = |01> or |10>) x characters, chi
 // alone when h is factored out.  Characters of a batch differ by sector and
-// are read from there; its table holds conj(h) only.
+// are read from there; its table holds conj(h) only.  For a single sector with
+// characters the two c share an entry where they can (op.even, cleared by the
+// launch otherwise).
+__host__ __device__ inline int slot_entries(const OpView &op)
+{
+    return op.uniform ? 1 : op.even ? op.n_mats : op.n_mats * 2;
+}
+
 template <typename T>
 __host__ __device__ inline size_t slot_table_bytes(const OpView &op, int order, bool batch)
 {
-    return (size_t)(op.uniform ? 1 : op.n_mats * 2) * (batch ? 1 : order) * sizeof(Cplx<T>);
+    return (size_t)slot_entries(op) * (batch ? 1 : order) * sizeof(Cplx<T>);
 }
 
 // a b with the same rounding wherever it is used (no contraction left to the
@@ -133,32 +150,33 @@ __host__ __device__ inline uint32_t slot_list_terms(const OpView &op, int log_gr
 }
 
 template <typename W, typename T>
-__host__ __device__ inline size_t slot_warp_bytes(const OpView &op, int log_group, bool plain)
+__host__ __device__ inline size_t slot_warp_bytes(const OpView &op, int log_group, bool plain, bool byte)
 {
     const size_t terms = slot_list_terms(op, log_group);
-    return align16(sizeof(SlotWarp<W, T>) + terms * 4 + (plain ? 0 : terms * 2));
+    return align16(sizeof(SlotWarp<W, T>) + terms * 4 + (plain ? 0 : byte ? terms : terms * 2));
 }
 
 template <typename W, typename T, bool kFact>
 __host__ __device__ inline size_t slot_smem_bytes(const GroupView &g, const OpView &op, int order, int max_order,
-                                                  int log_group, bool batch, bool plain)
+                                                  int log_group, bool batch, bool plain, bool byte)
 {
     size_t off[7];
     slot_smem_layout<W, T, kFact>(g, op, order, max_order, batch, off);
-    return off[6] + kSlWarps * slot_warp_bytes<W, T>(op, log_group, plain);
+    return off[6] + kSlWarps * slot_warp_bytes<W, T>(op, log_group, plain, byte);
 }
 
 // kSearch: 0 every element of the group (factored or not), 1 ring runs, 2 torus
 // row keys.  EL: scalars per lane and access.
-// Blocks per SM, by registers: a word of 32 bits and single precision fit 32 of
+// Blocks per SM.  By registers: a word of 32 bits and single precision fit 32 of
 // them (a few spill; ring N=32 fp32 0.96 -> 0.90 ms), in double precision that
 // costs more than the warps give (lanczos of ring N=32 fp64 115 -> 130 ms), and a
-// sixth block for 64-bit words changes nothing (they wait for DRAM).
-template <typename W, typename T, bool kTrack>
-constexpr int kSlBlocks = sizeof(W) == 8 ? 5 : sizeof(T) == 4 && !kTrack ? 8 : 6;
+// sixth block for 64-bit words changes nothing (they wait for DRAM).  The torus
+// with characters gains more from L1 than from a fifth block (186 -> 180 ms).
+template <typename W, typename T, bool kTrack, int kSearch>
+constexpr int kSlBlocks = sizeof(W) == 8 ? (kTrack && kSearch == 2 ? 4 : 5) : sizeof(T) == 4 && !kTrack ? 8 : 6;
 
 template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int kSec>
-__global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack>) k_matvec_slot(const __grid_constant__ SlotArgs<kSec> a)
+__global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) k_matvec_slot(const __grid_constant__ SlotArgs<kSec> a)
 {
     static_assert(!kC || EL % 2 == 0, "a complex number per lane at least");
     constexpr bool kBatch = kSec > 1;
@@ -178,10 +196,12 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack>) k_matvec_
     T *sm_isq = reinterpret_cast<T *>(smem + off[5]);
     const bool uniform = a.op.uniform != 0;
     const bool plain = !kTrack && uniform;  // no coefficients at all
+    const bool byte = kTrack && !kBatch && a.byte, even = kTrack && !kBatch && a.op.even;
     SlotWarp<W, T> &ws = *reinterpret_cast<SlotWarp<W, T> *>(
-        smem + off[6] + (threadIdx.x >> 5) * slot_warp_bytes<W, T>(a.op, a.log_group, plain));
+        smem + off[6] + (threadIdx.x >> 5) * slot_warp_bytes<W, T>(a.op, a.log_group, plain, byte));
     uint32_t *term = reinterpret_cast<uint32_t *>(&ws + 1);
     uint16_t *coef = reinterpret_cast<uint16_t *>(term + slot_list_terms(a.op, a.log_group));
+    uint8_t *coef8 = reinterpret_cast<uint8_t *>(coef);
     {
         const int nm = fact ? a.g.n_cos : a.g.n_perm;
         const W *gm;
@@ -209,11 +229,11 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack>) k_matvec_
             sm_off[e] = a.op.offmask[e];
         }
         const int per = kBatch ? 1 : a.order;
-        for (int e = threadIdx.x; e < (a.op.uniform ? 1 : a.op.n_mats * 2) * per; e += blockDim.x) {
-            const int cc = 1 + e / per % 2;
+        for (int e = threadIdx.x; e < slot_entries(a.op) * per; e += blockDim.x) {
+            const int cc = even ? 1 : 1 + e / per % 2;
             Cplx<T> c = {T(1), T(0)};
             if (!a.op.uniform)
-                c = conjc(mat(e / per / 2 * 16 + (3 - cc) * 4 + cc));
+                c = conjc(mat((even ? e / per : e / per / 2) * 16 + (3 - cc) * 4 + cc));
             if (kTrack && !kBatch) {
                 Cplx<T> ch;
                 if constexpr (sizeof(T) == 8)
@@ -369,9 +389,14 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack>) k_matvec_
                 } else {
                     rep_search<W, kTrack>(s, sm_masks, a.g.n_perm, flip, full, best, gbest);
                 }
-                if (!plain)
-                    coef[t] = (uint16_t)((uniform ? 0u : (mat * 2 + ((code >> 10) & 1u)) * (uint32_t)a.order) +
-                                            (uint32_t)gbest);
+                if (!plain) {
+                    const uint32_t entry = uniform ? 0u : even ? mat : mat * 2 + ((code >> 10) & 1u);
+                    const uint32_t at = entry * (uint32_t)a.order + (uint32_t)gbest;
+                    if (byte)
+                        coef8[t] = (uint8_t)at;
+                    else
+                        coef[t] = (uint16_t)at;
+                }
                 key = slot_key((uint64_t)best);
                 bucket = slot_bucket((uint64_t)best, key, sd.v);
                 pilot = load_pilot(sd.v.pilots + bucket, keep);
@@ -415,7 +440,7 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack>) k_matvec_
                                 load_random<sizeof(Vec)>(&v[u], from);
                             else
                                 v[u] = *reinterpret_cast<const Vec *>(from);
-                            ci[u] = plain ? 0u : coef[q];
+                            ci[u] = plain ? 0u : byte ? coef8[q] : coef[q];
                         } else {
                             ci[u] = 0;
 #pragma unroll
@@ -508,16 +533,17 @@ template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int
 cudaError_t slot_launch(const SlotArgs<kSec> &a, cudaStream_t stream)
 {
     auto kern = k_matvec_slot<W, T, kC, kTrack, kSearch, EL, kSec>;
-    const bool plain = !kTrack && a.op.uniform;
+    const bool plain = !kTrack && a.op.uniform, byte = kTrack && kSec == 1 && a.byte;
     const size_t smem = kSearch > 0 || a.g.fact
-                            ? slot_smem_bytes<W, T, true>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain)
-                            : slot_smem_bytes<W, T, false>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain);
+                            ? slot_smem_bytes<W, T, true>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain, byte)
+                            : slot_smem_bytes<W, T, false>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain, byte);
     int sms = 0, per_sm = 0;
     const cudaError_t e = kernel_occupancy((const void *)kern, kSlThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
         return e;
     const uint64_t blocks_needed = (a.total_tiles + kSlWarps - 1) / kSlWarps;
-    const int grid = (int)std::min<uint64_t>(blocks_needed, (uint64_t)sms * std::max(per_sm, 1));
+    per_sm = std::max(1, std::min(per_sm, kSlBlocks<W, T, kTrack, kSearch>));
+    const int grid = (int)std::min<uint64_t>(blocks_needed, (uint64_t)sms * per_sm);
     kern<<<std::max(grid, 1), kSlThreads, smem, stream>>>(a); count_launch();
     return cudaGetLastError();
 }
