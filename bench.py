@@ -55,12 +55,13 @@ INT_LANES_PER_SM = 64
 # DRAM bytes (read + write) per stored nonzero of one launch of the timed
 # kernel (fp32 block product, keyed by kernel and nvec), from one ncu --set
 # full capture of the same kernel on the ring N=36 sector with 1 230 759 430
-# nonzeros (term-parallel, nvec = 8: 162.13 + 2.02 GB; row-per-lane: 161.04 +
-# 2.02 GB).  A ring N=40 launch is too large for a many-pass capture, so its
+# nonzeros (slot, nvec = 8: 121.49 + 2.02 GB; term-parallel: 162.13 + 2.02 GB;
+# row-per-lane: 161.04 + 2.02 GB).  A ring N=40 launch is too large for a many-pass capture, so its
 # traffic is this figure times the nonzeros it processes.  Retake the capture
 # and update the figure whenever the kernel changes (the roofline reports null
 # traffic for kernels not listed).
-KERNEL_DRAM_BYTES_PER_NNZ = {("term-parallel", 8): (162.133806e9 + 2.022193e9) / 1230759430,
+KERNEL_DRAM_BYTES_PER_NNZ = {("slot", 8): (121.490340e9 + 2.021443e9) / 1230759430,
+                             ("term-parallel", 8): (162.133806e9 + 2.022193e9) / 1230759430,
                              ("row-per-lane", 8): (161.040283e9 + 2.023800e9) / 1230759430}
 
 
@@ -761,10 +762,12 @@ def run_job(args, w):
     pk, pk_kind = peaks()
     hbm_peak = pk.get("hbm_gbs", 6800.0)
     alg_bytes = dim * (8 + 2 + 2 * 4 * nvec) + terms * (4 * nvec + 2)  # keys, norms, x_r, y_r; x_j, n(r')
-    sector_bytes = dim * (8 + 2 * 4 * nvec) + terms * (32 + max(32, 4 * nvec))  # bucket + x row per term
+    kern_kind = {1: "row-per-lane", 2: "term-parallel"}.get(
+        tuning.get("kernel"), "slot" if ed.basis_slots(B)[0] else "term-parallel")
+    slot = kern_kind == "slot"  # x row per term, bucket too without slots
+    sector_bytes = dim * (8 + 2 * 4 * nvec) + terms * ((0 if slot else 32) + max(32, 4 * nvec))
     t_s = prod_ms * 1e-3
     achieved_int = int_ops / t_s / 1e12
-    kern_kind = "row-per-lane" if tuning.get("kernel") == 1 else "term-parallel"
     roofline = {
         "bound": "alu", "achieved": achieved_int, "peak": int_peak / 1e12, "unit": "TOP/s",
         "frac": achieved_int / (int_peak / 1e12),
@@ -772,10 +775,11 @@ def run_job(args, w):
                     if (kern_kind, nvec) in KERNEL_DRAM_BYTES_PER_NNZ else None),
         "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the ring N=36 launch, "
                           "scaled by stored nonzeros",
-        "kernel": (("k_matvec (row-per-lane" if kern_kind == "row-per-lane" else "k_matvec_tp (term-parallel")
+        "kernel": ({"slot": "k_matvec_slot (slot", "row-per-lane": "k_matvec (row-per-lane",
+                    "term-parallel": "k_matvec_tp (term-parallel"}[kern_kind]
                    + f", fp32, nvec={nvec}, "
                    + ("pruned rotation search" if tuning.get("search") != 0 else "search over every rotation")
-                   + ", 64-bit words, bucketed index)"),
+                   + ", 64-bit words, " + ("slot index)" if slot else "bucketed index)")),
         "peak_kind": "measured live: int32 op mix of the search (funnel shift, lop3, min, add) on every SM",
         "int_ops_per_launch": int_ops, "int_ops_per_term": ops_term,
         "run_length_iterations_per_term": run_iters, "candidate_tops_per_term_and_coset": cands,
@@ -788,7 +792,8 @@ def run_job(args, w):
     buf.fill_(1)
     gather_peak, _ = ed.peak("gather32", buf)
     del buf
-    accesses = terms * 2 + dim  # one bucket and one x row per term, one key/x/y row per basis row
+    # one x row per term (and one bucket without slots), one key/x/y row per basis row
+    accesses = terms * (1 if slot else 2) + dim
     roofline["random_access"] = {"accesses_per_launch": accesses, "achieved_per_s": accesses / t_s,
                                  "peak_per_s": gather_peak, "frac": accesses / t_s / gather_peak,
                                  "peak_kind": "measured live: random 32-byte reads over 8 GiB"}
@@ -874,7 +879,7 @@ def run_job(args, w):
                 "d2h_bytes_per_step": 8 * nvec / args.steps,
                 "path": "pinned host start block -> device, ed_lanczos_block over the same steps, Ritz "
                         "values -> host"},
-        "autotune": {"product": tuning, "kernel_names": {"0": "library rule (term-parallel for fp32 blocks of 8)",
+        "autotune": {"product": tuning, "kernel_names": {"0": "library rule (slot kernel where the sector has a slot index)",
                                                           "1": "row-per-lane", "2": "term-parallel"},
                      "search_names": {"-1": "n/a", "0": "every rotation", "1": "pruned to the longest runs"}},
         "gpu_launches": launches,

@@ -123,7 +123,9 @@ ed_status ed_stream_status(void *stream);
  * norms) plus about 1 byte of prefix table, plus the index: about 18-36 bytes
  * for the bucketed index (sectors of 2^23 states or more; 32-byte buckets,
  * one per 1.8 states or fewer), else 10-20 bytes for the hash index and 8 for
- * packed (state, norm) keys.  Errors:
+ * packed (state, norm) keys, plus about 0.3 bytes for the slot index of the
+ * products (left out when the memory for building it, about 10 bytes per state,
+ * cannot be had).  Errors:
  * ED_ERR_INVALID_ARG, ED_ERR_NOT_A_GROUP, ED_ERR_BAD_CHARACTER, ED_ERR_OOM,
  * ED_ERR_CUDA, ED_ERR_INTERNAL.
  */
@@ -228,20 +230,25 @@ void ed_operator_destroy(ed_operator *op);
  *   dtype     ED_F64 / ED_F32 (real sectors only) or ED_C128 / ED_C64;
  *             the arithmetic is done in that precision
  *
- * Two kernels: rows handed to lanes (each lane walks its row's terms), and,
- * for nvec = 1 in single precision (and in double precision above 32 sites)
- * or an fp32 block of nvec = 8, with an operator whose off-diagonal entries
+ * Operators whose off-diagonal entries only exchange antiparallel spins are
+ * multiplied by the slot kernel: it places a copy of the vectors by a perfect
+ * hash of the basis and sums each row from a list of its terms.  The copy
+ * (some 1.2 dim rows of nvec numbers, padded to a power of two bytes up to 64 and
+ * to multiples of 32 beyond) comes from the library's memory pool in stream
+ * order.  Where it cannot be had, for other operators, and for nvec > 1 on fewer than 1024 states, two
+ * kernels: rows handed to lanes (each lane walks its row's terms), and, for
+ * nvec = 1 in single precision (and in double precision above 32 sites) or an fp32 block of nvec = 8, with an operator whose off-diagonal entries
  * only exchange antiparallel spins (|01> <-> |10>), a term-parallel
  * kernel (a warp lays a tile's terms out flat, one term per lane per round,
- * and sums each row with a segmented warp scan).  The two sum a row's terms in
+ * and sums each row with a segmented warp scan).  They sum a row's terms in
  * different orders, so a column of an nvec > 1 product may differ from the
  * nvec = 1 product in the last bits.  ed_autotune replaces this rule (and the
  * choice of representative search) by measured choices for sectors of the
  * same shape.  On a real block of 8 vectors the term-parallel kernel sums
  * every column in the order of its single-vector form.
  *
- * No allocation and no host synchronisation.  Deterministic: the same inputs
- * give bit-identical y.  Errors: ED_ERR_INVALID_ARG (including a complex
+ * No host synchronisation, no allocation but that copy.  Deterministic: the same
+ * inputs and the same kernel give bit-identical y.  Errors: ED_ERR_INVALID_ARG (including a complex
  * sector with a real dtype, or operator/basis with different n_sites),
  * ED_ERR_SYMMETRY_MISMATCH, ED_ERR_CUDA.
  */
@@ -256,12 +263,15 @@ typedef struct {
 } ed_sector;
 
 /*
- * ed_matvec_multi -- y_s = H x_s for up to 160 symmetry sectors in one
- * persistent launch (the matvec of Sec. "Matrix-vector product" applied to a
+ * ed_matvec_multi -- y_s = H x_s for up to 160 symmetry sectors in few
+ * persistent launches (the matvec of Sec. "Matrix-vector product" applied to a
  * batch of sectors of uneven dimension, so that no launch tail is paid per
- * sector).  The launch's warps take 32-row tiles from a device work queue (an
- * atomic counter over the tiles of all sectors, largest sectors first), the
- * role the paper's producer/consumer balancing plays across nodes.  Every basis must be built from the same n_sites and the same list
+ * sector).  A launch's warps take tiles of rows from a device work queue (an
+ * atomic counter over the tiles of its sectors, largest sectors first), the
+ * role the paper's producer/consumer balancing plays across nodes.  Sectors that
+ * go through the slot kernel (ed_matvec) are grouped so that the copies of a launch
+ * take at most 96 MB together, or one sector's; the others share one launch.
+ * Every basis must be built from the same n_sites and the same list
  * of lattice permutations (characters, spin inversion and n_up may differ);
  * dtype must be complex if any sector is.  Sectors with dimension 0 are
  * skipped.  Results equal those of ed_matvec on each sector, bit for bit.
@@ -269,7 +279,7 @@ typedef struct {
  *   sectors   host array of n_sectors entries
  *   nvec, dtype, stream   as ed_matvec
  *
- * No allocation; no host synchronisation.  Errors: ED_ERR_INVALID_ARG (also
+ * No allocation but those copies; no host synchronisation.  Errors: ED_ERR_INVALID_ARG (also
  * for sectors with different permutations), ED_ERR_SYMMETRY_MISMATCH,
  * ED_ERR_CUDA.
  */
