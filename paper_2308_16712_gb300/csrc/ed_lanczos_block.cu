@@ -11,7 +11,8 @@
 //   W = V_{j+1} B_{j+1}                 (Cholesky QR, twice)
 // so that H V_j = V_{j-1} B_j^T + V_j A_j + V_{j+1} B_{j+1} and the projected
 // matrix T is block tridiagonal with bandwidth p.  Its lowest eigenpairs come
-// from Sturm counts of a banded LDL^T factorisation (bisection, one warp) and
+// from Sturm counts of a banded LDL^T factorisation (multisection, its points
+// spread over the SMs; ring N=32, 8 vectors, 48 steps: 15.1 -> 2.8 ms) and
 // banded inverse iteration; the Ritz vector from a second, bit-identical pass;
 // the energy from a short fp64 single-vector Lanczos refinement of it
 // (ed_lanczos), as in the single-vector fp32-matvec mode.
@@ -711,7 +712,7 @@ __device__ bool chol_upper(const double *G, double *R, double *Ri, double *w)
 // coupling to the next block; for j < 0 (the start block) nothing is stored).
 // A failed Cholesky stops the recurrence: *stop = 1, *m_eff = j + 1 blocks.
 // Latency-bound (square roots and divisions of one chain): spreading the rest
-// over the warp took a step from 30 to 12 us at P = 8.
+// over the warp took a step from 30 to 9 us at P = 8.
 template <int P>
 __global__ void __launch_bounds__(32) k_bl_small(double *sm, double *A, double *B, int j, int which, int *stop,
                                                  int *m_eff)

@@ -5,8 +5,8 @@ namespace edk {
 
 int g_kernel_policy = 0;
 
-// The library's kernel rule for one vector of an exchange-only operator: the
-// term-parallel kernel in single precision, and in double precision for
+// The rule where the slot kernel does not run (launch_matvec_v), for one vector of
+// an exchange-only operator: the term-parallel kernel in single precision, and in double precision for
 // 64-bit words (ring N=36 / 40 fp64: 42.5 / 714 ms against 45.1 / 750 ms
 // row-per-lane); row-per-lane otherwise.
 bool use_term_parallel(int nvec, const OpView &op, ed_dtype dtype, int n_sites)

@@ -26,7 +26,7 @@ CtlWords g_ctl[kCtlDevices];
 bool g_inject_stall = false;
 // One batch's slotted copies: what stays in L2 between the fill and the product.
 constexpr size_t kSlotBatchBytes = 96ull << 20;
-// 0 and 1: one batched launch (measured faster than per-sector launches on
+// Sectors without a slot index.  0 and 1: one batched launch (measured faster than per-sector launches on
 // all 140 XXZ N=28 sectors, also for single vectors in single precision:
 // 51.7 against 54.4 ms); 2: one launch per sector where the term-parallel
 // kernel applies (test hook)

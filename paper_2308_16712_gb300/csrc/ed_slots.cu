@@ -75,6 +75,7 @@ struct SlotBuild {
 // depends on timing; the slots of the keys are distinct in any case, and
 // results do not depend on which slot a value lies in.
 // Bound by shared-memory latency (a dozen probes per bucket); two blocks per SM.
+// Ring N=36 (6.3e7 states): 9.9 ms.
 __global__ void __launch_bounds__(kSlotThreads) k_slot_pilots(const uint2 *list, const uint32_t *cursor,
                                                               const uint32_t *part_cell, const uint2 *cells,
                                                               uint8_t *pilots, uint2 *exc,
