@@ -1134,7 +1134,10 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     int *stop = flags;
     const int yk = f32 ? 0 : 1;
     MatvecVariant tuned = tuned_variant(b, P, f32 ? ED_F32 : ED_F64);
-    if (iv.slots.pilots) {  // scratch of the slot kernel, kept for the whole call where half of what is left has room
+    // scratch of the slot kernel, kept for the whole call where half of what is left
+    // has room; without it the other kernels take every product, so that the
+    // second pass repeats the first one's bits
+    if (iv.slots.pilots) {
         const size_t want = slot_scratch_bytes(iv.slots, P, f32 ? ED_F32 : ED_F64);
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
@@ -1143,6 +1146,8 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
             S.ptrs.push_back(ws);
             tuned.scratch = ws;
             tuned.scratch_bytes = want;
+        } else if (tuned.kernel == 0) {
+            tuned.kernel = 4;
         }
         (void)cudaGetLastError();
     }
