@@ -877,7 +877,8 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     uint64_t *d_offsets = nullptr, *d_tmp = nullptr, *d_binom = nullptr;
     uint8_t *d_inv = nullptr;
     int *d_flag = nullptr;  // [0] not ascending, largest bucket of [1] the prefix table, [2] the hash index, [3] slots failed
-    TableImage tables;
+    TableImage tables;  // this and slot_cells outlive their copies: every way out waits for the stream
+    std::vector<uint2> slot_cells;
     tables.add(&b->d_masks32, m32.data(), m32.size());
     tables.add(&b->d_masks64, m64.data(), m64.size());
     tables.add(&b->d_chi, chi.data(), chi.size());
@@ -1084,7 +1085,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         if (ok && n_ghost)
             ok = cudaMemcpyAsync(list, d_ghosts, n_ghost * sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream) ==
                  cudaSuccess;
-        ok = ok && edk::build_slot_index(b, list, n_ghost, d_flag + 3, stream);
+        ok = ok && edk::build_slot_index(b, list, n_ghost, d_flag + 3, slot_cells, stream);
         if (!ok) {
             (void)cudaGetLastError();
             edk::ws_free(list, stream);

@@ -166,7 +166,8 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
 // ---- slot index (ed_slots.cu) and the product over it (ed_matvec_slot.cuh) --------
 // Sectors of at least this many states get a slot index (test hook: any size).
 uint64_t slot_min_dim();
-bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, cudaStream_t stream);
+bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, std::vector<uint2> &cells,
+                      cudaStream_t stream);
 void free_slot_index(ed_basis *b);
 // Layout of a row of the slotted copy: scalars of a row, scalars per access, row stride.
 struct SlotRow {

@@ -384,6 +384,11 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         }
     }
     sec_blk[ns] = (int)blk_sec.size();
+    uint64_t *d_off = nullptr;
+    struct Wait {  // the tables above outlive their asynchronous copies on every way out
+        cudaStream_t st;
+        ~Wait() { cudaStreamSynchronize(st); }
+    } wait{st};
     const unsigned nblk = (unsigned)blk_sec.size();
     const int stride = std::max(steps, kRefine) + 2;
     const size_t sc = (size_t)ns * stride;
@@ -409,7 +414,6 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
     bool fused = true;
     for (int k = 0; k < ns; ++k)
         fused = fused && sectors[k].basis->dim <= kFusedMax;
-    uint64_t *d_off = nullptr;
     LM_TRY(O.get(&d_off, ns + 1));
     LM_TRY(cudaMemcpyAsync(d_off, off.data(), (ns + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
     D *x0, *ring0, *ring1, *w, *psi;

@@ -359,8 +359,12 @@ cudaError_t launch_slot_fill(const SlotFill *sec, int n, int nvec, ed_dtype dtyp
 // representatives (ghosts: ownership passes to the basis on success).  False,
 // with nothing kept, when memory is short or the slots exceed 32 bits; *err
 // (device, zero) becomes 1 when no pilots were found: the caller then takes the
-// index back.  The products then use the other index kinds.
-bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, cudaStream_t stream)
+// index back.  The products then use the other index kinds.  cells: the caller's,
+// to be kept until the stream has been waited for, whatever the outcome: its
+// copy to the device is asynchronous, and from pageable memory CUDA does not
+// promise that the call has read the source when it returns.
+bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, std::vector<uint2> &cells,
+                      cudaStream_t stream)
 {
     if (!b->dim)
         return false;
@@ -402,7 +406,7 @@ bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err,
         (void)cudaGetLastError();
         return false;
     }
-    std::vector<uint2> cells(v.n_cells);
+    cells.resize(v.n_cells);
     uint64_t parts = 0;
     const uint32_t part_keys = b->dim + n_ghost <= kSlotSmallMax ? kSlotSmallKeys : kSlotPartKeys;
     for (uint32_t c = 0; c < v.n_cells; ++c) {
