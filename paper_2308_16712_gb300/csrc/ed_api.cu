@@ -987,28 +987,40 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         void *d_work = nullptr;
         uint32_t n_seg = 0;
         uint64_t total = 0;
-        cudaError_t pe = edk::ws_alloc(&d_work, edk::prefix_filter_bytes(bits), stream);
-        if (pe == cudaSuccess)
-            pe = edk::ws_alloc((void **)&d_prefix, ((1ULL << bits) + 1) * sizeof(uint32_t), stream);
-        if (pe == cudaSuccess)
-            pe = edk::ws_alloc((void **)&d_start, ((1ULL << bits) + 1) * sizeof(uint64_t), stream);
-        if (pe == cudaSuccess)
+        // some 130 MB of work memory at 22 bits; without it every state is visited
+        const bool room =
+            edk::ws_alloc_optional(&d_work, edk::prefix_filter_bytes(bits), stream) == cudaSuccess &&
+            edk::ws_alloc_optional((void **)&d_prefix, ((1ULL << bits) + 1) * sizeof(uint32_t), stream) ==
+                cudaSuccess &&
+            edk::ws_alloc_optional((void **)&d_start, ((1ULL << bits) + 1) * sizeof(uint64_t), stream) ==
+                cudaSuccess;
+        cudaError_t pe = cudaSuccess;
+        if (room) {
             pe = edk::launch_prefix_filter(n_sites, n_up, odd, bits, d_inv, n_elems, spin_inversion != 0, d_binom,
                                            d_work, d_prefix, d_start, d_prefix + (1ULL << bits), stream);
-        if (pe == cudaSuccess)
-            pe = cudaMemcpyAsync(&n_seg, d_prefix + (1ULL << bits), sizeof(n_seg), cudaMemcpyDeviceToHost, stream);
-        if (pe == cudaSuccess)
-            pe = cudaMemcpyAsync(&total, d_start + (1ULL << bits), sizeof(total), cudaMemcpyDeviceToHost, stream);
-        if (pe == cudaSuccess)
-            pe = cudaStreamSynchronize(stream);
+            if (pe == cudaSuccess)
+                pe = cudaMemcpyAsync(&n_seg, d_prefix + (1ULL << bits), sizeof(n_seg), cudaMemcpyDeviceToHost,
+                                     stream);
+            if (pe == cudaSuccess)
+                pe = cudaMemcpyAsync(&total, d_start + (1ULL << bits), sizeof(total), cudaMemcpyDeviceToHost, stream);
+            if (pe == cudaSuccess)
+                pe = cudaStreamSynchronize(stream);
+        }
         edk::ws_free(d_work, stream);
         ED_B_TRY(pe);
-        plan.total = total;
-        plan.seg_prefix = d_prefix;
-        plan.seg_start = d_start;
-        plan.n_seg = n_seg;
-        plan.low_bits = n_sites - bits;
-        plan.odd = odd;
+        if (room) {
+            plan.total = total;
+            plan.seg_prefix = d_prefix;
+            plan.seg_start = d_start;
+            plan.n_seg = n_seg;
+            plan.low_bits = n_sites - bits;
+            plan.odd = odd;
+        } else {
+            edk::ws_free(d_prefix, stream);
+            edk::ws_free(d_start, stream);
+            d_prefix = nullptr;
+            d_start = nullptr;
+        }
     }
     const uint64_t threads = (uint64_t)sms * 2048 * 4;
     plan.chunk = std::max<uint64_t>(16, (plan.total + threads - 1) / threads);
@@ -1024,24 +1036,22 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
         cudaMemGetInfo(&free_b, &total_b);
         const uint64_t words = (plan.chunk + 31) / 32;
         const uint64_t bytes = plan.n_chunks * words * sizeof(uint32_t);
-        if (bytes <= free_b / 8 && edk::ws_alloc((void **)&d_flags, bytes, stream) == cudaSuccess) {
+        if (bytes <= free_b / 8 && edk::ws_alloc_optional((void **)&d_flags, bytes, stream) == cudaSuccess) {
             plan.flags = d_flags;
             plan.flag_words = (uint32_t)words;
         }
-        (void)cudaGetLastError();
     }
     if (!count_only) {
         // the weightless representatives, for the slot index: they are fixed by
         // some element, a vanishing share of all at the sizes where it is built
         const uint64_t cap = std::min<uint64_t>(1ULL << 24, states / b->order / 8 + 65536);
-        if (edk::ws_alloc((void **)&d_ghosts, cap * sizeof(uint64_t), stream) == cudaSuccess &&
-            edk::ws_alloc((void **)&d_ghost_n, sizeof(uint32_t), stream) == cudaSuccess) {
+        if (edk::ws_alloc_optional((void **)&d_ghosts, cap * sizeof(uint64_t), stream) == cudaSuccess &&
+            edk::ws_alloc_optional((void **)&d_ghost_n, sizeof(uint32_t), stream) == cudaSuccess) {
             plan.ghosts = d_ghosts;
             plan.ghost_count = d_ghost_n;
             plan.ghost_cap = (uint32_t)cap;
             ED_B_TRY(cudaMemsetAsync(d_ghost_n, 0, sizeof(uint32_t), stream));
         }
-        (void)cudaGetLastError();
     }
     ED_B_TRY(edk::launch_enum_count(plan, gv, d_counts, stream));
     ED_B_TRY(edk::launch_scan(d_counts, plan.n_chunks, d_offsets, d_tmp, stream));
@@ -1081,7 +1091,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
     if (plan.ghosts && dim >= edk::slot_min_dim() && n_ghost <= plan.ghost_cap) {
         // the list shrunk to its length, owned by the index
         uint64_t *list = nullptr;
-        bool ok = !n_ghost || edk::ws_alloc((void **)&list, n_ghost * sizeof(uint64_t), stream) == cudaSuccess;
+        bool ok = !n_ghost || edk::ws_alloc_optional((void **)&list, n_ghost * sizeof(uint64_t), stream) == cudaSuccess;
         if (ok && n_ghost)
             ok = cudaMemcpyAsync(list, d_ghosts, n_ghost * sizeof(uint64_t), cudaMemcpyDeviceToDevice, stream) ==
                  cudaSuccess;

@@ -10,6 +10,9 @@ namespace edk {
 // Library-owned, stream-ordered device memory (see ed_pool.cu): allocations
 // and frees are ordered on stream s; freed memory stays cached for later calls.
 cudaError_t ws_alloc(void **p, size_t bytes, cudaStream_t s);
+// The same for memory that the caller can do without: no error is left pending
+// and *p is null when it cannot be had.
+cudaError_t ws_alloc_optional(void **p, size_t bytes, cudaStream_t s);
 cudaError_t ws_free(void *p, cudaStream_t s);
 // Bytes the pool holds freed and ready for reuse (counted as free memory when
 // a solver decides whether its vectors fit).

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -62,6 +63,23 @@ cudaError_t ws_alloc(void **p, size_t bytes, cudaStream_t s)
     return cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 1), pool, s);
 }
 
+namespace {
+std::atomic<uint64_t> g_optional_limit{~0ull};
+}  // namespace
+
+cudaError_t ws_alloc_optional(void **p, size_t bytes, cudaStream_t s)
+{
+    *p = nullptr;
+    if (bytes > g_optional_limit.load(std::memory_order_relaxed))
+        return cudaErrorMemoryAllocation;
+    const cudaError_t e = ws_alloc(p, bytes, s);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        *p = nullptr;
+    }
+    return e;
+}
+
 cudaError_t ws_free(void *p, cudaStream_t s)
 {
     return p ? cudaFreeAsync(p, s) : cudaSuccess;
@@ -109,6 +127,13 @@ cudaError_t kernel_occupancy(const void *kern, int threads, size_t smem, int *sm
 }
 
 }  // namespace edk
+
+// Test hook: later requests for work memory that the library can do without are
+// refused above this many bytes, as if the device had none.
+extern "C" void edx_optional_memory(uint64_t bytes)
+{
+    edk::g_optional_limit.store(bytes, std::memory_order_relaxed);
+}
 
 extern "C" ed_status ed_release_cached_memory(void)
 {

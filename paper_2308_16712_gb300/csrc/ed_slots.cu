@@ -389,7 +389,7 @@ bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err,
         count.resize(v.n_cells);
         uint32_t *d_count = nullptr;
         if (e == cudaSuccess)
-            e = ws_alloc((void **)&d_count, v.n_cells * sizeof(uint32_t), stream);
+            e = ws_alloc_optional((void **)&d_count, v.n_cells * sizeof(uint32_t), stream);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(d_count, 0, v.n_cells * sizeof(uint32_t), stream);
         if (e == cudaSuccess) {
@@ -425,18 +425,18 @@ bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err,
     uint8_t *pilots = nullptr;
     uint2 *exc = nullptr, *list = nullptr, *d_cells = nullptr;
     uint32_t *cursor = nullptr;
-    e = ws_alloc((void **)&pilots, parts << kSlotLogB, stream);
+    e = ws_alloc_optional((void **)&pilots, parts << kSlotLogB, stream);
     if (e == cudaSuccess)
-        e = ws_alloc((void **)&exc, exc_n * sizeof(uint2), stream);
+        e = ws_alloc_optional((void **)&exc, exc_n * sizeof(uint2), stream);
     // cells, and behind them the cell of each partition (build only)
     cells.resize(v.n_cells + (parts + 1) / 2);
     std::memcpy(cells.data() + v.n_cells, part_cell.data(), parts * sizeof(uint32_t));
     if (e == cudaSuccess)
-        e = ws_alloc((void **)&d_cells, cells.size() * sizeof(uint2), stream);
+        e = ws_alloc_optional((void **)&d_cells, cells.size() * sizeof(uint2), stream);
     if (e == cudaSuccess)
-        e = ws_alloc((void **)&list, n_slots * sizeof(uint2), stream);
+        e = ws_alloc_optional((void **)&list, n_slots * sizeof(uint2), stream);
     if (e == cudaSuccess)
-        e = ws_alloc((void **)&cursor, parts * sizeof(uint32_t), stream);
+        e = ws_alloc_optional((void **)&cursor, parts * sizeof(uint32_t), stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_cells, cells.data(), cells.size() * sizeof(uint2), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)

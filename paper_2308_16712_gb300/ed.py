@@ -90,6 +90,7 @@ _SIGS = {
     "edx_peak": (_d, [_i32, _P, _u64, ctypes.POINTER(_d), _P]),
     "edx_basis_bucket": (_i32, [_P, ctypes.POINTER(_i32), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_slot_min_dim": (None, [_u64]),
+    "edx_optional_memory": (None, [_u64]),
     "edx_basis_slots": (_i32, [_P, ctypes.POINTER(_u64), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_count_nnz": (_i32, [_P, _P, ctypes.POINTER(ctypes.c_ulonglong)]),
     "edx_force_prefix_search": (None, [_i32]),
@@ -316,6 +317,13 @@ def index_policy(policy: str) -> None:
     index for large sectors), "hash" (always the hash index) or "bucket" (the
     bucketed index wherever its 64-bit entry can hold the key)."""
     _lib.edx_index_policy(INDEX_POLICIES[policy])
+
+
+def optional_memory(limit: int | None) -> None:
+    """Test hook: later requests for work memory that the library can do without
+    (the enumeration's filter and flags, the slot index, slotted copies) are
+    refused above ``limit`` bytes, as if the device had none; None: no limit."""
+    _lib.edx_optional_memory(2 ** 64 - 1 if limit is None else limit)
 
 
 def slot_min_dim(dim: int) -> None:
