@@ -235,8 +235,10 @@ void ed_operator_destroy(ed_operator *op);
  * hash of the basis and sums each row from a list of its terms.  The copy
  * (some 1.2 dim rows of nvec numbers, padded to a power of two bytes up to 64 and
  * to multiples of 32 beyond) comes from the library's memory pool in stream
- * order.  Where it cannot be had, for other operators, and for nvec > 1 on fewer than 1024 states, two
- * kernels: rows handed to lanes (each lane walks its row's terms), and, for
+ * order.  Where it cannot be had, and while the stream is being captured, the
+ * kernel reads x itself instead, which takes longer and gives the same bits.  For
+ * other operators, for bases without a slot index, and for nvec > 1 on fewer than
+ * 1024 states, two kernels: rows handed to lanes (each lane walks its row's terms), and, for
  * nvec = 1 in single precision (and in double precision above 32 sites) or an fp32 block of nvec = 8, with an operator whose off-diagonal entries
  * only exchange antiparallel spins (|01> <-> |10>), a term-parallel
  * kernel (a warp lays a tile's terms out flat, one term per lane per round,
@@ -247,8 +249,9 @@ void ed_operator_destroy(ed_operator *op);
  * same shape.  On a real block of 8 vectors the term-parallel kernel sums
  * every column in the order of its single-vector form.
  *
- * No host synchronisation, no allocation but that copy.  Deterministic: the same
- * inputs and the same kernel give bit-identical y.  Errors: ED_ERR_INVALID_ARG (including a complex
+ * No host synchronisation, no allocation but that copy (none during capture).
+ * Deterministic: the same inputs and the same kernel give bit-identical y,
+ * whatever memory is free.  Errors: ED_ERR_INVALID_ARG (including a complex
  * sector with a real dtype, or operator/basis with different n_sites),
  * ED_ERR_SYMMETRY_MISMATCH, ED_ERR_CUDA.
  */
@@ -270,7 +273,8 @@ typedef struct {
  * atomic counter over the tiles of its sectors, largest sectors first), the
  * role the paper's producer/consumer balancing plays across nodes.  Sectors that
  * go through the slot kernel (ed_matvec) are grouped so that the copies of a launch
- * take at most 96 MB together, or one sector's; the others share one launch.
+ * take at most 96 MB together, or one sector's (without copies, one group); the
+ * others share one launch.
  * Every basis must be built from the same n_sites and the same list
  * of lattice permutations (characters, spin inversion and n_up may differ);
  * dtype must be complex if any sector is.  Sectors with dimension 0 are
@@ -279,7 +283,7 @@ typedef struct {
  *   sectors   host array of n_sectors entries
  *   nvec, dtype, stream   as ed_matvec
  *
- * No allocation but those copies; no host synchronisation.  Errors: ED_ERR_INVALID_ARG (also
+ * No allocation but those copies (none during capture); no host synchronisation.  Errors: ED_ERR_INVALID_ARG (also
  * for sectors with different permutations), ED_ERR_SYMMETRY_MISMATCH,
  * ED_ERR_CUDA.
  */

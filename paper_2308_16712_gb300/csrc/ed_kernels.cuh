@@ -163,6 +163,7 @@ struct MatvecVariant {
     int prune = -1;
     void *scratch = nullptr;   // the caller's memory for the slotted copy of x, if any
     size_t scratch_bytes = 0;
+    bool alloc = true;         // the product may take that memory from the pool
 };
 cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, bool track, const void *x,
                             void *y, int nvec, ed_dtype dtype, MatvecVariant v, cudaStream_t stream);

@@ -742,9 +742,8 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
     ED_L_TRY(cudaMemsetAsync(beta, 0, (mmax + 2) * sizeof(double), st));
 
     // scratch of the slot kernel, for every product of the call where half of what
-    // is left has room, else for those of the main run.  Products without it keep
-    // to the other kernels: the second pass has to repeat the first one's bits,
-    // whatever memory is free by then.
+    // is left has room, else for those of the main run; products without it give
+    // the same bits from x itself
     void *slot_ws = nullptr;
     size_t slot_bytes = 0;
     for (const ed_dtype dt : {dt64, dt32}) {
@@ -752,11 +751,10 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
             break;
         const size_t want = slot_scratch_bytes(iv.slots, 1, dt);
         cudaMemGetInfo(&free_b, &total_b);
-        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc(&slot_ws, want, st) == cudaSuccess) {
+        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc_optional(&slot_ws, want, st) == cudaSuccess) {
             S.ptrs.push_back(slot_ws);
             slot_bytes = want;
         }
-        (void)cudaGetLastError();
     }
     auto variant = [&](ed_dtype dt) {
         MatvecVariant v = tuned_variant(b, 1, dt);
@@ -766,11 +764,11 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
         // the order of sums they always had, at 8 % more time (ring N=32).
         // So do those of reorthogonalised runs, whose time the vectors dominate
         // and whose end (a vanishing beta) is a matter of rounding, too.
-        if (v.kernel == 0 && (reorth || (dt == dt32 && n < kSlotMixedMinDim) ||
-                              (iv.slots.pilots && slot_scratch_bytes(iv.slots, 1, dt) > slot_bytes)))
+        if (v.kernel == 0 && (reorth || (dt == dt32 && n < kSlotMixedMinDim)))
             v.kernel = 4;
         v.scratch = slot_ws;
         v.scratch_bytes = slot_bytes;
+        v.alloc = false;
         return v;
     };
 

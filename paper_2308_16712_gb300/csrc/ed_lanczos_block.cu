@@ -1135,22 +1135,19 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     const int yk = f32 ? 0 : 1;
     MatvecVariant tuned = tuned_variant(b, P, f32 ? ED_F32 : ED_F64);
     // scratch of the slot kernel, kept for the whole call where half of what is left
-    // has room; without it the other kernels take every product, so that the
-    // second pass repeats the first one's bits
+    // has room; products without it give the same bits from x itself
     if (iv.slots.pilots) {
         const size_t want = slot_scratch_bytes(iv.slots, P, f32 ? ED_F32 : ED_F64);
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
         void *ws = nullptr;
-        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc(&ws, want, st) == cudaSuccess) {
+        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc_optional(&ws, want, st) == cudaSuccess) {
             S.ptrs.push_back(ws);
             tuned.scratch = ws;
             tuned.scratch_bytes = want;
-        } else if (tuned.kernel == 0) {
-            tuned.kernel = 4;
         }
-        (void)cudaGetLastError();
     }
+    tuned.alloc = false;
     const void *Yh = f32 ? (const void *)W32 : (const void *)W64;
     auto bh = [&](int k) { return Vh + (size_t)(reorth ? k : (k & 1)) * blk; };
     auto bl = [&](int k) { return Vl + (size_t)(reorth ? k : (k & 1)) * blk; };

@@ -486,27 +486,24 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         track = track || !sectors[k].basis->trivial_chars;
         max_order = std::max(max_order, sectors[k].basis->order);
     }
-    // scratch of the slot kernel (allocated here: products are captured); without
-    // it the other kernels serve every sector
+    // scratch of the slot kernel (allocated here: products are captured)
     void *scratch = nullptr;
     size_t scratch_bytes = slot_batch_bytes(sectors, ns, 1, C ? ED_C128 : ED_F64);
-    if (scratch_bytes && ws_alloc(&scratch, scratch_bytes, st) == cudaSuccess) {
+    if (scratch_bytes && ws_alloc_optional(&scratch, scratch_bytes, st) == cudaSuccess)
         O.ptrs.push_back(scratch);
-    } else {
-        (void)cudaGetLastError();
+    else
         scratch_bytes = 0;
-    }
     auto matvec = [&](const void *xin, void *yout, bool single, cudaStream_t s) -> cudaError_t {
         const size_t esize = single ? sizeof(F) : sizeof(D);
         std::vector<char> taken(ns, 0);
-        if (scratch_bytes) {
+        {
             std::vector<ed_sector> prod(sectors, sectors + ns);
             for (int k = 0; k < ns; ++k) {
                 prod[k].d_x = (const char *)xin + off[k] * esize;
                 prod[k].d_y = (char *)yout + off[k] * esize;
             }
             LM_CHK(launch_slot_batch(ov, prod.data(), ns, 1, single ? (C ? ED_C64 : ED_F32) : (C ? ED_C128 : ED_F64),
-                                     scratch, scratch_bytes, taken, s));
+                                     scratch, scratch_bytes, false, taken, s));
         }
         if (std::find(taken.begin(), taken.end(), 0) == taken.end())
             return cudaSuccess;

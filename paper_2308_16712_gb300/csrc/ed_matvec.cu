@@ -93,7 +93,7 @@ int slot_chunk(uint64_t tiles) { return (int)std::max<uint64_t>(1, std::min<uint
 
 bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, bool track, int nvec, ed_dtype dtype)
 {
-    if (!ix.slots.pilots || !op.exchange_only || op.max_terms > kSlTerms)
+    if (!ix.slots.pilots || !(ix.htab || ix.bkt) || !op.exchange_only || op.max_terms > kSlTerms)
         return false;
     if (g_kernel_policy != 0 && g_kernel_policy != 3)
         return false;
@@ -115,7 +115,11 @@ SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix
                        void *y, bool alone)
 {
     SlotSector d;
-    d.v = ix.slots;
+    if (xs)
+        d.v = ix.slots;
+    else
+        d.find = SlotFind{ix.htab, ix.hent, ix.bkt, ix.stash, ix.n_stash, ix.hbits, ix.hwide, ix.norm_bits,
+                          ix.bbits, ix.brem};
     d.states = ix.states;
     d.norms = ix.norms;
     d.chi = g.fact ? g.fchi : g.chi;
@@ -136,14 +140,28 @@ SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix
 
 uint64_t slot_tiles(const SlotSector &d) { return (d.dim + (1ull << d.log_rows) - 1) >> d.log_rows; }
 
+bool stream_captured(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// xs: the slotted copy with the tile queue behind it, or null (gather from x)
 static cudaError_t launch_slot(const OpView &op, const GroupView &g, const IndexView &ix, bool track, const void *x,
                                void *y, void *xs, int nvec, ed_dtype dtype, cudaStream_t stream)
 {
-    unsigned long long *queue = (unsigned long long *)((char *)xs + slot_copy_bytes(ix.slots, nvec, dtype));
-    const SlotFill fill{ix.slots, ix.states, ix.norms, ix.dim, x, xs};
-    cudaError_t e = launch_slot_fill(&fill, 1, nvec, dtype, queue, stream);
-    if (e != cudaSuccess)
-        return e;
+    unsigned long long *queue = nullptr;
+    if (xs) {
+        queue = (unsigned long long *)((char *)xs + slot_copy_bytes(ix.slots, nvec, dtype));
+        const SlotFill fill{ix.slots, ix.states, ix.norms, ix.dim, x, xs};
+        const cudaError_t e = launch_slot_fill(&fill, 1, nvec, dtype, queue, stream);
+        if (e != cudaSuccess)
+            return e;
+    }
     const SlotRow row = slot_row(nvec, dtype);
     SlotArgs<1> a;
     a.op = op;
@@ -165,6 +183,15 @@ static cudaError_t launch_slot(const OpView &op, const GroupView &g, const Index
     a.total_tiles = slot_tiles(a.sec[0]);
     a.chunk = slot_chunk(a.total_tiles);
     const int search = slot_search(g);
+    if (!xs) {
+        switch (dtype) {
+        case ED_F64: return slot1_direct_f64(a, track, row.el, stream);
+        case ED_F32: return slot1_direct_f32(a, track, row.el, stream);
+        case ED_C128: return slot1_direct_c128(a, track, row.el, stream);
+        case ED_C64: return slot1_direct_c64(a, track, row.el, stream);
+        }
+        return cudaErrorInvalidValue;
+    }
     switch (dtype) {
     case ED_F64: return slot1_f64(a, search, track, row.el, stream);
     case ED_F32: return slot1_f32(a, search, track, row.el, stream);
@@ -179,24 +206,18 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
 {
     if (v.prune >= 0 && g.fact && g.rot_d == 1)
         g.prune = v.prune;  // ring translations: pruned or exhaustive (autotuner)
-    // the slot kernel wherever the sector has a slot index and memory for the
-    // slotted copy can be had (ring N=32 fp32 / N=36 fp64 / 6x6 torus
-    // complex128: see ed_matvec_slot.cuh); else the kernels below
+    // the slot kernel wherever the sector has a slot index (ring N=32 fp32 / N=36
+    // fp64 / 6x6 torus complex128: see ed_matvec_slot.cuh), without the slotted
+    // copy where that cannot be had; else the kernels below
     if (v.kernel == 0 && slot_applies(op, g, ix, track, nvec, dtype)) {
         const size_t bytes = slot_scratch_bytes(ix.slots, nvec, dtype);
         void *xs = v.scratch_bytes >= bytes ? v.scratch : nullptr;
         void *own = nullptr;
-        if (!xs) {
-            if (ws_alloc(&own, bytes, stream) == cudaSuccess)
-                xs = own;
-            else
-                (void)cudaGetLastError();
-        }
-        if (xs) {
-            const cudaError_t e = launch_slot(op, g, ix, track, x, y, xs, nvec, dtype, stream);
-            const cudaError_t e2 = ws_free(own, stream);
-            return e != cudaSuccess ? e : e2;
-        }
+        if (!xs && v.alloc && !stream_captured(stream) && ws_alloc_optional(&own, bytes, stream) == cudaSuccess)
+            xs = own;
+        const cudaError_t e = launch_slot(op, g, ix, track, x, y, xs, nvec, dtype, stream);
+        const cudaError_t e2 = ws_free(own, stream);
+        return e != cudaSuccess ? e : e2;
     }
     // the term-parallel kernel: one vector (use_term_parallel), or a real
     // block of 8 vectors: by default in fp32 (ring N=32 / 36 / 40: 1.69 /

@@ -111,8 +111,10 @@ cudaError_t multi_c64(const MultiArgs &a, bool track, cudaStream_t s) { return m
 // differ, and a sector's result must not depend on its company).  The slotted
 // copies of a launch share one scratch area of at most kSlotBatchBytes (more
 // only for a single sector that needs it): filled right before they are read,
-// they are still in L2 where they fit.  `taken` marks the sectors done here;
-// the rest, also when no scratch memory can be had, are left to the caller.
+// they are still in L2 where they fit.  Where no scratch memory can be had (or
+// the launch is being captured) the sectors left share one launch without the
+// copies, with the same bits.  `taken` marks the sectors done here; those without
+// a slot index are left to the caller.
 static_assert(kSlotMaxBatch >= kMaxSectors, "a fill takes a whole batch");
 
 size_t slot_batch_bytes(const ed_sector *sectors, int n, int nvec, ed_dtype dtype)
@@ -127,7 +129,8 @@ size_t slot_batch_bytes(const ed_sector *sectors, int n, int nvec, ed_dtype dtyp
 }
 
 cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n, int nvec, ed_dtype dtype,
-                              void *scratch, size_t scratch_bytes, std::vector<char> &taken, cudaStream_t s)
+                              void *scratch, size_t scratch_bytes, bool alloc, std::vector<char> &taken,
+                              cudaStream_t s)
 {
     const SlotRow row = slot_row(nvec, dtype);
     static thread_local SlotArgs<kMaxSectors> a;  // host staging (22 KB); copied at launch
@@ -141,6 +144,7 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
         }
         std::stable_sort(todo.begin(), todo.end(),
                          [&](int u, int v) { return sectors[u].basis->dim > sectors[v].basis->dim; });
+        bool direct = false;
         for (size_t i = 0; i < todo.size();) {
             size_t j = i, bytes = 0;
             for (; j < todo.size(); ++j) {
@@ -151,14 +155,16 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
             }
             char *xs = scratch_bytes >= bytes + kSlotQueueBytes ? (char *)scratch : nullptr;
             void *own = nullptr;
-            if (!xs) {
-                if (ws_alloc(&own, bytes + kSlotQueueBytes, s) != cudaSuccess) {
-                    (void)cudaGetLastError();
-                    return cudaSuccess;  // the remaining sectors take the other kernels
-                }
+            if (!xs && !direct) {
+                direct = !alloc || stream_captured(s) ||
+                         ws_alloc_optional(&own, bytes + kSlotQueueBytes, s) != cudaSuccess;
                 xs = (char *)own;
             }
-            unsigned long long *queue = (unsigned long long *)(xs + bytes);
+            if (direct) {
+                xs = nullptr;
+                j = todo.size();
+            }
+            unsigned long long *queue = direct ? nullptr : (unsigned long long *)(xs + bytes);
             const ed_basis *b0 = sectors[todo[i]].basis;
             a.op = op;
             a.op.even = 0;
@@ -179,9 +185,10 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
             for (size_t q = i; q < j; ++q) {
                 const ed_sector &sec = sectors[todo[q]];
                 const IndexView iv = sec.basis->index_view();
-                fill.push_back(SlotFill{iv.slots, iv.states, iv.norms, iv.dim, sec.d_x, xs + at});
+                char *copy = direct ? nullptr : xs + at;
+                fill.push_back(SlotFill{iv.slots, iv.states, iv.norms, iv.dim, sec.d_x, copy});
                 SlotSector &d = a.sec[q - i];
-                d = slot_sector(op, sec.basis->group_view(), iv, sec.d_x, xs + at, sec.d_y, j - i == 1);
+                d = slot_sector(op, sec.basis->group_view(), iv, sec.d_x, copy, sec.d_y, j - i == 1);
                 d.tile_begin = tiles;
                 tiles += slot_tiles(d);
                 at += slot_copy_bytes(iv.slots, nvec, dtype);
@@ -193,11 +200,19 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
             a.order = track ? a.max_order : 1;
             a.beyond_l2 = bytes > kSlotL2Bytes;
             a.total_tiles = tiles;
-            cudaError_t e = launch_slot_fill(fill.data(), (int)fill.size(), nvec, dtype, queue, s);
+            cudaError_t e = direct ? cudaSuccess
+                                   : launch_slot_fill(fill.data(), (int)fill.size(), nvec, dtype, queue, s);
             if (e == cudaSuccess)
                 e = batch_gate(&a.ctl);
             a.ctl.queue = queue;
-            if (e == cudaSuccess)
+            if (e == cudaSuccess && direct)
+                switch (dtype) {
+                case ED_F64: e = slotn_direct_f64(a, track != 0, row.el, s); break;
+                case ED_F32: e = slotn_direct_f32(a, track != 0, row.el, s); break;
+                case ED_C128: e = slotn_direct_c128(a, track != 0, row.el, s); break;
+                case ED_C64: e = slotn_direct_c64(a, track != 0, row.el, s); break;
+                }
+            else if (e == cudaSuccess)
                 switch (dtype) {
                 case ED_F64: e = slotn_f64(a, search, track != 0, row.el, s); break;
                 case ED_F32: e = slotn_f32(a, search, track != 0, row.el, s); break;
@@ -298,7 +313,7 @@ extern "C" ed_status ed_matvec_multi(const ed_operator *op, const ed_sector *sec
     }
     std::vector<char> taken(n_sectors, 0);
     if (g_multi_policy != 2 &&
-        launch_slot_batch(ov, sectors, n_sectors, nvec, dtype, nullptr, 0, taken, (cudaStream_t)stream) != cudaSuccess) {
+        launch_slot_batch(ov, sectors, n_sectors, nvec, dtype, nullptr, 0, true, taken, (cudaStream_t)stream) != cudaSuccess) {
         (void)cudaGetLastError();
         return ED_ERR_CUDA;
     }

@@ -534,9 +534,11 @@ cudaError_t multi_dispatch_prec(const MultiArgs &a, bool track, cudaStream_t str
 cudaError_t batch_ctl(cudaStream_t s, BatchCtl *out);
 cudaError_t batch_gate(BatchCtl *out);
 // the sectors of a batch that the slot kernel serves (see ed_matvec_multi.cu),
-// and the scratch memory that lets it run without allocating
+// and the scratch memory that lets it run with slotted copies and without
+// allocating (alloc: it may take them from the pool where scratch is too small)
 cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n, int nvec, ed_dtype dtype,
-                              void *scratch, size_t scratch_bytes, std::vector<char> &taken, cudaStream_t s);
+                              void *scratch, size_t scratch_bytes, bool alloc, std::vector<char> &taken,
+                              cudaStream_t s);
 size_t slot_batch_bytes(const ed_sector *sectors, int n, int nvec, ed_dtype dtype);
 void set_inject_stall(bool on);
 int multi_policy_get();

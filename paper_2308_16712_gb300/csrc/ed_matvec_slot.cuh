@@ -57,14 +57,28 @@ constexpr int kSlMaxTable = 16384; // bytes of the coefficient table
 // 8 vectors, 180 MB, 1.8 -> 2.2 ms), and at 600 MB (ring N=36 fp64) it is even.
 constexpr size_t kSlotL2Bytes = 512ull << 20;
 
+// Index of a basis as a launch without the slotted copy reads it (the fields of
+// IndexView).
+struct SlotFind {
+    const uint32_t *htab;
+    const void *hent;
+    const uint64_t *bkt;
+    const ulonglong2 *stash;
+    uint32_t n_stash;
+    int hbits, hwide, norm_bits, bbits, brem;
+};
+
 struct SlotSector {
-    SlotView v;
+    union {
+        SlotView v;
+        SlotFind find;        // launches without the slotted copy
+    };
     const uint64_t *states;
     const uint16_t *norms;
     const double2 *chi;       // characters in the order of the search used
     const float2 *chif;
     const void *x;
-    const void *xs;           // slotted copy
+    const void *xs;           // slotted copy (null: gathered from x)
     void *y;
     uint64_t dim;
     uint64_t tile_begin;      // first tile of this sector in the batch
@@ -86,7 +100,7 @@ struct SlotArgs {
     int beyond_l2;            // the slotted copies exceed L2: gather past L1
     int byte;                 // the coefficient table has at most 256 entries
     uint64_t total_tiles;
-    BatchCtl ctl;             // tile queue (zeroed by the fill), status word and gate
+    BatchCtl ctl;             // tile queue (zeroed by the fill; null: static tiles), status word and gate
     SlotSector sec[kSec];     // read from the launch parameters (constant bank)
 };
 
@@ -150,19 +164,23 @@ __host__ __device__ inline uint32_t slot_list_terms(const OpView &op, int log_gr
 }
 
 template <typename W, typename T>
-__host__ __device__ inline size_t slot_warp_bytes(const OpView &op, int log_group, bool plain, bool byte)
+__host__ __device__ inline size_t slot_warp_bytes(const OpView &op, int log_group, bool plain, bool byte,
+                                                  bool direct = false)
 {
     const size_t terms = slot_list_terms(op, log_group);
+    if (direct)  // coefficient index and norm of every term
+        return align16(sizeof(SlotWarp<W, T>) + terms * 8);
     return align16(sizeof(SlotWarp<W, T>) + terms * 4 + (plain ? 0 : byte ? terms : terms * 2));
 }
 
 template <typename W, typename T, bool kFact>
 __host__ __device__ inline size_t slot_smem_bytes(const GroupView &g, const OpView &op, int order, int max_order,
-                                                  int log_group, bool batch, bool plain, bool byte)
+                                                  int log_group, bool batch, bool plain, bool byte,
+                                                  bool direct)
 {
     size_t off[7];
     slot_smem_layout<W, T, kFact>(g, op, order, max_order, batch, off);
-    return off[6] + kSlWarps * slot_warp_bytes<W, T>(op, log_group, plain, byte);
+    return off[6] + kSlWarps * slot_warp_bytes<W, T>(op, log_group, plain, byte, direct);
 }
 
 // kSearch: 0 every element of the group (factored or not), 1 ring runs, 2 torus
@@ -175,10 +193,26 @@ __host__ __device__ inline size_t slot_smem_bytes(const GroupView &g, const OpVi
 template <typename W, typename T, bool kTrack, int kSearch>
 constexpr int kSlBlocks = sizeof(W) == 8 ? (kTrack && kSearch == 2 ? 4 : 5) : sizeof(T) == 4 && !kTrack ? 8 : 6;
 
-template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int kSec>
-__global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) k_matvec_slot(const __grid_constant__ SlotArgs<kSec> a)
+// a b rounded by itself, never contracted into a following addition
+__device__ __forceinline__ float mul_alone(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_alone(double a, double b) { return __dmul_rn(a, b); }
+
+// kDirect: without the slotted copy, for calls that cannot have it (no memory, or
+// a product that is being captured: a graph with an allocation in it can
+// neither be a child of another nor be instantiated twice, and takes its memory
+// only when it is launched).  Phase B finds a term's row and norm through the
+// basis's own index, phase C forms sqrt(n) x with the rounding of the fill, and
+// all else is the same, so the result is the one with the copy bit for bit.  The
+// price is a second random read per term, waited for in its round: with the copy
+// / without / by the kernels below, ring N=36 fp64 25.9 / 33.2 / 41.0 ms, ring N=38
+// 8 vectors fp32 104 / 151 / 180, 6x6 torus complex128 179 / 332 / 837, ring N=32
+// fp32 0.91 / 1.32 / 1.21, the batch of XXZ N=28 43 / 63 / 57.  Four blocks per SM
+// (ring N=36: five, with spills and less L1, 41.1; three 32.6 but N=32 1.51).
+template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int kSec, bool kDirect = false>
+__global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTrack, kSearch>) k_matvec_slot(const __grid_constant__ SlotArgs<kSec> a)
 {
     static_assert(!kC || EL % 2 == 0, "a complex number per lane at least");
+    static_assert(!kDirect || kSearch == 0, "the search is chosen at run time");
     constexpr bool kBatch = kSec > 1;
     extern __shared__ __align__(16) unsigned char smem[];
     const bool fact = kSearch > 0 || a.g.fact;
@@ -196,12 +230,13 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
     T *sm_isq = reinterpret_cast<T *>(smem + off[5]);
     const bool uniform = a.op.uniform != 0;
     const bool plain = !kTrack && uniform;  // no coefficients at all
-    const bool byte = kTrack && !kBatch && a.byte, even = kTrack && !kBatch && a.op.even;
+    const bool byte = kTrack && !kBatch && !kDirect && a.byte, even = kTrack && !kBatch && a.op.even;
     SlotWarp<W, T> &ws = *reinterpret_cast<SlotWarp<W, T> *>(
-        smem + off[6] + (threadIdx.x >> 5) * slot_warp_bytes<W, T>(a.op, a.log_group, plain, byte));
+        smem + off[6] + (threadIdx.x >> 5) * slot_warp_bytes<W, T>(a.op, a.log_group, plain, byte, kDirect));
     uint32_t *term = reinterpret_cast<uint32_t *>(&ws + 1);
     uint16_t *coef = reinterpret_cast<uint16_t *>(term + slot_list_terms(a.op, a.log_group));
     uint8_t *coef8 = reinterpret_cast<uint8_t *>(coef);
+    uint16_t *norm = coef + slot_list_terms(a.op, a.log_group);  // kDirect
     {
         const int nm = fact ? a.g.n_cos : a.g.n_perm;
         const W *gm;
@@ -262,13 +297,20 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
     // Tiles from a queue: dealt statically, the warps of an SM drift apart (the
     // scheduler favours some) and a third of them had finished for most of the
     // launch (ring N=36: 45 % of the warp slots in use on average, 62 % resident).
+    // Without a fill to zero a queue (kDirect) they are dealt all the same.
     uint64_t tile = 0, tile_end = 0;
+    uint64_t dealt = ((uint64_t)blockIdx.x * kSlWarps + (threadIdx.x >> 5)) * (uint64_t)a.chunk;
     while (true) {
         if (tile == tile_end) {
-            unsigned long long t = 0;
-            if (lane == 0)
-                t = atomicAdd(a.ctl.queue, (unsigned long long)a.chunk);
-            tile = __shfl_sync(kAll, t, 0);
+            if constexpr (kDirect) {
+                tile = dealt;
+                dealt += (uint64_t)gridDim.x * kSlWarps * (uint64_t)a.chunk;
+            } else {
+                unsigned long long t = 0;
+                if (lane == 0)
+                    t = atomicAdd(a.ctl.queue, (unsigned long long)a.chunk);
+                tile = __shfl_sync(kAll, t, 0);
+            }
             tile_end = min(tile + (uint64_t)a.chunk, a.total_tiles);
             if (tile >= a.total_tiles)
                 break;
@@ -378,7 +420,9 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
                     rep_search_rot1<W, kTrack>(s, sm_kind, sm_masks, a.g, flip, full, best, gbest);
                 } else if constexpr (kSearch == 2) {
                     rep_search_blocks<W, kTrack>(s, sm_masks, a.g, flip, full, best, gbest);
-                } else if (kBatch && a.g.fact && a.g.prune == 2) {
+                } else if (kDirect && a.g.fact && a.g.prune == 1) {
+                    rep_search_rot1<W, kTrack>(s, sm_kind, sm_masks, a.g, flip, full, best, gbest);
+                } else if ((kBatch || kDirect) && a.g.fact && a.g.prune == 2) {
                     rep_search_blocks<W, kTrack>(s, sm_masks, a.g, flip, full, best, gbest);
                 } else if (a.g.fact) {
                     if (kTrack)
@@ -397,11 +441,30 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
                     else
                         coef[t] = (uint16_t)at;
                 }
-                key = slot_key((uint64_t)best);
-                bucket = slot_bucket((uint64_t)best, key, sd.v);
-                pilot = load_pilot(sd.v.pilots + bucket, keep);
+                if constexpr (kDirect) {
+                    uint32_t row = 0, nj = 0;
+                    bool found;
+                    if (sd.find.bkt) {
+                        found = find_bucketed((uint64_t)best, sd.find.bkt, sd.find.stash, sd.find.n_stash, n,
+                                              sd.find.bbits, sd.find.brem, row, nj);
+                    } else {
+                        IndexView ix;
+                        ix.htab = sd.find.htab;
+                        ix.hent = sd.find.hent;
+                        ix.hbits = sd.find.hbits;
+                        ix.hwide = sd.find.hwide;
+                        ix.norm_bits = sd.find.norm_bits;
+                        found = find_hashed((uint64_t)best, ix, row, nj);
+                    }
+                    term[t] = row;
+                    norm[t] = found ? (uint16_t)nj : (uint16_t)0;  // 0: without weight, not in the basis
+                } else {
+                    key = slot_key((uint64_t)best);
+                    bucket = slot_bucket((uint64_t)best, key, sd.v);
+                    pilot = load_pilot(sd.v.pilots + bucket, keep);
+                }
             }
-            if (base && t - 32 < total)
+            if (!kDirect && base && t - 32 < total)
                 term[t - 32] = slot_finish(key_p, bucket_p, pilot_p, sd.v);
         }
         __syncwarp();
@@ -434,7 +497,18 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const uint32_t q = k + u * split;
-                        if (q < k1) {
+                        if (kDirect && q < k1) {
+                            // row 0 stands in for a state that is not in the basis
+                            const T *from = x + (uint64_t)term[q] * (uint32_t)a.scalars + e0;
+                            if (whole) {
+                                v[u] = *reinterpret_cast<const Vec *>(from);
+                            } else {
+#pragma unroll
+                                for (int e = 0; e < EL; ++e)
+                                    v[u].e[e] = e0 + e < a.scalars ? from[e] : T(0);
+                            }
+                            ci[u] = plain ? 0u : coef[q];
+                        } else if (q < k1) {
                             const T *from = xs + (uint64_t)term[q] * (uint32_t)a.stride;
                             if (a.beyond_l2)
                                 load_random<sizeof(Vec)>(&v[u], from);
@@ -446,6 +520,19 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
 #pragma unroll
                             for (int e = 0; e < EL; ++e)
                                 v[u].e[e] = T(0);
+                        }
+                    }
+                    if constexpr (kDirect) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const uint32_t q = k + u * split;
+                            const uint32_t nj = q < k1 ? norm[q] : 1u;
+                            if (nj != 1) {  // few states of a large sector
+                                const T sq = sqrt((T)nj);
+#pragma unroll
+                                for (int e = 0; e < EL; ++e)
+                                    v[u].e[e] = nj ? mul_alone(sq, v[u].e[e]) : T(0);
+                            }
                         }
                     }
 #pragma unroll
@@ -529,36 +616,37 @@ __global__ void __launch_bounds__(kSlThreads, kSlBlocks<W, T, kTrack, kSearch>) 
     }
 }
 
-template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int kSec>
+template <typename W, typename T, bool kC, bool kTrack, int kSearch, int EL, int kSec, bool kDirect>
 cudaError_t slot_launch(const SlotArgs<kSec> &a, cudaStream_t stream)
 {
-    auto kern = k_matvec_slot<W, T, kC, kTrack, kSearch, EL, kSec>;
+    auto kern = k_matvec_slot<W, T, kC, kTrack, kSearch, EL, kSec, kDirect>;
     const bool plain = !kTrack && a.op.uniform, byte = kTrack && kSec == 1 && a.byte;
     const size_t smem = kSearch > 0 || a.g.fact
-                            ? slot_smem_bytes<W, T, true>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain, byte)
-                            : slot_smem_bytes<W, T, false>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain, byte);
+                            ? slot_smem_bytes<W, T, true>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain, byte, kDirect)
+                            : slot_smem_bytes<W, T, false>(a.g, a.op, a.order, a.max_order, a.log_group, kSec > 1, plain, byte, kDirect);
     int sms = 0, per_sm = 0;
     const cudaError_t e = kernel_occupancy((const void *)kern, kSlThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
         return e;
     const uint64_t blocks_needed = (a.total_tiles + kSlWarps - 1) / kSlWarps;
-    per_sm = std::max(1, std::min(per_sm, kSlBlocks<W, T, kTrack, kSearch>));
-    const int grid = (int)std::min<uint64_t>(blocks_needed, (uint64_t)sms * per_sm);
+    if (!kDirect)
+        per_sm = std::min(per_sm, kSlBlocks<W, T, kTrack, kSearch>);
+    const int grid = (int)std::min<uint64_t>(blocks_needed, (uint64_t)sms * std::max(1, per_sm));
     kern<<<std::max(grid, 1), kSlThreads, smem, stream>>>(a); count_launch();
     return cudaGetLastError();
 }
 
-template <typename T, bool kC, int kSearch, int kSec>
+template <typename T, bool kC, int kSearch, int kSec, bool kDirect = false>
 cudaError_t slot_dispatch(const SlotArgs<kSec> &a, bool track, int el, cudaStream_t s)
 {
     const bool w32 = a.g.n_sites <= 32;
 #define ED_SL_W(EL)                                                                                  \
     do {                                                                                             \
         if (w32)                                                                                     \
-            return track ? slot_launch<uint32_t, T, kC, true, kSearch, EL, kSec>(a, s)               \
-                         : slot_launch<uint32_t, T, kC, false, kSearch, EL, kSec>(a, s);             \
-        return track ? slot_launch<uint64_t, T, kC, true, kSearch, EL, kSec>(a, s)                   \
-                     : slot_launch<uint64_t, T, kC, false, kSearch, EL, kSec>(a, s);                 \
+            return track ? slot_launch<uint32_t, T, kC, true, kSearch, EL, kSec, kDirect>(a, s)      \
+                         : slot_launch<uint32_t, T, kC, false, kSearch, EL, kSec, kDirect>(a, s);    \
+        return track ? slot_launch<uint64_t, T, kC, true, kSearch, EL, kSec, kDirect>(a, s)          \
+                     : slot_launch<uint64_t, T, kC, false, kSearch, EL, kSec, kDirect>(a, s);        \
     } while (0)
     if constexpr (!kC)
         if (el == 1)
@@ -572,18 +660,23 @@ cudaError_t slot_dispatch(const SlotArgs<kSec> &a, bool track, int el, cudaStrea
     return cudaErrorInvalidValue;
 }
 
-// ed_matvec.cu: lanes of a row (log2), a sector's descriptor (tile_begin 0) and its
-// number of tiles; alone: tiles small enough to occupy the GPU
+// ed_matvec.cu: lanes of a row (log2), a sector's descriptor (tile_begin 0; xs
+// null: without the copy) and its number of tiles; alone: tiles small enough to
+// occupy the GPU; whether the stream is being captured
+bool stream_captured(cudaStream_t s);
 int slot_log_group(const OpView &op);
 SlotSector slot_sector(const OpView &op, const GroupView &g, const IndexView &ix, const void *x, const void *xs,
                        void *y, bool alone);
 int slot_chunk(uint64_t tiles);
 uint64_t slot_tiles(const SlotSector &d);
 
-// one sector / a batch, per dtype and search, in the ed_matvec_slot_*.cu units
+// one sector / a batch, per dtype and search, and without the copy, in the
+// ed_matvec_slot_*.cu units
 #define ED_SLOT_DECL(NAME)                                                                        \
     cudaError_t slot1_##NAME(const SlotArgs<1> &a, int search, bool track, int el, cudaStream_t s); \
-    cudaError_t slotn_##NAME(const SlotArgs<kMaxSectors> &a, int search, bool track, int el, cudaStream_t s);
+    cudaError_t slotn_##NAME(const SlotArgs<kMaxSectors> &a, int search, bool track, int el, cudaStream_t s); \
+    cudaError_t slot1_direct_##NAME(const SlotArgs<1> &a, bool track, int el, cudaStream_t s);    \
+    cudaError_t slotn_direct_##NAME(const SlotArgs<kMaxSectors> &a, bool track, int el, cudaStream_t s);
 ED_SLOT_DECL(f64)
 ED_SLOT_DECL(f32)
 ED_SLOT_DECL(c128)
