@@ -720,10 +720,12 @@ def run_job(args, w):
     # ---- FP32 batched: block-Lanczos steps (the timed headline) --------------
     ed.lanczos_block(O, B, X0, nvec, args.warmup, ed.ED_LANCZOS_F32_MATVEC | VO)
     launches0 = ed.launch_count()
+    products0 = ed.product_counts()
     sampler = ClockSampler(local) if rank == 0 else None
     ms_blk, (_, rb) = timed(lambda: ed.lanczos_block(O, B, X0, nvec, args.steps, ed.ED_LANCZOS_F32_MATVEC | VO))
     clocks = sampler.stop() if sampler else None
     launches = ed.launch_count() - launches0
+    products = {k: v - products0[k] for k, v in ed.product_counts().items() if v > products0[k]}
     ms_blk = max_over_ranks(ms_blk, world)
     per_step = ms_blk / args.steps
     rows_blk = dim * nvec * args.steps / (ms_blk * 1e-3)
@@ -762,9 +764,8 @@ def run_job(args, w):
     pk, pk_kind = peaks()
     hbm_peak = pk.get("hbm_gbs", 6800.0)
     alg_bytes = dim * (8 + 2 + 2 * 4 * nvec) + terms * (4 * nvec + 2)  # keys, norms, x_r, y_r; x_j, n(r')
-    kern_kind = {1: "row-per-lane", 2: "term-parallel"}.get(
-        tuning.get("kernel"), "slot" if ed.basis_slots(B)[0] else "term-parallel")
-    slot = kern_kind == "slot"  # x row per term, bucket too without slots
+    kern_kind = max(products, key=products.get)  # what served the timed products
+    slot = kern_kind == "slot"  # x row per term, bucket too without the copy
     sector_bytes = dim * (8 + 2 * 4 * nvec) + terms * ((0 if slot else 32) + max(32, 4 * nvec))
     t_s = prod_ms * 1e-3
     achieved_int = int_ops / t_s / 1e12
@@ -775,7 +776,8 @@ def run_job(args, w):
                     if (kern_kind, nvec) in KERNEL_DRAM_BYTES_PER_NNZ else None),
         "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the ring N=36 launch, "
                           "scaled by stored nonzeros",
-        "kernel": ({"slot": "k_matvec_slot (slot", "row-per-lane": "k_matvec (row-per-lane",
+        "kernel": ({"slot": "k_matvec_slot (slot", "slot without copy": "k_matvec_slot (slot without copy",
+                    "row-per-lane": "k_matvec (row-per-lane",
                     "term-parallel": "k_matvec_tp (term-parallel"}[kern_kind]
                    + f", fp32, nvec={nvec}, "
                    + ("pruned rotation search" if tuning.get("search") != 0 else "search over every rotation")
@@ -792,7 +794,7 @@ def run_job(args, w):
     buf.fill_(1)
     gather_peak, _ = ed.peak("gather32", buf)
     del buf
-    # one x row per term (and one bucket without slots), one key/x/y row per basis row
+    # one x row per term (and one bucket without the copy), one key/x/y row per basis row
     accesses = terms * (1 if slot else 2) + dim
     roofline["random_access"] = {"accesses_per_launch": accesses, "achieved_per_s": accesses / t_s,
                                  "peak_per_s": gather_peak, "frac": accesses / t_s / gather_peak,
@@ -882,6 +884,7 @@ def run_job(args, w):
         "autotune": {"product": tuning, "kernel_names": {"0": "library rule (slot kernel where the sector has a slot index)",
                                                           "1": "row-per-lane", "2": "term-parallel"},
                      "search_names": {"-1": "n/a", "0": "every rotation", "1": "pruned to the longest runs"}},
+        "products": products,
         "gpu_launches": launches,
         "clocks": clocks,
         "secondary": secondary,

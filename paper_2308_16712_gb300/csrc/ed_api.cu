@@ -683,6 +683,10 @@ uint64_t binomial_host(int n, int k) { return binomial(n, k); }
 
 static std::atomic<unsigned long long> g_launches{0};
 void count_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+namespace {
+std::atomic<unsigned long long> g_products[kProductKinds];
+}  // namespace
+void count_product(ProductKernel k) { g_products[k].fetch_add(1, std::memory_order_relaxed); }
 void uncount_launch(unsigned n) { g_launches.fetch_sub(n, std::memory_order_relaxed); }
 unsigned long long launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 
@@ -1436,6 +1440,14 @@ void edx_force_prefix_search(int on) { g_force_prefix = on != 0; }
 // Test hook: the index later basis builds make (0 automatic, 1 hash index,
 // 2 bucketed index wherever its entry fits).
 void edx_index_policy(int policy) { g_index_policy = policy; }
+
+// Diagnostics hook: products issued since the library was loaded, by kernel:
+// row-per-lane, term-parallel, slot kernel with and without the slotted copy.
+void edx_product_counts(unsigned long long *out)
+{
+    for (int k = 0; k < edk::kProductKinds; ++k)
+        out[k] = edk::g_products[k].load(std::memory_order_relaxed);
+}
 
 // Test hook: later basis builds make a slot index for sectors of at least this
 // many states (0: the library's own threshold).

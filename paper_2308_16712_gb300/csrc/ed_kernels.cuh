@@ -23,6 +23,10 @@ void count_launch(unsigned n = 1);
 // Takes back n counted launches (kernels recorded into a graph by stream
 // capture are counted again each time the graph is launched).
 void uncount_launch(unsigned n);
+// Products issued (a captured one counts once), by the kernel that serves them;
+// one batched launch is one product (diagnostics).
+enum ProductKernel { kProductRows, kProductTerms, kProductSlots, kProductDirect, kProductKinds };
+void count_product(ProductKernel k);
 unsigned long long launches_so_far();
 
 // ---- basis build (Sec. "States enumeration") --------------------------------

@@ -183,6 +183,7 @@ static cudaError_t launch_slot(const OpView &op, const GroupView &g, const Index
     a.total_tiles = slot_tiles(a.sec[0]);
     a.chunk = slot_chunk(a.total_tiles);
     const int search = slot_search(g);
+    count_product(xs ? kProductSlots : kProductDirect);
     if (!xs) {
         switch (dtype) {
         case ED_F64: return slot1_direct_f64(a, track, row.el, stream);
@@ -229,6 +230,7 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
     const bool rule = block8 ? (g_kernel_policy == 2 || (g_kernel_policy == 0 && dtype == ED_F32))
                              : use_term_parallel(nvec, op, dtype, g.n_sites);
     const bool tp = tp_ok && (v.kernel == 2 || ((v.kernel == 0 || v.kernel == 4) && rule));
+    count_product(tp ? kProductTerms : kProductRows);
     if (tp) {
         const TpArgs<1> t = single_tp_args(op, g, ix, x, y);
         const int k = tp_index_kind(t.sec[0]);

@@ -205,6 +205,7 @@ cudaError_t launch_slot_batch(const OpView &op, const ed_sector *sectors, int n,
             if (e == cudaSuccess)
                 e = batch_gate(&a.ctl);
             a.ctl.queue = queue;
+            count_product(direct ? kProductDirect : kProductSlots);
             if (e == cudaSuccess && direct)
                 switch (dtype) {
                 case ED_F64: e = slotn_direct_f64(a, track != 0, row.el, s); break;
@@ -236,7 +237,9 @@ cudaError_t multi_launch_any(const MultiArgs &a, bool track, ed_dtype dtype, cud
     bool same_kind = true;
     for (int k = 1; k < a.n_sectors; ++k)
         same_kind = same_kind && tp_index_kind(a.sec[k]) == tp_index_kind(a.sec[0]);
-    if (same_kind && use_term_parallel(a.nvec, a.op, dtype, a.g.n_sites)) {
+    const bool terms = same_kind && use_term_parallel(a.nvec, a.op, dtype, a.g.n_sites);
+    count_product(terms ? kProductTerms : kProductRows);
+    if (terms) {
         const int kind = a.n_sectors > 0 ? tp_index_kind(a.sec[0]) : 0;
         static thread_local TpArgs<kMaxSectors> t;  // host staging (17 KB); copied at launch
         t.op = a.op;

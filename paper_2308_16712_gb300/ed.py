@@ -91,6 +91,7 @@ _SIGS = {
     "edx_basis_bucket": (_i32, [_P, ctypes.POINTER(_i32), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_slot_min_dim": (None, [_u64]),
     "edx_optional_memory": (None, [_u64]),
+    "edx_product_counts": (None, [ctypes.POINTER(ctypes.c_ulonglong)]),
     "edx_basis_slots": (_i32, [_P, ctypes.POINTER(_u64), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_count_nnz": (_i32, [_P, _P, ctypes.POINTER(ctypes.c_ulonglong)]),
     "edx_force_prefix_search": (None, [_i32]),
@@ -288,6 +289,17 @@ def matvec(op: Operator, basis: Basis, x, y, nvec: int = 1, stream=None):
 def launch_count() -> int:
     """Kernel launches the library has issued since it was loaded (diagnostics)."""
     return int(_lib.edx_launch_count())
+
+
+PRODUCT_KERNELS = ("row-per-lane", "term-parallel", "slot", "slot without copy")
+
+
+def product_counts() -> dict:
+    """Products issued since the library was loaded, by the kernel that serves
+    them (diagnostics; a captured product or a batched launch counts once)."""
+    c = (ctypes.c_ulonglong * len(PRODUCT_KERNELS))()
+    _lib.edx_product_counts(c)
+    return dict(zip(PRODUCT_KERNELS, c))
 
 
 def force_generic(on: bool) -> None:

@@ -174,3 +174,37 @@ def test_solvers_without_the_copy(mode, graph):
     finally:
         ed.lanczos_graph(old)
     assert got[0] == want[0] and torch.equal(got[1], want[1])
+
+
+def served(ed, call):
+    before = ed.product_counts()
+    call()
+    return {k: v - before[k] for k, v in ed.product_counts().items() if v > before[k]}
+
+
+def test_product_counts_name_the_kernel_that_ran():
+    torch, ed = gpu()
+    p, c = ei.ring_group(20, 0, +1)
+    S = build_pair(20, 10, +1, p, c, ei.heisenberg_ring(20), with_oracle=False)
+    x = to_torch(ei.x_by_index(1, S["dim"], 8), np.float32)
+    y = torch.empty_like(x)
+    x64 = x.to(torch.float64)
+
+    def product():
+        ed.matvec(S["O"], S["B"], x, y, 8)
+
+    def block():
+        ed.lanczos_block(S["O"], S["B"], x64, 8, 12, ed.ED_LANCZOS_F32_MATVEC | ed.ED_LANCZOS_VALUES_ONLY)
+
+    def batch():
+        ed.matvec_multi(S["O"], [(S["B"], x, y)], 8)
+
+    assert served(ed, product) == served(ed, batch) == {"slot": 1}
+    assert served(ed, block) == {"slot": 12}
+    ed.optional_memory(0)
+    assert served(ed, product) == served(ed, batch) == {"slot without copy": 1}
+    assert served(ed, block) == {"slot without copy": 12}
+    for policy, name in (("rowwise", "row-per-lane"), ("term_parallel", "term-parallel")):
+        ed.kernel_policy(policy)
+        assert served(ed, product) == {name: 1}
+        assert served(ed, block) == {name: 12}
