@@ -1441,6 +1441,12 @@ void edx_force_prefix_search(int on) { g_force_prefix = on != 0; }
 // 2 bucketed index wherever its entry fits).
 void edx_index_policy(int policy) { g_index_policy = policy; }
 
+// Test hook: the rule by which a solver takes the slot kernel's scratch (host only).
+int edx_slot_scratch_fits(uint64_t want, uint64_t free_bytes, uint64_t later)
+{
+    return edk::slot_scratch_fits(want, free_bytes, later) ? 1 : 0;
+}
+
 // Diagnostics hook: products issued since the library was loaded, by kernel:
 // row-per-lane, term-parallel, slot kernel with and without the slotted copy.
 void edx_product_counts(unsigned long long *out)

@@ -741,17 +741,19 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
         ED_L_TRY(S.get(&d_eigs, n_eig));
     ED_L_TRY(cudaMemsetAsync(beta, 0, (mmax + 2) * sizeof(double), st));
 
-    // scratch of the slot kernel, for every product of the call where half of what
-    // is left has room, else for those of the main run; products without it give
-    // the same bits from x itself
+    // scratch of the slot kernel, for every product of the call where it fits beside
+    // the vectors (the refinement of a mixed run may still need two), else for
+    // those of the main run; products without it give the same bits from x itself
     void *slot_ws = nullptr;
     size_t slot_bytes = 0;
+    const size_t later = f32 && !ring[0] ? 2 * vec_bytes : 0;
     for (const ed_dtype dt : {dt64, dt32}) {
         if (!iv.slots.pilots || slot_ws || (dt == dt32 && !f32))
             break;
         const size_t want = slot_scratch_bytes(iv.slots, 1, dt);
         cudaMemGetInfo(&free_b, &total_b);
-        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc_optional(&slot_ws, want, st) == cudaSuccess) {
+        if (slot_scratch_fits(want, free_b + ws_cached_bytes(), later) &&
+            ws_alloc_optional(&slot_ws, want, st) == cudaSuccess) {
             S.ptrs.push_back(slot_ws);
             slot_bytes = want;
         }

@@ -1134,14 +1134,15 @@ ed_status run_block(const ed_operator *op, const ed_basis *b, const double *x0, 
     int *stop = flags;
     const int yk = f32 ? 0 : 1;
     MatvecVariant tuned = tuned_variant(b, P, f32 ? ED_F32 : ED_F64);
-    // scratch of the slot kernel, kept for the whole call where half of what is left
-    // has room; products without it give the same bits from x itself
+    // scratch of the slot kernel, kept for the whole call where it fits beside the
+    // vectors, all of which are allocated by now; products without it give the same
+    // bits from x itself
     if (iv.slots.pilots) {
         const size_t want = slot_scratch_bytes(iv.slots, P, f32 ? ED_F32 : ED_F64);
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
         void *ws = nullptr;
-        if (want < (free_b + ws_cached_bytes()) / 2 && ws_alloc_optional(&ws, want, st) == cudaSuccess) {
+        if (slot_scratch_fits(want, free_b + ws_cached_bytes(), 0) && ws_alloc_optional(&ws, want, st) == cudaSuccess) {
             S.ptrs.push_back(ws);
             tuned.scratch = ws;
             tuned.scratch_bytes = want;

@@ -91,6 +91,7 @@ _SIGS = {
     "edx_basis_bucket": (_i32, [_P, ctypes.POINTER(_i32), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_slot_min_dim": (None, [_u64]),
     "edx_optional_memory": (None, [_u64]),
+    "edx_slot_scratch_fits": (_i32, [_u64, _u64, _u64]),
     "edx_product_counts": (None, [ctypes.POINTER(ctypes.c_ulonglong)]),
     "edx_basis_slots": (_i32, [_P, ctypes.POINTER(_u64), ctypes.POINTER(ctypes.c_uint32)]),
     "edx_count_nnz": (_i32, [_P, _P, ctypes.POINTER(ctypes.c_ulonglong)]),
