@@ -20,7 +20,6 @@
 #include <vector>
 
 #include "ed_kernels.cuh"
-#include "ed_lanczos_step.cuh"
 #include "ed_tridiag.cuh"
 
 namespace edk {
@@ -436,27 +435,6 @@ __global__ void k_finish_residual(const double2 *res_part, const double2 *den_pa
         *out = sqrt(fmax(r, 0.0) / d);
 }
 
-// dot, update and normalisation of a step in one block (ed_lanczos_step.cuh);
-// with a step index jp, alpha, beta and the store are offset by *jp, which is
-// then advanced
-template <bool kC>
-__global__ void __launch_bounds__(kFusedThreads) k_step_fused(typename Vec<kC>::D *w, const typename Vec<kC>::D *v,
-                                                              const typename Vec<kC>::D *vp,
-                                                              typename Vec<kC>::D *vn, uint64_t n, double *alpha,
-                                                              double *beta, typename Vec<kC>::D *store, int *jp)
-{
-    using D = typename Vec<kC>::D;
-    using F = typename Vec<kC>::F;
-    const int j = jp ? *jp : 0;
-    lanczos_step<D, F, D>(n, w, w, v, vp, vn, (F *)nullptr, store ? store + (uint64_t)(j + 1) * n : nullptr,
-                          (F *)nullptr, alpha + j, beta + j);
-    if (jp) {
-        __syncthreads();  // every thread has read *jp
-        if (threadIdx.x == 0)
-            *jp = j + 1;
-    }
-}
-
 // ---- full reorthogonalisation against the kept Krylov vectors ----------------
 struct Part4 {  // compensated real and imaginary parts of one block's partial
     double rs, rc, is, ic;
@@ -692,7 +670,6 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
     if (reorth && !store)
         return ED_ERR_UNSUPPORTED;
 
-    const bool fused = !reorth && n <= kFusedMax;  // the vector part of an fp64 step in one block
     const bool graph = !reorth && !push && (g_lanczos_graph == 1 || (g_lanczos_graph < 0 && n <= kGraphMaxDim));
     Scratch S(st);
     Graphs GR;
@@ -809,13 +786,6 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
                 return e;
             }
             D *vn = Vs ? Vs + (uint64_t)(j + 1) * n : (vp ? vp : ring[1]);
-            if (fused && !use_f32) {
-                k_step_fused<kC><<<1, kFusedThreads, 0, st>>>(w, v, vp, vn, n, alpha + j, beta + j, nullptr, nullptr);
-                count_launch();
-                vp = v;
-                v = vn;
-                continue;
-            }
             if (use_f32) {
                 k_dot_part<kC, true><<<nparts, kRedThreads, 0, st>>>(v, w32, n, part_a, tickets, alpha + j); count_launch();
                 k_update<kC, true><<<nparts, kRedThreads, 0, st>>>(w32, w, v, vp, n, alpha + j, beta + j, part_b,
@@ -869,11 +839,6 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
                 if ((e2 = launch_matvec_v(ov, gv, iv, track, v, w, 1, dt64, variant(dt64), s)) !=
                     cudaSuccess)
                     return e2;
-                if (fused) {
-                    k_step_fused<kC><<<1, kFusedThreads, 0, s>>>(w, v, vp, vn, n, alpha, beta, Vs, jdev);
-                    count_launch();
-                    return cudaGetLastError();
-                }
                 k_dot_part<kC, false><<<nparts, kRedThreads, 0, s>>>(v, w, n, part_a, tickets, alpha, jdev); count_launch();
                 k_update<kC, false><<<nparts, kRedThreads, 0, s>>>(w, w, v, vp, n, alpha, beta, part_b,
                                                                     tickets + 1, beta + 1, jdev); count_launch();

@@ -22,7 +22,6 @@
 
 #include "ed_kernels.cuh"
 #include "ed_matvec_multi_impl.cuh"
-#include "ed_lanczos_step.cuh"
 #include "ed_tridiag.cuh"
 
 namespace edk {
@@ -268,26 +267,6 @@ __global__ void __launch_bounds__(kThr) k_seg_resid(Seg sg, const typename El<C>
         part[blockIdx.x] = make_double2(k.s, k.c);
 }
 
-// dot, update and normalisation of a step, one block per sector (all sectors of
-// at most kFusedMax states); off: n_sec + 1 first elements
-template <bool C, typename WI>
-__global__ void __launch_bounds__(kFusedThreads) k_seg_fused(const uint64_t *off, int stride, const WI *w_in,
-                                                             typename El<C>::D *w, const typename El<C>::D *v,
-                                                             const typename El<C>::D *vp, typename El<C>::D *vn,
-                                                             typename El<C>::F *x32, double *alpha, double *beta,
-                                                             const int *step, Store st)
-{
-    using D = typename El<C>::D;
-    using F = typename El<C>::F;
-    const int s = blockIdx.x, j = *step;
-    const uint64_t lo = off[s], n = off[s + 1] - lo;
-    const bool keep = st.base && j + 1 < st.count;
-    const uint64_t at = (uint64_t)(j + 1) * st.total + lo;
-    lanczos_step<D, F, WI>(n, w_in + lo, w + lo, v + lo, vp ? vp + lo : nullptr, vn + lo, x32 ? x32 + lo : nullptr,
-                           keep && !st.f32 ? (D *)st.base + at : nullptr, keep && st.f32 ? (F *)st.base + at : nullptr,
-                           alpha + (size_t)s * stride + j, beta + (size_t)s * stride + j);
-}
-
 __global__ void k_step_set(int *step, int v) { *step = v; }
 __global__ void k_step_inc(int *step) { *step += 1; }
 
@@ -384,7 +363,6 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         }
     }
     sec_blk[ns] = (int)blk_sec.size();
-    uint64_t *d_off = nullptr;
     struct Wait {  // the tables above outlive their asynchronous copies on every way out
         cudaStream_t st;
         ~Wait() { cudaStreamSynchronize(st); }
@@ -411,11 +389,6 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         sg.blk_sec = p_bs;
         sg.sec_blk = p_sb;
     }
-    bool fused = true;
-    for (int k = 0; k < ns; ++k)
-        fused = fused && sectors[k].basis->dim <= kFusedMax;
-    LM_TRY(O.get(&d_off, ns + 1));
-    LM_TRY(cudaMemcpyAsync(d_off, off.data(), (ns + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
     D *x0, *ring0, *ring1, *w, *psi;
     F *x32 = nullptr, *w32 = nullptr;
     double *alpha, *beta, *y, *work, *lam, *nrm, *num, *den, *res;
@@ -565,23 +538,11 @@ ed_status run_multi(const ed_operator *op, const ed_sector *sectors, int ns, int
         }
         if (single) {
             LM_CHK(matvec(x32, w32, true, s));
-            if (fused) {
-                k_seg_fused<C, F><<<ns, kFusedThreads, 0, s>>>(d_off, stride, w32, w, v, vp, vn, x32, alpha, beta, step, keep);
-                count_launch();
-                k_step_inc<<<1, 1, 0, s>>>(step); count_launch();
-                return cudaGetLastError();
-            }
             k_seg_dot<C, F><<<nblk, kThr, 0, s>>>(sg, v, w32, part); count_launch();
             k_seg_final<<<ns, kThr, 0, s>>>(sg, part, alpha, step, 0, 0); count_launch();
             k_seg_update<C, F><<<nblk, kThr, 0, s>>>(sg, w32, w, v, vp, alpha, beta, step, part); count_launch();
         } else {
             LM_CHK(matvec(v, w, false, s));
-            if (fused) {
-                k_seg_fused<C, D><<<ns, kFusedThreads, 0, s>>>(d_off, stride, w, w, v, vp, vn, (F *)nullptr, alpha, beta, step, keep);
-                count_launch();
-                k_step_inc<<<1, 1, 0, s>>>(step); count_launch();
-                return cudaGetLastError();
-            }
             k_seg_dot<C, D><<<nblk, kThr, 0, s>>>(sg, v, w, part); count_launch();
             k_seg_final<<<ns, kThr, 0, s>>>(sg, part, alpha, step, 0, 0); count_launch();
             k_seg_update<C, D><<<nblk, kThr, 0, s>>>(sg, w, w, v, vp, alpha, beta, step, part); count_launch();
