@@ -485,10 +485,10 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
         for (int first = 0; first < rows; first += 32 >> group) {  // same trip count for all lanes
             const int rr = first + (lane >> group);
             const bool mine = rr < rows && e0 < a.scalars;
-            T acc[EL];
+            T acc[2][EL];
 #pragma unroll
             for (int e = 0; e < EL; ++e)
-                acc[e] = T(0);
+                acc[0][e] = acc[1][e] = T(0);
             if (mine) {
                 const uint32_t k1 = ws.off[rr + 1];
                 for (uint32_t k = ws.off[rr] + sp; k < k1; k += 4 * split) {
@@ -535,13 +535,22 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                             }
                         }
                     }
+                    // short chains of additions: four terms as a tree; with
+                    // coefficients two sums for alternate terms, of complex vectors
+                    // for the whole row (a tree would add 12 % to the arithmetic), of
+                    // real ones for the four
+                    if (plain) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (plain) {
+                        for (int e = 0; e < EL; ++e)
+                            acc[0][e] += (v[0].e[e] + v[1].e[e]) + (v[2].e[e] + v[3].e[e]);
+                    } else {
+                        T four[2][EL];
 #pragma unroll
-                            for (int e = 0; e < EL; ++e)
-                                acc[e] += v[u].e[e];
-                        } else {
+                        for (int e = 0; e < EL; ++e)
+                            four[0][e] = four[1][e] = T(0);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            T (&sum)[EL] = kC ? acc[u & 1] : four[u & 1];
                             Cplx<T> c;
                             if (kBatch && kTrack) {
                                 const uint32_t m = uniform ? 0u : ci[u] / (uint32_t)a.order;
@@ -558,22 +567,32 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                             if constexpr (kC) {
 #pragma unroll
                                 for (int e = 0; e < EL; e += 2) {
-                                    acc[e] = fma(c.re, v[u].e[e], fma(-c.im, v[u].e[e + 1], acc[e]));
-                                    acc[e + 1] = fma(c.re, v[u].e[e + 1], fma(c.im, v[u].e[e], acc[e + 1]));
+                                    sum[e] = fma(c.re, v[u].e[e], fma(-c.im, v[u].e[e + 1], sum[e]));
+                                    sum[e + 1] = fma(c.re, v[u].e[e + 1], fma(c.im, v[u].e[e], sum[e + 1]));
                                 }
                             } else {
 #pragma unroll
                                 for (int e = 0; e < EL; ++e)
-                                    acc[e] = fma(c.re, v[u].e[e], acc[e]);
+                                    sum[e] = fma(c.re, v[u].e[e], sum[e]);
                             }
                         }
+                        if constexpr (!kC) {
+#pragma unroll
+                            for (int e = 0; e < EL; ++e)
+                                acc[0][e] += four[0][e] + four[1][e];
+                        }
                     }
+                }
+                if (kC && !plain) {
+#pragma unroll
+                    for (int e = 0; e < EL; ++e)
+                        acc[0][e] += acc[1][e];
                 }
             }
             for (int o = split >> 1; o > 0; o >>= 1)
 #pragma unroll
                 for (int e = 0; e < EL; ++e)
-                    acc[e] += __shfl_xor_sync(kAll, acc[e], o << a.log_parts);
+                    acc[0][e] += __shfl_xor_sync(kAll, acc[0][e], o << a.log_parts);
             if (sp == 0 && mine && row0 + rr < sd.dim) {
                 const uint64_t at = (row0 + rr) * (uint32_t)a.scalars + e0;
                 Vec xv;
@@ -590,8 +609,8 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                 if constexpr (kC) {
 #pragma unroll
                     for (int e = 0; e < EL; e += 2) {  // conj(d) x + w acc
-                        out.e[e] = fma(w, acc[e], dg.re * xv.e[e]);
-                        out.e[e + 1] = fma(w, acc[e + 1], dg.re * xv.e[e + 1]);
+                        out.e[e] = fma(w, acc[0][e], dg.re * xv.e[e]);
+                        out.e[e + 1] = fma(w, acc[0][e + 1], dg.re * xv.e[e + 1]);
                         if (!real_op) {
                             out.e[e] = fma(dg.im, xv.e[e + 1], out.e[e]);
                             out.e[e + 1] = fma(-dg.im, xv.e[e], out.e[e + 1]);
@@ -600,7 +619,7 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                 } else {
 #pragma unroll
                     for (int e = 0; e < EL; ++e)
-                        out.e[e] = fma(w, acc[e], dg.re * xv.e[e]);
+                        out.e[e] = fma(w, acc[0][e], dg.re * xv.e[e]);
                 }
                 if (whole) {
                     *reinterpret_cast<Vec *>(y + at) = out;
