@@ -24,15 +24,17 @@ constexpr int kTriShared = 768;  // matrices up to this size are worked on in sh
 // p_{i+1} = (a_i - x) p_i - b_i^2 p_{i-1} (b2[i] = b_i^2 couples i-1 and i),
 // rescaled every fourth step; a vanishing p_i takes the sign that counts.  The
 // computed sequence is the exact one of a matrix whose entries differ by a few
-// roundings, as for the quotients p_i / p_{i-1}.
-__device__ __forceinline__ int tri_count(const double *a, const double *b2, int m, double x)
+// roundings, as for the quotients p_i / p_{i-1}.  The entries are to be of order
+// one, or four steps leave the range of a double: a[i] f is the diagonal, and b2
+// and x are scaled alike by the caller.
+__device__ __forceinline__ int tri_count(const double *a, double f, const double *b2, int m, double x)
 {
-    double p0 = 1.0, p1 = a[0] - x;
+    double p0 = 1.0, p1 = fma(a[0], f, -x);
     bool neg = p1 <= 0.0;
     int cnt = neg ? 1 : 0;
     for (int i = 1; i < m; ++i) {
         const double t = b2[i] * p0;
-        const double p2 = fma(a[i] - x, p1, -t);
+        const double p2 = fma(fma(a[i], f, -x), p1, -t);
         p0 = p1;
         p1 = p2;
         const bool s = p1 == 0.0 ? !neg : p1 < 0.0;
@@ -40,18 +42,19 @@ __device__ __forceinline__ int tri_count(const double *a, const double *b2, int 
         neg = s;
         if ((i & 3) == 0) {  // divide both by the power of two of the larger
             const int e = (int)((max((unsigned)__double2hiint(fabs(p0)), (unsigned)__double2hiint(fabs(p1))) >> 20) & 0x7ffu);
-            const double f = __hiloint2double(max(1, min(2045, 2046 - e)) << 20, 0);
-            p0 *= f;
-            p1 *= f;
+            const double r = __hiloint2double(max(1, min(2045, 2046 - e)) << 20, 0);
+            p0 *= r;
+            p1 *= r;
         }
     }
     return cnt;
 }
 
 // Bracket of eigenvalue number k (0 = lowest) of the leading m x m matrix, by
-// the whole block; a and b2 may be shared or global.  Ends when it is a few
-// units in the last place wide.
-__device__ __forceinline__ double tri_eigenvalue(const double *a, const double *b2, int m, int k, double lo, double hi)
+// the whole block; a, f and b2 as in tri_count, lo and hi scaled like them.  Ends
+// when it is a few units in the last place wide.
+__device__ __forceinline__ double tri_eigenvalue(const double *a, double f, const double *b2, int m, int k, double lo,
+                                                 double hi)
 {
     __shared__ int first;
     for (int it = 0; it < 24; ++it) {
@@ -62,13 +65,13 @@ __device__ __forceinline__ double tri_eigenvalue(const double *a, const double *
             first = kTriThreads;
         __syncthreads();
         const double x = lo + width * (double)(threadIdx.x + 1) / (double)(kTriThreads + 1);
-        if (tri_count(a, b2, m, x) > k)
+        if (tri_count(a, f, b2, m, x) > k)
             atomicMin(&first, (int)threadIdx.x);
         __syncthreads();
-        const int f = first;
+        const int at = first;
         __syncthreads();
-        const double nlo = f == 0 ? lo : lo + width * (double)f / (double)(kTriThreads + 1);
-        const double nhi = f == kTriThreads ? hi : lo + width * (double)(f + 1) / (double)(kTriThreads + 1);
+        const double nlo = at == 0 ? lo : lo + width * (double)at / (double)(kTriThreads + 1);
+        const double nhi = at == kTriThreads ? hi : lo + width * (double)(at + 1) / (double)(kTriThreads + 1);
         if (!(nhi - nlo < width))
             break;
         lo = nlo;
@@ -136,15 +139,21 @@ __device__ __forceinline__ double tri_solve(const double *a, const double *b, in
 {
     const bool fits = me <= kTriShared;
     double *q = fits ? sm.b2 : b2;
+    double lo, hi;
+    tri_interval(a, b, me, lo, hi);
+    // the power of two that brings the largest entry near one: every step of the
+    // bisection is the same up to it, in every bit
+    const double top = fmax(fabs(lo), fabs(hi));
+    const int e = top > 0.0 && top < 1e300 ? max(-1000, min(1000, ilogb(top))) : 0;
+    const double f = scalbn(1.0, -e);
     for (int i = threadIdx.x; i < me; i += kTriThreads) {
-        q[i] = b[i] * b[i];
+        const double c = b[i] * f;
+        q[i] = c * c;
         if (fits)
             sm.a[i] = a[i];
     }
     __syncthreads();
-    double lo, hi;
-    tri_interval(a, b, me, lo, hi);
-    return tri_eigenvalue(fits ? sm.a : a, q, me, k, lo, hi);
+    return scalbn(tri_eigenvalue(fits ? sm.a : a, f, q, me, k, lo * f, hi * f), e);
 }
 
 // y_out[0..me) = normalised eigenvector for the eigenvalue lam by inverse iteration
