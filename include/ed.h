@@ -488,9 +488,10 @@ ed_status ed_lanczos_multi(const ed_operator *op, const ed_sector *sectors, int 
 
 /*
  * ed_autotune -- choose, by measurement on this GPU, how ed_matvec (and the
- * solvers) run the product for this basis, nvec and dtype: the row-per-lane or
- * the term-parallel kernel (the latter for single vectors of operators whose
- * off-diagonal entries only exchange antiparallel spins), and the pruned or
+ * solvers) run the product for this basis, nvec and dtype: the library's rule
+ * (see ed_matvec), the row-per-lane or the term-parallel kernel (the latter for
+ * single vectors, and real blocks of 8, of operators whose off-diagonal entries
+ * only exchange antiparallel spins), and, for those two, the pruned or
  * the exhaustive rotation search (rings: rotation step one site).  The paper
  * has no counterpart (its kernels are generated once for a CPU).  Every
  * candidate runs a warm-up and three timed products (CUDA events on
@@ -500,7 +501,8 @@ ed_status ed_lanczos_multi(const ed_operator *op, const ed_sector *sectors, int 
  * inversion, log2 of the dimension, nvec, dtype, index kind), and used by
  * every later product on a matching basis.  With the environment variable
  * ED_TUNE_FILE naming a file, the table is read from it on first use and
- * each choice is appended to it.  Synchronises `stream`.
+ * each choice is appended to it; product choices that a library with other
+ * kernels made are passed over.  Synchronises `stream`.
  *
  *   out   host (may be NULL): kernel (0 the library's rule, 1 row-per-lane,
  *         2 term-parallel), search (-1 not applicable, 0 every rotation,

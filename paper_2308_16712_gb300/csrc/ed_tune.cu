@@ -1,12 +1,16 @@
-// ed_tune.cu -- the autotuner of the product: which kernel (row-per-lane or
-// term-parallel), which group search (pruned to the longest runs, or every
+// ed_tune.cu -- the autotuner of the product: which kernel (the library's rule,
+// row-per-lane or term-parallel), which group search (pruned to the longest runs, or every
 // rotation) and which index (hash or bucketed) run fastest for a kind of
 // sector on this GPU.  Choices are measured (CUDA events, best of three after
 // a warm-up) and kept in a table keyed by (GPU name, n_sites, group order,
 // spin inversion, log2 of the dimension, nvec, dtype, index kind); with the
 // environment variable ED_TUNE_FILE set, the table is read from that file on
 // first use and every new choice is appended to it, so later processes reuse
-// it.  ed_matvec and the solvers take the tuned variant when one exists.
+// it.  ed_matvec and the solvers take the tuned variant when one exists.  A product
+// line ends with the number of the candidates it was chosen from (kCandidates);
+// lines without it, or with another, are from before the slot kernel, or after some
+// later change of the kernels, and are not used: a table of that time would keep
+// ring N=36 fp64 at 41 ms where the rule now takes 26.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -59,7 +63,10 @@ int log2_dim(uint64_t dim)
     return l;
 }
 
-// ED_TUNE_FILE lines: "P gpu n order flip log2dim nvec dtype idx kernel prune"
+// Raised when the kernels that product choices are measured among change.
+constexpr int kCandidates = 2;
+
+// ED_TUNE_FILE lines: "P gpu n order flip log2dim nvec dtype idx kernel prune candidates"
 //                     "I gpu n order flip log2dim kind"
 void load_locked()
 {
@@ -72,21 +79,17 @@ void load_locked()
     FILE *f = std::fopen(path, "r");
     if (!f)
         return;
-    char kind = 0;
-    char gpu[256];
-    while (std::fscanf(f, " %c %255s", &kind, gpu) == 2) {
-        if (kind == 'P') {
-            int n, order, flip, l2, nvec, dt, idx, kern, prune;
-            if (std::fscanf(f, "%d %d %d %d %d %d %d %d %d", &n, &order, &flip, &l2, &nvec, &dt, &idx, &kern,
-                            &prune) != 9)
-                break;
-            g_prod[ProdKey{gpu, n, order, flip, l2, nvec, dt, idx}] = MatvecVariant{kern, prune};
-        } else if (kind == 'I') {
-            int n, order, flip, l2, k;
-            if (std::fscanf(f, "%d %d %d %d %d", &n, &order, &flip, &l2, &k) != 5)
-                break;
+    char line[512], gpu[256];
+    while (std::fgets(line, sizeof line, f)) {
+        int n, order, flip, l2, nvec, dt, idx, kern, prune, cand = 0, k;
+        const int got = std::sscanf(line, " P %255s %d %d %d %d %d %d %d %d %d %d", gpu, &n, &order, &flip, &l2,
+                                    &nvec, &dt, &idx, &kern, &prune, &cand);
+        if (got >= 10) {
+            if (cand == kCandidates)
+                g_prod[ProdKey{gpu, n, order, flip, l2, nvec, dt, idx}] = MatvecVariant{kern, prune};
+        } else if (std::sscanf(line, " I %255s %d %d %d %d %d", gpu, &n, &order, &flip, &l2, &k) == 6) {
             g_index[IdxKey{gpu, n, order, flip, l2}] = k;
-        } else {
+        } else if (line[std::strspn(line, " \t\r\n")]) {
             break;
         }
     }
@@ -229,9 +232,9 @@ extern "C" ed_status ed_autotune(const ed_operator *op, const ed_basis *b, const
         const ProdKey k = prod_key(b, nvec, dtype);
         g_prod[k] = best;
         char line[512];
-        std::snprintf(line, sizeof line, "P %s %d %d %d %d %d %d %d %d %d\n", std::get<0>(k).c_str(),
+        std::snprintf(line, sizeof line, "P %s %d %d %d %d %d %d %d %d %d %d\n", std::get<0>(k).c_str(),
                       std::get<1>(k), std::get<2>(k), std::get<3>(k), std::get<4>(k), std::get<5>(k),
-                      std::get<6>(k), std::get<7>(k), best.kernel, best.prune);
+                      std::get<6>(k), std::get<7>(k), best.kernel, best.prune, kCandidates);
         append_line(line);
     }
     if (out) {
