@@ -39,6 +39,7 @@ constexpr int kTpThreads = 256;
 constexpr int kTpWarps = kTpThreads / 32;
 constexpr uint64_t kTpSmallTiles = 608;  // resident at once, four blocks per SM
 constexpr int kTpSmallTerms = 64;        // rounds of a tile, at most (32 rows x 64 terms)
+constexpr size_t kTpMaxShared = 227 * 1024;  // dynamic shared memory of a block, at most
 
 template <int kSec>
 struct TpArgs {
@@ -579,9 +580,11 @@ cudaError_t tp_launch(const TpArgs<kSec> &a, cudaStream_t stream)
     using V = TpVal<T, kC, NV>;
     const size_t smem = tp_smem_bytes<W, T, V, kFact>(a.g, a.op, a.n_sectors, a.max_order);
     if constexpr (kSec == 1 && !kPush && NV == 1 && sizeof(T) == 4) {
-        if (a.total_tiles <= kTpSmallTiles && a.op.max_terms <= kTpSmallTerms) {
+        // where the rounds' sums still have room beside the tables (groups and
+        // operators of many hundreds of entries fill a block's shared memory)
+        const size_t bytes = smem + (size_t)a.op.max_terms * 32 * sizeof(V);
+        if (a.total_tiles <= kTpSmallTiles && a.op.max_terms <= kTpSmallTerms && bytes <= kTpMaxShared) {
             auto small = k_matvec_tp<W, T, kC, kTrack, kFact, kIdx, kSec, kPush, NV, true>;
-            const size_t bytes = smem + (size_t)a.op.max_terms * 32 * sizeof(V);
             int sms = 0, per_sm = 0;
             const cudaError_t e = kernel_occupancy((const void *)small, kTpThreads, bytes, &sms, &per_sm);
             if (e != cudaSuccess)
