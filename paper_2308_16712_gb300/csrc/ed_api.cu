@@ -342,9 +342,6 @@ bool g_force_all_rotations = false;  // test hook: factored search over every ro
 // every lookup is DRAM traffic), else the hash index; 1 = always the hash
 // index; 2 = the bucketed index wherever its entry fits in 64 bits.
 int g_index_policy = 0;
-// Sectors of at least this many states get a slot index.
-constexpr uint64_t kSlotMinDim = 1;
-uint64_t g_slot_min_dim = kSlotMinDim;
 constexpr uint64_t kBucketAutoDim = 1ULL << 23;
 
 // Bucketed index over the basis (see find_bucketed): 2^bbits >= dim / 1.8
@@ -627,8 +624,6 @@ edk::OpView op_view(const ed_operator *op)
 namespace edk {
 
 OpView make_op_view(const ed_operator *op) { return op_view(op); }
-
-uint64_t slot_min_dim() { return g_slot_min_dim; }
 
 int index_policy_get() { return g_index_policy; }
 void index_policy_set(int policy) { g_index_policy = policy; }
@@ -1092,7 +1087,7 @@ ed_status basis_build_impl(int n_sites, int n_up, int spin_inversion, int n_elem
 
     ED_B_TRY(edk::ws_alloc((void **)&d_flag, 4 * sizeof(int), stream));
     ED_B_TRY(cudaMemsetAsync(d_flag, 0, 4 * sizeof(int), stream));
-    if (plan.ghosts && dim >= edk::slot_min_dim() && n_ghost <= plan.ghost_cap) {
+    if (plan.ghosts && dim && n_ghost <= plan.ghost_cap) {
         // the list shrunk to its length, owned by the index
         uint64_t *list = nullptr;
         bool ok = !n_ghost || edk::ws_alloc_optional((void **)&list, n_ghost * sizeof(uint64_t), stream) == cudaSuccess;
@@ -1454,10 +1449,6 @@ void edx_product_counts(unsigned long long *out)
     for (int k = 0; k < edk::kProductKinds; ++k)
         out[k] = edk::g_products[k].load(std::memory_order_relaxed);
 }
-
-// Test hook: later basis builds make a slot index for sectors of at least this
-// many states (0: the library's own threshold).
-void edx_slot_min_dim(uint64_t dim) { g_slot_min_dim = dim ? dim : kSlotMinDim; }
 
 // Diagnostics hook: whether a basis has a slot index, its slots and the
 // weightless representatives among its keys.

@@ -536,7 +536,7 @@ struct ed_basis {
     ulonglong2 *d_stash = nullptr;
     uint32_t n_stash = 0;
     int bbits = 0, brem = 0;
-    edk::SlotView slots{};  // slot index, sectors of at least slot_min_dim() states
+    edk::SlotView slots{};  // slot index (none: no memory to build it, or more than 2^32 slots)
 
     edk::GroupView group_view() const;
     edk::IndexView index_view() const;

@@ -172,8 +172,6 @@ struct MatvecVariant {
 cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, bool track, const void *x,
                             void *y, int nvec, ed_dtype dtype, MatvecVariant v, cudaStream_t stream);
 // ---- slot index (ed_slots.cu) and the product over it (ed_matvec_slot.cuh) --------
-// Sectors of at least this many states get a slot index (test hook: any size).
-uint64_t slot_min_dim();
 bool build_slot_index(ed_basis *b, uint64_t *ghosts, uint32_t n_ghost, int *err, std::vector<uint2> &cells,
                       cudaStream_t stream);
 void free_slot_index(ed_basis *b);

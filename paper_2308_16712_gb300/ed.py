@@ -89,7 +89,6 @@ _SIGS = {
     "edx_lanczos_graph": (_i32, [_i32]),
     "edx_peak": (_d, [_i32, _P, _u64, ctypes.POINTER(_d), _P]),
     "edx_basis_bucket": (_i32, [_P, ctypes.POINTER(_i32), ctypes.POINTER(ctypes.c_uint32)]),
-    "edx_slot_min_dim": (None, [_u64]),
     "edx_optional_memory": (None, [_u64]),
     "edx_slot_scratch_fits": (_i32, [_u64, _u64, _u64]),
     "edx_product_counts": (None, [ctypes.POINTER(ctypes.c_ulonglong)]),
@@ -337,12 +336,6 @@ def optional_memory(limit: int | None) -> None:
     (the enumeration's filter and flags, the slot index, slotted copies) are
     refused above ``limit`` bytes, as if the device had none; None: no limit."""
     _lib.edx_optional_memory(2 ** 64 - 1 if limit is None else limit)
-
-
-def slot_min_dim(dim: int) -> None:
-    """Test hook: later basis builds make a slot index for sectors of at least
-    ``dim`` states (0: the library's own threshold)."""
-    _lib.edx_slot_min_dim(dim)
 
 
 def basis_slots(basis: Basis):
