@@ -169,6 +169,27 @@ struct MatvecVariant {
     size_t scratch_bytes = 0;
     bool alloc = true;         // the product may take that memory from the pool
 };
+// The search of the row-per-lane and term-parallel kernels, from the group's own
+// (GroupView::prune).  The pruned searches take fewer instructions in longer
+// chains, which loses where a product is latency.  Rows: every element up to 17
+// of them on a ring (16 sites without reflection, 415 states, 8 vectors fp64 34.1
+// against 36.0 us; 18 sites at momentum 1, 2700 states, complex128 36.4 against
+// 36.2), and on a torus below kRowsTableDim states (4x4, 441 states, 8 vectors
+// fp64 128 against 167 us; 4x10, 96045 states, fp64 297 against 416; 4x9, 231880
+// states, 589 against 530; in a batch each sector by its own dimension).  Terms: every
+// element for blocks of 8 on a ring of up to 24 elements (16 sites, 21.7 against
+// 23.2 us), and on tori whose table keys are one row or rows of two sites, which
+// leave many candidates (8x8, 4 up, fp64 184 against 311 us; 2x8 102 against 110).
+constexpr uint64_t kRowsTableDim = 1ULL << 17;
+inline int rows_prune(const GroupView &g, uint64_t dim)
+{
+    return (g.prune == 1 && g.n_perm < 18) || (g.prune == 2 && dim < kRowsTableDim) ? 0 : g.prune;
+}
+inline int terms_prune(const GroupView &g, bool block8)
+{
+    return (g.prune == 1 && block8 && g.n_perm <= 24) || (g.prune == 2 && (g.blk_rows == 1 || g.rot_d == 2))
+               ? 0 : g.prune;
+}
 cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, bool track, const void *x,
                             void *y, int nvec, ed_dtype dtype, MatvecVariant v, cudaStream_t stream);
 // ---- slot index (ed_slots.cu) and the product over it (ed_matvec_slot.cuh) --------

@@ -231,6 +231,8 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
                              : use_term_parallel(nvec, op, dtype, g.n_sites);
     const bool tp = tp_ok && (v.kernel == 2 || ((v.kernel == 0 || v.kernel == 4) && rule));
     count_product(tp ? kProductTerms : kProductRows);
+    if (v.prune < 0)
+        g.prune = tp ? terms_prune(g, block8) : rows_prune(g, ix.dim);
     if (tp) {
         const TpArgs<1> t = single_tp_args(op, g, ix, x, y);
         const int k = tp_index_kind(t.sec[0]);

@@ -244,6 +244,7 @@ cudaError_t multi_launch_any(const MultiArgs &a, bool track, ed_dtype dtype, cud
         static thread_local TpArgs<kMaxSectors> t;  // host staging (17 KB); copied at launch
         t.op = a.op;
         t.g = a.g;
+        t.g.prune = terms_prune(a.g, false);
         t.n_sectors = a.n_sectors;
         t.max_order = a.max_order;
         t.total_tiles = a.total_tiles;
@@ -258,11 +259,15 @@ cudaError_t multi_launch_any(const MultiArgs &a, bool track, ed_dtype dtype, cud
         }
         return cudaErrorInvalidValue;
     }
+    static thread_local MultiArgs r;  // host staging (17 KB); copied at launch
+    r = a;
+    if (a.g.prune == 1)  // on a torus the lanes go by their sector's dimension
+        r.g.prune = rows_prune(a.g, 0);
     switch (dtype) {
-    case ED_F64: return multi_f64(a, track, s);
-    case ED_F32: return multi_f32(a, track, s);
-    case ED_C128: return multi_c128(a, track, s);
-    case ED_C64: return multi_c64(a, track, s);
+    case ED_F64: return multi_f64(r, track, s);
+    case ED_F32: return multi_f32(r, track, s);
+    case ED_C128: return multi_c128(r, track, s);
+    case ED_C64: return multi_c64(r, track, s);
     }
     return cudaErrorInvalidValue;
 }

@@ -151,13 +151,13 @@ __host__ __device__ inline size_t multi_smem_bytes(const GroupView &g, const OpV
 // is uniform across the warp)
 template <typename W, bool kTrack, bool kFact>
 __device__ __forceinline__ void search_lane(W s, const uint8_t *kinds, const W *masks, const GroupView &g,
-                                            int lane_flip, W full, W &best, int &gbest)
+                                            int lane_flip, uint64_t lane_dim, W full, W &best, int &gbest)
 {
     if (kFact && g.prune == 1) {
         rep_search_rot1<W, kTrack>(s, kinds, masks, g, lane_flip, full, best, gbest);
         return;
     }
-    if (kFact && g.prune == 2) {
+    if (kFact && g.prune == 2 && lane_dim >= kRowsTableDim) {
         rep_search_blocks<W, kTrack>(s, masks, g, lane_flip, full, best, gbest);
         return;
     }
@@ -420,7 +420,8 @@ __global__ void __launch_bounds__(kMvThreads) k_matvec_multi(const __grid_consta
         W best;
         int gbest = 0;
         const int lane_flip = has ? sm_sec[sec].flip : 0;
-        search_lane<W, kTrack, kFact>(has ? cur : W(0), sm_kind, sm_masks, a.g, lane_flip, full, best, gbest);
+        search_lane<W, kTrack, kFact>(has ? cur : W(0), sm_kind, sm_masks, a.g, lane_flip, has ? sm_sec[sec].dim : 0,
+                                       full, best, gbest);
 
         if (has) {
             const SectorDesc &sd = sm_sec[sec];
