@@ -219,9 +219,13 @@ __device__ __forceinline__ W rep_min_fact(W s, const uint8_t *kinds, const W *ma
     return flip ? min(mn, (W)(mx ^ full)) : mn;
 }
 
-template <typename W, typename T, bool kC, bool kTrack, bool kFact, int NV>
+// kSearch: -1 every element of an unfactored group, 0 of a factored one, 1 ring runs,
+// 2 torus row keys.  One search per kernel: with all of them behind a branch the
+// small sectors' products, a few rounds long, took 5 to 9 % more.
+template <typename W, typename T, bool kC, bool kTrack, int kSearch, int NV>
 __global__ void __launch_bounds__(kMvThreads) k_matvec(const MatvecArgs a)
 {
+    constexpr bool kFact = kSearch >= 0;
     using V = typename ValT<T, kC>::type;
     extern __shared__ __align__(16) unsigned char smem[];
     size_t off[8];
@@ -426,11 +430,11 @@ __global__ void __launch_bounds__(kMvThreads) k_matvec(const MatvecArgs a)
         W best;
         int gbest = 0;
         const W s = has ? cur : W(0);
-        if (kFact && a.g.prune == 1) {
+        if constexpr (kSearch == 1) {
             rep_search_rot1<W, kTrack>(s, sm_kind, sm_masks, a.g, a.g.flip, full, best, gbest);
-        } else if (kFact && a.g.prune == 2) {
+        } else if constexpr (kSearch == 2) {
             rep_search_blocks<W, kTrack>(s, sm_masks, a.g, a.g.flip, full, best, gbest);
-        } else if (kFact) {
+        } else if constexpr (kSearch == 0) {
             if (kTrack)
                 rep_search_fact<W, true>(s, sm_kind, sm_masks, a.g.n_cos, a.g.rot_L, a.g.rot_d, n,
                                          a.g.n_perm, a.g.flip, full, best, gbest);
@@ -501,11 +505,11 @@ __global__ void __launch_bounds__(kMvThreads) k_matvec(const MatvecArgs a)
     }
 }
 
-template <typename W, typename T, bool kC, bool kTrack, bool kFact, int NV>
+template <typename W, typename T, bool kC, bool kTrack, int kSearch, int NV>
 cudaError_t matvec_launch(const MatvecArgs &a, cudaStream_t stream)
 {
-    auto kern = k_matvec<W, T, kC, kTrack, kFact, NV>;
-    const size_t smem = matvec_smem_bytes<W, T, kTrack, kFact>(a.g, a.op);
+    auto kern = k_matvec<W, T, kC, kTrack, kSearch, NV>;
+    const size_t smem = matvec_smem_bytes<W, T, kTrack, (kSearch >= 0)>(a.g, a.op);
     int sms = 0, per_sm = 0;
     const cudaError_t e = kernel_occupancy((const void *)kern, kMvThreads, smem, &sms, &per_sm);
     if (e != cudaSuccess)
@@ -521,7 +525,7 @@ template <typename T, bool kC>
 cudaError_t matvec_dispatch_prec(const MatvecArgs &a, bool track, cudaStream_t stream)
 {
     const bool w32 = a.g.n_sites <= 32;
-    const bool fact = a.g.fact != 0;
+    const int search = a.g.fact ? a.g.prune : -1;
 #define ED_MV_NV(W, TR, FA)                                                       \
     do {                                                                          \
         if (a.nvec == 1) return matvec_launch<W, T, kC, TR, FA, 1>(a, stream);    \
@@ -531,8 +535,10 @@ cudaError_t matvec_dispatch_prec(const MatvecArgs &a, bool track, cudaStream_t s
     } while (0)
 #define ED_MV_FA(W, TR)                  \
     do {                                 \
-        if (fact) ED_MV_NV(W, TR, true); \
-        ED_MV_NV(W, TR, false);          \
+        if (search == 1) ED_MV_NV(W, TR, 1); \
+        if (search == 2) ED_MV_NV(W, TR, 2); \
+        if (search == 0) ED_MV_NV(W, TR, 0); \
+        ED_MV_NV(W, TR, -1);             \
     } while (0)
     if (w32) {
         if (track) ED_MV_FA(uint32_t, true);
