@@ -235,11 +235,11 @@ void ed_operator_destroy(ed_operator *op);
  * hash of the basis and sums each row from a list of its terms.  The copy
  * (some 1.2 dim rows of nvec numbers, padded to a power of two bytes up to 64 and
  * to multiples of 32 beyond) comes from the library's memory pool in stream
- * order.  Where it cannot be had, and while the stream is being captured, the
- * kernel reads x itself instead, which takes longer and gives the same bits.  For
- * other operators, for bases without a slot index, and for nvec > 1 on fewer than
- * 1024 states, two kernels: rows handed to lanes (each lane walks its row's terms), and, for
- * nvec = 1 in single precision (and in double precision above 32 sites) or an fp32 block of nvec = 8, with an operator whose off-diagonal entries
+ * order.  Where it cannot be had, while the stream is being captured, and for the
+ * smallest sectors, where that is faster, the kernel reads x itself instead, which
+ * gives the same bits.  For other operators, for bases without a slot index, and
+ * for nvec > 1 (but 8 in single precision) on fewer than 1024 states, two kernels:
+ * rows handed to lanes (each lane walks its row's terms), and, for nvec = 1 in single precision (and in double precision above 32 sites) or an fp32 block of nvec = 8, with an operator whose off-diagonal entries
  * only exchange antiparallel spins (|01> <-> |10>), a term-parallel
  * kernel (a warp lays a tile's terms out flat, one term per lane per round,
  * and sums each row with a segmented warp scan).  They sum a row's terms in

@@ -72,6 +72,12 @@ cudaError_t launch_matvec(const OpView &op, const GroupView &g, const IndexView 
 namespace {
 
 constexpr uint64_t kSlotBlockMinDim = 1024;
+// Up to this many states a product of one vector goes without the slotted copy: one
+// launch instead of two that wait for each other, and everything is in L2 (8-site
+// ring, 7 states, fp32 13.2 -> 8.7 us, 10.3 by the term-parallel kernel; 20 sites,
+// momentum 1, 9225 states, complex128 41.3 -> 38.2; 4x6 torus, 56664 states, fp64 73
+// with the copy, 89 without).
+constexpr uint64_t kSlotDirectDim = 16384;
 
 int slot_search(const GroupView &g) { return g.fact ? g.prune : 0; }
 
@@ -98,8 +104,10 @@ bool slot_applies(const OpView &op, const GroupView &g, const IndexView &ix, boo
     if (g_kernel_policy != 0 && g_kernel_policy != 3)
         return false;
     // blocks of vectors over the smallest sectors stay with the row-per-lane
-    // kernel, whose columns are those of its single products bit for bit
-    if (nvec > 1 && ix.dim < kSlotBlockMinDim && g_kernel_policy != 3)
+    // kernel, whose columns are those of its single products bit for bit; it does
+    // not serve blocks of 8 in fp32 (16 sites, 415 states: 21.2 us term-parallel, 9.7
+    // here)
+    if (nvec > 1 && ix.dim < kSlotBlockMinDim && !(nvec == 8 && dtype == ED_F32) && g_kernel_policy != 3)
         return false;
     // the coefficient table: in shared memory, its entries counted in 16 bits
     const int order = track ? g.order : 1;
@@ -212,9 +220,10 @@ cudaError_t launch_matvec_v(const OpView &op, GroupView g, const IndexView &ix, 
     // copy where that cannot be had; else the kernels below
     if (v.kernel == 0 && slot_applies(op, g, ix, track, nvec, dtype)) {
         const size_t bytes = slot_scratch_bytes(ix.slots, nvec, dtype);
-        void *xs = v.scratch_bytes >= bytes ? v.scratch : nullptr;
+        const bool direct = g_kernel_policy == 0 && ix.dim <= (nvec == 1 ? kSlotDirectDim : kSlotBlockMinDim - 1);
+        void *xs = !direct && v.scratch_bytes >= bytes ? v.scratch : nullptr;
         void *own = nullptr;
-        if (!xs && v.alloc && !stream_captured(stream) && ws_alloc_optional(&own, bytes, stream) == cudaSuccess)
+        if (!xs && !direct && v.alloc && !stream_captured(stream) && ws_alloc_optional(&own, bytes, stream) == cudaSuccess)
             xs = own;
         const cudaError_t e = launch_slot(op, g, ix, track, x, y, xs, nvec, dtype, stream);
         const cudaError_t e2 = ws_free(own, stream);

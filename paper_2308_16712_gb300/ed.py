@@ -439,8 +439,10 @@ KERNEL_POLICIES = {"auto": 0, "rowwise": 1, "term_parallel": 2, "slots": 3}
 
 def kernel_policy(policy: str) -> None:
     """Testing aid: which matvec kernel serves an exchange-only operator: "auto"
-    (the slot kernel where the basis has a slot index, except for blocks of
-    vectors over fewer than 1024 states), "slots" (there, too), "rowwise", or
+    (the slot kernel where the basis has a slot index, without the slotted copy
+    for the smallest sectors, but not for blocks of vectors over fewer than 1024
+    states other than 8 in fp32), "slots" (there, too, and with the copy),
+    "rowwise", or
     "term_parallel" (one vector or a real block of 8).  Affects later launches."""
     _lib.edx_kernel_policy(KERNEL_POLICIES[policy])
 

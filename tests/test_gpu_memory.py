@@ -208,3 +208,19 @@ def test_product_counts_name_the_kernel_that_ran():
         ed.kernel_policy(policy)
         assert served(ed, product) == {name: 1}
         assert served(ed, block) == {name: 12}
+
+
+def test_small_sectors_take_one_launch():
+    torch, ed = gpu()
+    h = ei.heisenberg_ring(20)
+    O = ed.operator_create(20, h["sites"], h["coeff"], h["local"])
+    for (z, grp), one in (((+1, ei.ring_group(20, 0, +1)), True), ((0, ei.ring_group(20, 0)), True),
+                          ((+1, (np.arange(20, dtype=np.int32).reshape(1, 20), np.array([[1.0, 0.0]]))), False)):
+        B = ed.basis_build(20, 10, z, *grp)  # 2518, 9252, 92378 states
+        x = to_torch(ei.x_by_index(3, ed.basis_size(B), 1)[:, 0], np.float64)
+        y, want = torch.empty_like(x), torch.empty_like(x)
+        assert served(ed, lambda: ed.matvec(O, B, x, y)) == {"slot without copy" if one else "slot": 1}
+        ed.kernel_policy("slots")
+        assert served(ed, lambda: ed.matvec(O, B, x, want)) == {"slot": 1}
+        ed.kernel_policy("auto")
+        assert torch.equal(y, want)

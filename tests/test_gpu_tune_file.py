@@ -43,6 +43,6 @@ def test_saved_choices(tmp_path):
     path.write_text("\n".join([" ".join(current), ""]))
     assert run(path) == "row-per-lane"
     path.write_text("\n".join([" ".join(older), ""]))
-    assert run(path) == "slot"
+    assert run(path) == "slot without copy"  # a small sector
     path.write_text("\n".join([" ".join(older), " ".join(current), ""]))
     assert run(path) == "row-per-lane"
