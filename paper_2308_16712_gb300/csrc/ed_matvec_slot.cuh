@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
     static_assert(!kC || EL % 2 == 0, "a complex number per lane at least");
     static_assert(!kDirect || kSearch == 0, "the search is chosen at run time");
     constexpr bool kBatch = kSec > 1;
+    constexpr bool kWhole = kC || (sizeof(T) == 8 && EL > 1);  // two sums of a row's terms with coefficients
     extern __shared__ __align__(16) unsigned char smem[];
     const bool fact = kSearch > 0 || a.g.fact;
     size_t off[7];
@@ -536,9 +537,12 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                         }
                     }
                     // short chains of additions: four terms as a tree; with
-                    // coefficients two sums for alternate terms, of complex vectors
-                    // for the whole row (a tree would add 12 % to the arithmetic), of
-                    // real ones for the four
+                    // coefficients two sums for alternate terms, for the whole row, or
+                    // (real, but for several fp64 vectors) for the four.  Two per four
+                    // terms add 12 % to a complex sum and half to a real one, which the
+                    // fp64 pipe feels (5x6 torus, 8 vectors fp64, 3.72 -> 4.95 ms); one
+                    // fp64 vector does not (2.76 ms either way), and on the 6x6 torus
+                    // took 199 ms with them and 362 with the longer-lived two
                     if (plain) {
 #pragma unroll
                         for (int e = 0; e < EL; ++e)
@@ -550,7 +554,7 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                             four[0][e] = four[1][e] = T(0);
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            T (&sum)[EL] = kC ? acc[u & 1] : four[u & 1];
+                            T (&sum)[EL] = kWhole ? acc[u & 1] : four[u & 1];
                             Cplx<T> c;
                             if (kBatch && kTrack) {
                                 const uint32_t m = uniform ? 0u : ci[u] / (uint32_t)a.order;
@@ -576,14 +580,14 @@ __global__ void __launch_bounds__(kSlThreads, kDirect ? 4 : kSlBlocks<W, T, kTra
                                     sum[e] = fma(c.re, v[u].e[e], sum[e]);
                             }
                         }
-                        if constexpr (!kC) {
+                        if constexpr (!kWhole) {
 #pragma unroll
                             for (int e = 0; e < EL; ++e)
                                 acc[0][e] += four[0][e] + four[1][e];
                         }
                     }
                 }
-                if (kC && !plain) {
+                if (kWhole && !plain) {
 #pragma unroll
                     for (int e = 0; e < EL; ++e)
                         acc[0][e] += acc[1][e];
