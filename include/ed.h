@@ -138,9 +138,8 @@ ed_status ed_basis_build(int n_sites, int n_up, int spin_inversion, int n_elems,
  * enumeration and its scan, without keeping the basis (Table 2 of the paper
  * lists such dimensions, up to 48 spins, which no single GPU could store).
  * Arguments as ed_basis_build; the dimension may exceed 2^32.  The per-chunk
- * counts and the scan's arrays come from the library's memory pool and go
- * back to it; the group and binomial tables are allocated with cudaMalloc and
- * freed (which synchronises the device).  Synchronises `stream`.
+ * counts, the scan's arrays and the tables come from the library's memory pool
+ * and go back to it.  Synchronises the device.
  */
 ed_status ed_basis_count(int n_sites, int n_up, int spin_inversion, int n_elems,
                          const int32_t *perms, const double *chars, void *stream, uint64_t *dim);
@@ -357,7 +356,8 @@ typedef struct {
  * a second pass in the same way), whose lowest Ritz value is returned
  * together with its residual.  Work memory beyond the caller's vectors: four
  * fp64 vectors, plus two fp32 vectors in the fp32-matvec mode, when the
- * Krylov vectors are not stored.  Sectors of at most 2^22 states are
+ * Krylov vectors are not stored; and the slotted copy of one vector (ed_matvec)
+ * where it fits beside them with half a gigabyte to spare.  Sectors of at most 2^22 states are
  * launch-bound: there the steps after the first are replayed from a CUDA
  * graph of two steps (same kernels, same results).  Not to be called while
  * `stream` is being captured.  Takes its work vectors from the library's
@@ -435,7 +435,8 @@ ed_status ed_lanczos_eigs(const ed_operator *op, const ed_basis *basis, const vo
  * fp32-matvec mode does (a short fp64 single-vector Lanczos run from the
  * Ritz vector; fp64 Rayleigh quotient and residual).  Memory: three blocks
  * of fp64 (two in the fp32 mode, plus two fp32 blocks) from the library's
- * pool.  Synchronises `stream` before returning.
+ * pool, and the slotted copy of one block (ed_matvec) where it fits beside them
+ * with half a gigabyte to spare.  Synchronises `stream` before returning.
  * Errors: ED_ERR_INVALID_ARG (also nvec not in {2, 4, 8, 16}, a sector
  * smaller than nvec or a start block of lower rank), ED_ERR_SYMMETRY_MISMATCH,
  * ED_ERR_UNSUPPORTED (complex sectors or operators), ED_ERR_OOM, ED_ERR_CUDA.

@@ -249,11 +249,12 @@ int tuned_index_kind(int n_sites, int order, int flip, uint64_t dim);
 cudaError_t launch_matvec_push(const OpView &op, const GroupView &g, const IndexView &ix, bool track,
                                const void *x, void *y, ed_dtype dtype, cudaStream_t stream);
 
-// Kernel choice for one vector and an exchange-only operator: 0 = the
-// term-parallel kernel in single precision, the row-per-lane kernel in double
-// precision (where the term-parallel kernel's fp64 segmented sums cost more
-// than they save); 1 = always row-per-lane; 2 = always term-parallel.
+// Kernel choice for exchange-only operators (test hook): 0 = the slot kernel where
+// slot_applies, without the copy for the smallest sectors, else use_term_parallel's
+// rule; 1 = always row-per-lane; 2 = term-parallel (one vector, real blocks of 8);
+// 3 = the slot kernel for every block of vectors, with the copy where it can be had.
 extern int g_kernel_policy;
+// The rule without the slot kernel, for one vector.
 bool use_term_parallel(int nvec, const OpView &op, ed_dtype dtype, int n_sites);
 
 }  // namespace edk

@@ -740,9 +740,11 @@ ed_status run_lanczos(const ed_operator *op, const ed_basis *b, const void *x0, 
         // The fp32 recurrence loses orthogonality after some 50 steps (fp64: 80),
         // and from then on the Ritz vector's sign follows the rounding of every
         // product: below kSlotMixedMinDim states the products of that mode keep
-        // the order of sums they always had, at 8 % more time (ring N=32).
-        // So do those of reorthogonalised runs, whose time the vectors dominate
-        // and whose end (a vanishing beta) is a matter of rounding, too.
+        // the order of sums they always had, at a third more time (ring N=32: 1.21
+        // against 0.90 ms).  So do those of reorthogonalised runs, whose time the
+        // vectors dominate and whose end (a vanishing beta) is a matter of
+        // rounding, too.  Above, where the older kernels lose most, and in batches
+        // of sectors the sign is left to the rounding.
         if (v.kernel == 0 && (reorth || (dt == dt32 && n < kSlotMixedMinDim)))
             v.kernel = 4;
         v.scratch = slot_ws;

@@ -22,7 +22,8 @@
 //      for several vectors, its columns), each lane gathers with 4 reads in
 //      flight and accumulates in registers; a shuffle tree joins the group.
 // Summing in phase C takes one addition per term and vector spread over all
-// lanes.  The segmented warp scan of the term-parallel kernel it replaces took
+// lanes, in chains short enough that no sum is less accurate than by the scan
+// (ring N=32 fp32 5.0e-8 of the 64-bit value either way; 5.7e-8 in one chain a lane).  The segmented warp scan of the term-parallel kernel it replaces took
 // 5 shuffles and 5 additions per round of 32 terms and vector (and 4 fp64
 // multiplications for the coefficients), which on the 1/74-rate fp64 pipe was
 // half of an fp64 product and, for 8 vectors, 80 shuffles per round.  Matrix
@@ -32,11 +33,11 @@
 //
 // Beyond L2 the reads of xs are bound by DRAM's rate of random accesses (5.1e10 /s
 // over 0.5 GB, 4.1e10 /s over 2 GB, whatever the load's form): ring N=36 fp64
-// 25.6 ms of 23, ring N=38 8 vectors fp32 123 of 116.  Within L2 issue slots and the
+// 25.9 ms of 23, ring N=38 8 vectors fp32 126 of 116.  Within L2 issue slots and the
 // L2's 2.9e11 random reads /s overlap in part (ring N=32 fp32: 71 % of the issue
 // slots, 0.90 ms against 0.53 for the reads alone).  Against the kernels it
 // replaced: those three 41.0, 181 and 1.18 ms; ring N=33 3 vectors complex128
-// 99.8 -> 20.5, 6x6 torus complex128 838 -> 180.
+// 99.8 -> 21.1, 6x6 torus complex128 838 -> 184.
 //
 // The order of every sum depends only on the operator, the type and the number of
 // vectors, not on R: results are deterministic, and the same for a sector alone

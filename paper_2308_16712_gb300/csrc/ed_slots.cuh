@@ -32,8 +32,8 @@ constexpr int kSlotLogB = 11;                 // buckets per partition
 constexpr uint32_t kSlotPartKeys = 7168;      // keys per partition (average, at most)
 constexpr uint32_t kSlotSmallKeys = 2560;     // the same for up to kSlotSmallMax keys: at load 0.3 the
 constexpr uint64_t kSlotSmallMax = 1u << 18;  // longest pilot search of a partition takes 0.05 ms, not 0.3
-constexpr uint32_t kSlotCap = 8533;           // slots per partition: load 0.84, and room for
-                                              // the fullest of 1e6 partitions (+ 5.5 sigma)
+constexpr uint32_t kSlotCap = 8533;           // slots per partition: load 0.84, and room for any
+                                              // partition (16 sigma above the average)
 constexpr uint32_t kPilotEscape = 255;        // pilot kept in the exception table instead
 
 struct SlotView {
