@@ -212,7 +212,7 @@ inline size_t slot_scratch_bytes(const SlotView &v, int nvec, ed_dtype dtype)
 // free device memory (what the pool holds cached included) less what the call
 // still allocates, with room left for what the driver loads at a first launch.
 // Ring N=40, 8 vectors in single precision: 32.9 of some 56 GB; a block step takes
-// 0.60 s with it, 0.91 s by the term-parallel kernel.
+// 0.61 s with it, 0.91 s by the term-parallel kernel.
 constexpr size_t kSlotReserve = 512ull << 20;
 inline bool slot_scratch_fits(size_t want, size_t free_bytes, size_t later)
 {
